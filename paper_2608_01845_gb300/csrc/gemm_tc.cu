@@ -10,10 +10,11 @@
 //               of two TMEM accumulators (2 x 256 columns), commits the smem
 //               stage back to the producer and the accumulator to the
 //               epilogue;
-//   warps 2-5   epilogue: tcgen05.ld 32 columns at a time (each warp owns its
-//               32-lane TMEM quarter = 32 rows), bias / GELU / gated residual /
-//               QKV scatter / unpatchify, 16-byte global stores; then release
-//               the accumulator so the next tile's MMAs overlap this epilogue.
+//   warps 2-5   epilogue (epilogue_tile): each warp owns its 32-lane TMEM
+//               quarter = 32 rows and works through the tile 64 columns at a
+//               time: tcgen05.ld, bias / GELU / gated residual, bf16 into a
+//               swizzled shared-memory slab, one TMA store per slab; then
+//               release the accumulator so the next tile's MMAs overlap.
 // Tiles are visited N-fastest inside groups of N tiles sized so a group's
 // slab of W stays in L2 (about 40 MB), so W is read from DRAM about once and
 // A once per group.
@@ -30,14 +31,33 @@ namespace wdc {
 
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 4;
+constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int kGemmThreads = 192;
 constexpr uint32_t A_BYTES = BM * BK * 2;
-constexpr uint32_t B_BYTES = BN * BK * 2;
-constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-constexpr uint32_t TMEM_COLS = 2 * BN;
-constexpr uint32_t IDESC = idesc_bf16(BM, BN);
-constexpr size_t SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+// Epilogue staging: two slabs of 32 rows x 64 bf16 columns (128-byte rows,
+// 128-byte swizzle) per epilogue warp.
+constexpr uint32_t SLAB_BYTES = 32 * 128;
+constexpr uint32_t STAGING_BYTES = 4 * 2 * SLAB_BYTES;
+
+// One-CTA kernel, tiles of 128 x BNT: as deep a ring as the tile leaves room for.
+template <int BNT>
+struct GemmCfg {
+    static constexpr uint32_t B_BYTES = BNT * BK * 2;
+    static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
+    static constexpr int STAGES = BNT == 256 ? 4 : (BNT == 128 ? 6 : 8);
+    static constexpr uint32_t TMEM_COLS = 2 * BNT;
+    static constexpr uint32_t IDESC = idesc_bf16(BM, BNT);
+    static constexpr size_t SMEM = STAGES * STAGE_BYTES + STAGING_BYTES + 1024 + 256;
+    static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
+};
+
+// Tensor maps of one problem's epilogue: `out` (kEpiStore, kEpiResid) and
+// `res` (kEpiResid) in boxes of 32 rows x 64 columns; for kEpiQKV `out` = Q,
+// `res` = K ([heads, L, d], boxes of 32 tokens x 64) and `vt` = V^T
+// ([heads, d, L], boxes of 64 x 32 tokens).
+struct EpiMaps {
+    CUtensorMap out, res, vt;
+};
 
 struct GemmArgs {
     int M, N, K;
@@ -50,6 +70,9 @@ struct GemmArgs {
     int nprob;              // 1 or 2
     int M1, m_pairs1;
     Epi e1;
+    // whether each problem's epilogue has its tensor maps (else every row goes
+    // through the direct stores of epilogue_chunk)
+    int staged, staged1;
 };
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
@@ -61,7 +84,13 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t u) {
     return __bfloat1622float2(h);
 }
 
-// Epilogue of 32 consecutive columns col0..col0+31 of one row.
+// Epilogue forms; each is its own instantiation of the kernels, so that the
+// epilogue's code stays small and without branches on the form.
+enum Form { kFormStore = 0, kFormGelu = 1, kFormResid = 2, kFormQKV = 3, kFormUnpatch = 4, kForms = 5 };
+
+// Direct epilogue of 32 consecutive columns col0..col0+31 of one row: the
+// unpatchify form, and the rows whose slab cannot be moved by one TMA copy.
+template <int FORM>
 __device__ __forceinline__ void epilogue_chunk(const Epi& e, int m, int col0, const uint32_t (&r)[32]) {
     float v[32];
     if (e.bias) {
@@ -78,14 +107,10 @@ __device__ __forceinline__ void epilogue_chunk(const Epi& e, int m, int col0, co
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
     }
-    if (e.gelu) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = gelu_tanh_f(v[j]);
-    }
-    if (e.mode == kEpiStore || e.mode == kEpiResid) {
+    if constexpr (FORM == kFormResid) {
         __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(e.out) + (size_t)m * e.ldo + col0;
         uint4* o4 = reinterpret_cast<uint4*>(out);
-        if (e.mode == kEpiResid) {
+        {
             const int rm = e.res_rows > 0 ? m % e.res_rows : m;
             const uint4* r4 = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(e.res) +
                                                              (size_t)rm * e.ldo + col0);
@@ -123,9 +148,7 @@ __device__ __forceinline__ void epilogue_chunk(const Epi& e, int m, int col0, co
             w.w = pack_bf16(v[8 * q + 6], v[8 * q + 7]);
             o4[q] = w;
         }
-        return;
-    }
-    if (e.mode == kEpiQKV) {
+    } else if constexpr (FORM == kFormQKV) {
         const int which = col0 / e.D, c = col0 % e.D, dd0 = c % e.d;
         int b, tok;
         batch_token(e.row_off + m, e.nb, e.Lc, e.L, b, tok);
@@ -150,27 +173,284 @@ __device__ __forceinline__ void epilogue_chunk(const Epi& e, int m, int col0, co
             for (int j = 0; j < 32; ++j) base[(size_t)j * e.ldv] = to_vt_half(v[j], sat);
             if (sat && e.err) atomicOr(e.err, kErrVSaturated);
         }
-        return;
+    } else {
+        // kEpiUnpatch: fp32 scatter into the latent.  The row's place is worked
+        // out once, the column's (c, ph, pw) counts up: element by element both
+        // were chains of integer divisions (a 272 x 64 tile took 42 us).
+        const int hp = e.Hh / e.p, wp = e.Ww / e.p, Lv = e.F * hp * wp;
+        const int b = m / Lv, mm = m - b * Lv;
+        const int f = mm / (hp * wp), rem = mm - f * (hp * wp), h2 = rem / wp, w2 = rem - h2 * wp;
+        const size_t plane = (size_t)e.F * e.Hh * e.Ww;
+        float* row = e.v + (size_t)b * e.C * plane + ((size_t)f * e.Hh + (size_t)h2 * e.p) * e.Ww + (size_t)w2 * e.p;
+        if (e.p == 2 && !((uintptr_t)e.v & 7)) {       // pw = 0, 1 side by side
+            float* o = row + (size_t)(col0 / 4) * plane;
+#pragma unroll
+            for (int j = 0; j < 32; j += 2)
+                *reinterpret_cast<float2*>(o + (size_t)(j / 4) * plane + (size_t)((j / 2) & 1) * e.Ww) =
+                    make_float2(v[j], v[j + 1]);
+            return;
+        }
+        const int pp = e.p * e.p;
+        int c = col0 / pp, ph = (col0 - c * pp) / e.p, pw = col0 - c * pp - ph * e.p;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            row[(size_t)c * plane + (size_t)ph * e.Ww + pw] = v[j];
+            if (++pw == e.p) {
+                pw = 0;
+                if (++ph == e.p) { ph = 0; ++c; }
+            }
+        }
     }
-    // kEpiUnpatch: fp32 scatter into the latent
-    Epi e2 = e;
-    e2.bias = nullptr;
-    e2.gelu = 0;
-#pragma unroll 4
-    for (int j = 0; j < 32; ++j) epi_apply<__nv_bfloat16>(e2, m, col0 + j, v[j]);
 }
 
+// ---------------------------------------------------------------------------
+// Staged epilogue of one warp's 32 rows of a tile, 64 columns at a time.
+//
+// Written straight from the accumulator with one row per lane, a 16-byte store
+// or residual load touches 32 different 128-byte lines, which the load/store
+// unit works through one by one, and every chunk waits for its bias and gate
+// from L2: 11-16k cycles (clock stamps) a 128 x 256 tile for a plain store,
+// 20k with GELU, 20-35k with a gated residual, where the tile's MMAs take 9k
+// (K = 1024) to 26k (K = 3072).  Now 3.7k, 8.1k and 8.0k, behind the MMAs from
+// K = 1024 on:
+//  * the accumulator is read in the 16x256b shape: lane t holds columns
+//    2 (t % 4), + 1 of every 8 in rows t / 4 + 8 i, so a lane needs 16 bias
+//    and gate values per chunk instead of 64, and they are fetched a chunk (for
+//    the first chunk a tile) ahead of their use;
+//  * packed to 16 bits those are the 8 x 8 fragments of stmatrix / ldmatrix,
+//    which move them to and from a slab of shared memory (32 rows x 64 columns,
+//    swizzled like the tensor map's box: no bank conflicts; transposed on the
+//    way for V^T);
+//  * one TMA store moves the slab; a residual slab comes in by a TMA load,
+//    the tile's first two while the tile's MMAs run, and is updated in place;
+//  * each form is a kernel of its own: with the forms as branches of one kernel
+//    the same epilogue took 14-25k cycles.
+// 17776 x 3072 x 3072 with the gated residual: 241 -> 193 us; 6400 x 4096 x
+// 1024 with GELU: 83 -> 46 us; 272 x 256 x 256 with the residual: 17 -> 13 us.
+// Rows past M and columns past N are clipped by the tensor map.  Slabs
+// alternate; one is written again once its store has read it
+// (cp.async.bulk.wait_group.read).
+struct WarpStage {
+    uint8_t* slab;        // [2][SLAB_BYTES]
+    uint64_t* rbar;       // [2] residual slab landed
+    uint32_t cnt;         // slabs used so far: the next one is cnt & 1, its residual's parity (cnt >> 1) & 1
+    uint32_t pending;     // residual slabs requested and not yet awaited (cnt, cnt + 1, ...)
+    float2 bias[8], gate[8];   // the next chunk's, columns 8 i + 2 (lane % 4), + 1
+};
+
+// Requests the residual of columns col0.. of rows m0.. into slab `cnt`.
+__device__ __forceinline__ void request_residual(WarpStage& ws, uint32_t cnt, const CUtensorMap* res, int m0, int col0,
+                                                 int lane) {
+    if (lane == 0) {
+        bulk_wait_read<0>();               // the slab's last store has read it
+        mbar_arrive_expect_tx(&ws.rbar[cnt & 1], SLAB_BYTES);
+        tma_load_2d(ws.slab + (cnt & 1) * SLAB_BYTES, res, &ws.rbar[cnt & 1], col0, m0);
+    }
+    ++ws.pending;
+}
+
+// Fetches the bias and gate of the chunk at col0.  Columns past `end` (whose
+// results are clipped) read the last valid ones: a clamped address, since a
+// select on the loaded value would wait for it here.
+template <int FORM>
+__device__ __forceinline__ void fetch_columns(const float* bias, const float* gate, int col0, int end, WarpStage& ws,
+                                              int lane) {
+    const int c = col0 + 2 * (lane & 3);
+    if (bias) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ws.bias[i] = __ldg(reinterpret_cast<const float2*>(bias + min(c + 8 * i, end - 2)));
+    }
+    if (FORM == kFormResid && gate) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ws.gate[i] = __ldg(reinterpret_cast<const float2*>(gate + min(c + 8 * i, end - 2)));
+    }
+}
+
+// Before the tile's accumulator is awaited: its first chunk's columns and its
+// first two residual slabs.
+template <int FORM>
+__device__ __forceinline__ void epilogue_prefetch(const float* bias, const float* gate, int staged,
+                                                  const CUtensorMap* res, int M, int n0, int end, int m0, WarpStage& ws,
+                                                  int lane) {
+    if (FORM == kFormUnpatch || !staged || m0 >= M) return;
+    fetch_columns<FORM>(bias, gate, n0, end, ws, lane);
+    if (FORM != kFormResid) return;
+    request_residual(ws, ws.cnt, res, m0, n0, lane);
+    if (n0 + 64 < end) request_residual(ws, ws.cnt + 1, res, m0, n0 + 64, lane);
+}
+
+// After a wait has given up: no residual copy is left in flight at exit.
+__device__ __forceinline__ void epilogue_drain(WarpStage& ws) {
+    for (; ws.pending > 0; --ws.pending, ++ws.cnt) {
+        const unsigned long long t0 = globaltimer();
+        while (!mbar_try_wait(&ws.rbar[ws.cnt & 1], (ws.cnt >> 1) & 1) && globaltimer() - t0 < kWaitLimitNs) {
+        }
+    }
+}
+
+// The tile's columns [n0, end) of rows [m0, m0 + 32), accumulator at taddr;
+// `release` runs once the accumulator has been read.  Returns false when a
+// residual slab did not arrive in time.
+template <int FORM, class Release>
+__device__ __forceinline__ bool epilogue_tile(const Epi& e, int staged, const EpiMaps* maps, int M, int m0, int n0, int end,
+                                              uint32_t taddr, WarpStage& ws, volatile int* abort_flag,
+                                              unsigned* err, int lane, Release release) {
+    if (m0 >= M) {
+        release();
+        return true;
+    }
+    // QKV: the slab's rows are consecutive tokens of one sample, and rows past
+    // M (if any) fall off the end of the tensor
+    int b0 = 0, tok0 = 0;
+    if (FORM == kFormQKV && staged) {
+        const int last = min(m0 + 31, M - 1);
+        int b1, tok1;
+        batch_token(e.row_off + m0, e.nb, e.Lc, e.L, b0, tok0);
+        batch_token(e.row_off + last, e.nb, e.Lc, e.L, b1, tok1);
+        staged = b0 == b1 && tok1 - tok0 == last - m0 && (last == m0 + 31 || tok1 == e.L - 1);
+    }
+    // this lane's row address in an x4 matrix store: row lane % 8 of matrix
+    // lane / 8; matrices 0, 1 are row groups 2 hb, 2 hb + 1 of column group i,
+    // matrices 2, 3 the same of column group i + 1
+    const int mrow = lane & 7, mrg = (lane >> 3) & 1, mcg = lane >> 4;
+    for (int col0 = n0; col0 < end; col0 += 64) {
+        const uint32_t sl = ws.cnt & 1;
+        const uint32_t slab = smem_u32(ws.slab) + sl * SLAB_BYTES;
+        const bool vt = FORM == kFormQKV && col0 >= 2 * e.D;
+        if (FORM != kFormStore && FORM != kFormGelu && (FORM == kFormUnpatch || !staged || (vt && (tok0 & 7)))) {
+            // (a V^T slab must start on a 16-byte boundary of its token row)
+#pragma unroll 1
+            for (int c32 = col0; c32 < min(col0 + 64, end); c32 += 32) {
+                uint32_t r[32];
+                tmem_ld32(taddr + (c32 - n0), r);
+                tmem_ld_wait();
+                if (c32 + 32 >= end) release();
+                if (m0 + lane < M) epilogue_chunk<FORM>(e, m0 + lane, c32, r);
+            }
+            if (FORM == kFormQKV && col0 + 64 < end) fetch_columns<FORM>(e.bias, e.gate, col0 + 64, end, ws, lane);
+            continue;
+        }
+        if constexpr (FORM != kFormUnpatch) {
+            float v[2][8][4];                  // [rows 16 hb ..][column group][row t/4: 2, row t/4 + 8: 2]
+            tmem_ld16x256(taddr + (col0 - n0), *reinterpret_cast<float(*)[32]>(&v[0]));
+            tmem_ld16x256(taddr + (16u << 16) + (col0 - n0), *reinterpret_cast<float(*)[32]>(&v[1]));
+            if constexpr (FORM == kFormResid) {
+                const bool landed = mbar_wait(&ws.rbar[sl], (ws.cnt >> 1) & 1, abort_flag, err);
+                if (!__all_sync(0xffffffffu, landed)) {
+                    release();                     // every other wait of the CTA gives up too
+                    return false;
+                }
+                --ws.pending;
+            } else {
+                if (lane == 0) bulk_wait_read<1>();
+            }
+            __syncwarp();
+            tmem_ld_wait();
+            if (col0 + 64 >= end) release();
+            if (e.bias) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int hb = 0; hb < 2; ++hb) {
+                        v[hb][i][0] += ws.bias[i].x; v[hb][i][1] += ws.bias[i].y;
+                        v[hb][i][2] += ws.bias[i].x; v[hb][i][3] += ws.bias[i].y;
+                    }
+            }
+            if constexpr (FORM == kFormGelu) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+#pragma unroll
+                    for (int hb = 0; hb < 2; ++hb)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) v[hb][i][j] = gelu_tanh_f(v[hb][i][j]);
+            }
+            if (vt) {
+                // rows = d, 32 tokens (64 bytes) each, 64-byte swizzle
+                bool sat[4] = {false, false, false, false};
+#pragma unroll
+                for (int hb = 0; hb < 2; ++hb)
+#pragma unroll
+                    for (int i = 0; i < 8; i += 2) {
+                        uint32_t w[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {          // matrix q: column group i + q / 2, rows of 2 hb + q % 2
+                            const float* x = &v[hb][i + (q >> 1)][2 * (q & 1)];
+                            const __half2 h = __halves2half2(to_vt_half(x[0], sat[2 * hb + (q & 1)]),
+                                                             to_vt_half(x[1], sat[2 * hb + (q & 1)]));
+                            w[q] = *reinterpret_cast<const uint32_t*>(&h);
+                        }
+                        const int dd = 8 * (i + mcg) + mrow;
+                        stmatrix_x4_trans(slab + dd * 64 + (((2 * hb + mrg) ^ ((dd >> 1) & 3)) << 4), w);
+                    }
+                bool any = false;
+#pragma unroll
+                for (int g = 0; g < 4; ++g) any |= sat[g] && m0 + 8 * g + (lane >> 2) < M;
+                if (any && e.err) atomicOr(e.err, kErrVSaturated);
+            } else {
+#pragma unroll
+                for (int hb = 0; hb < 2; ++hb)
+#pragma unroll
+                    for (int i = 0; i < 8; i += 2) {
+                        const uint32_t at = slab + (16 * hb + 8 * mrg + mrow) * 128 + (((i + mcg) ^ mrow) << 4);
+                        if constexpr (FORM == kFormResid) {
+                            uint32_t rr[4];
+                            ldmatrix_x4(at, rr);
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                float* x = &v[hb][i + (q >> 1)][2 * (q & 1)];
+                                const float2 f = unpack_bf16(rr[q]);
+                                const float2 g = e.gate ? ws.gate[i + (q >> 1)] : make_float2(1.f, 1.f);
+                                x[0] = fmaf(g.x, x[0], f.x);
+                                x[1] = fmaf(g.y, x[1], f.y);
+                            }
+                        }
+                        uint32_t w[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float* x = &v[hb][i + (q >> 1)][2 * (q & 1)];
+                            w[q] = pack_bf16(x[0], x[1]);
+                        }
+                        stmatrix_x4(at, w);
+                    }
+            }
+            if (col0 + 64 < end) fetch_columns<FORM>(e.bias, e.gate, col0 + 64, end, ws, lane);
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                const uint8_t* src = ws.slab + sl * SLAB_BYTES;
+                if constexpr (FORM != kFormQKV) {
+                    tma_store_2d(&maps->out, src, col0, m0);
+                } else {
+                    const int c = col0 % e.D, head = b0 * e.H + c / e.d, dd = c % e.d;
+                    if (vt) tma_store_3d(&maps->vt, src, tok0, dd, head);
+                    else tma_store_3d(col0 < e.D ? &maps->out : &maps->res, src, dd, tok0, head);
+                }
+                bulk_commit();
+            }
+            if (FORM == kFormResid && col0 + 128 < end) request_residual(ws, ws.cnt, &maps->res, m0, col0 + 128, lane);
+            ++ws.cnt;
+        }
+    }
+    return true;
+}
+
+template <int BNT, int FORM>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ GemmArgs g) {
+                   const __grid_constant__ EpiMaps maps, const __grid_constant__ GemmArgs g) {
+    using C = GemmCfg<BNT>;
+    constexpr int STAGES = C::STAGES;
+    constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+    uint8_t* staging = smem + STAGES * STAGE_BYTES;
+    uint64_t* full = reinterpret_cast<uint64_t*>(staging + STAGING_BYTES);
     uint64_t* empty = full + STAGES;
     uint64_t* tfull = empty + STAGES;
     uint64_t* tempty = tfull + 2;
     uint64_t* mma_done = tempty + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
+    uint64_t* rbars = mma_done + 1;            // [4 warps][2] residual slabs
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rbars + 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -184,6 +464,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             mbar_init(&tempty[a], 4);
         }
         mbar_init(mma_done, 1);
+        for (int i = 0; i < 8; ++i) mbar_init(&rbars[i], 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -192,7 +473,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         prefetch_tmap(&tmB);
     }
     if (warp == 1) {
-        tmem_alloc(tmem_slot, TMEM_COLS);
+        tmem_alloc(tmem_slot, C::TMEM_COLS);
         tmem_relinquish();
     }
     __syncthreads();
@@ -215,7 +496,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
                     uint8_t* sa = smem + stage * STAGE_BYTES;
                     tma_load_2d(sa, &tmA, &full[stage], kb * BK, m_blk * BM);
-                    tma_load_2d(sa + A_BYTES, &tmB, &full[stage], kb * BK, n_blk * BN);
+                    tma_load_2d(sa + A_BYTES, &tmB, &full[stage], kb * BK, n_blk * BNT);
                     armed[stage] = true;
                     armed_phase[stage] = phase;
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -239,7 +520,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
                 if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, g.err)) break;
                 tc_fence_after();
-                const uint32_t d = tmem_base + (uint32_t)(acc * BN);
+                const uint32_t d = tmem_base + (uint32_t)(acc * BNT);
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
                     if (!mbar_wait(&full[stage], phase, abort_flag, g.err)) { ok = false; break; }
                     tc_fence_after();
@@ -247,7 +528,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                     const uint32_t b0 = a0 + A_BYTES;
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
-                        tc_mma(d, sdesc_sw128(a0 + k * 32), sdesc_sw128(b0 + k * 32), IDESC, (kb | k) != 0);
+                        tc_mma(d, sdesc_sw128(a0 + k * 32), sdesc_sw128(b0 + k * 32), C::IDESC, (kb | k) != 0);
                     tc_commit(&empty[stage]);
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
@@ -265,31 +546,30 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const int lg = warp & 3;   // TMEM lane quarter this warp may access
         int acc = 0;
         uint32_t acc_phase = 0;
+        WarpStage ws{staging + lg * 2 * SLAB_BYTES, rbars + lg * 2, 0, 0, {}, {}};
         for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x) {
             const int m_blk = tile / g.n_tiles, n_blk = tile % g.n_tiles;
+            const int m0 = m_blk * BM + lg * 32, n0 = n_blk * BNT, end = min(n0 + BNT, g.N);
+            epilogue_prefetch<FORM>(g.e.bias, g.e.gate, g.staged, &maps.res, g.M, n0, end, m0, ws, lane);
             if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, g.err)) break;
             tc_fence_after();
-            const int m = m_blk * BM + lg * 32 + lane;
-            const uint32_t taddr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(acc * BN);
-            for (int c0 = 0; c0 < BN; c0 += 32) {
-                const int col0 = n_blk * BN + c0;
-                if (col0 >= g.N) break;
-                uint32_t r[32];
-                tmem_ld32(taddr + c0, r);
-                tmem_ld_wait();
-                if (m < g.M) epilogue_chunk(g.e, m, col0, r);
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&tempty[acc]);
+            const uint32_t taddr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(acc * BNT);
+            const bool ok = epilogue_tile<FORM>(g.e, g.staged, &maps, g.M, m0, n0, end, taddr, ws, abort_flag, g.err, lane, [&] {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&tempty[acc]);
+            });
+            if (!ok) break;
             acc ^= 1;
             if (acc == 0) acc_phase ^= 1u;
         }
+        if (lane == 0) bulk_wait_read<0>();    // the slabs stay until their stores have read them
+        epilogue_drain(ws);
     }
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem_base, TMEM_COLS);
+        tmem_dealloc(tmem_base, C::TMEM_COLS);
     }
 }
 
@@ -297,20 +577,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 // CTA-pair variant (clusters of 2, tcgen05 .cta_group::2): each pair computes a
 // 256 x 256 tile with 256 x 256 x 16 MMAs issued by the even CTA; each CTA
 // holds its 128 rows of A and its 128-row half of the W tile (32 KB per stage,
-// 6 stages), so twice the MMA work is buffered per shared-memory byte.  Both
-// CTAs' tile copies complete on the even CTA's mbarrier (the pair form of the
-// tensor copy), which the even CTA arms with both CTAs' bytes; the even CTA's
-// commits release both CTAs' stages and accumulators.  The
-// pair allocation is collective (both CTAs receive the same TMEM base; the
+// 6 stages beside the 32 KB of epilogue slabs), so twice the MMA work is
+// buffered per shared-memory byte.  Both CTAs' tile copies complete on the
+// even CTA's mbarrier (the pair form of the tensor copy), which the even CTA
+// arms with both CTAs' bytes; the even CTA's commits release both CTAs'
+// stages and accumulators.  The pair allocation is collective (both CTAs receive the same TMEM base; the
 // leader's base is used for every access and a mismatch is reported), and two
 // 256-column accumulators let a tile's epilogue overlap the next tile's MMAs.
-constexpr int STAGES2 = 7;
+constexpr int STAGES2 = 6;
 constexpr uint32_t A2_BYTES = 128 * BK * 2;
 constexpr uint32_t B2_BYTES = 128 * BK * 2;                  // half of the 256-row W tile
 constexpr uint32_t STAGE2_BYTES = A2_BYTES + B2_BYTES;
 constexpr uint32_t TMEM2_COLS = 512;
 constexpr uint32_t IDESC2 = idesc_bf16(256, 256);
-constexpr size_t SMEM2_BYTES = STAGES2 * STAGE2_BYTES + 1024 + 512;
+constexpr size_t SMEM2_BYTES = STAGES2 * STAGE2_BYTES + STAGING_BYTES + 1024 + 512;
+static_assert(SMEM2_BYTES <= 227 * 1024, "shared memory per CTA");
 
 // Pair-kernel raster: the N tiles are split into groups of group_n; inside a
 // group the tiles run N-fastest over every 256-row M block.  A group's slab
@@ -341,18 +622,22 @@ __device__ __forceinline__ int grouped_tile(const GemmArgs& g, int m_pairs0, int
     return 1;
 }
 
+template <int FORM>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
+                    const __grid_constant__ EpiMaps maps, const __grid_constant__ EpiMaps maps1,
                     const __grid_constant__ GemmArgs g) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES2 * STAGE2_BYTES);   // even CTA: both halves landed
+    uint8_t* staging = smem + STAGES2 * STAGE2_BYTES;
+    uint64_t* full = reinterpret_cast<uint64_t*>(staging + STAGING_BYTES);   // even CTA: both halves landed
     uint64_t* empty = full + STAGES2;
     uint64_t* tfull = empty + STAGES2;         // [2]
     uint64_t* tempty = tfull + 2;              // [2] even CTA: both CTAs' epilogues are done
     uint64_t* mma_done = tempty + 2;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
+    uint64_t* rbars = mma_done + 1;            // [4 warps][2] residual slabs
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rbars + 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -371,6 +656,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             mbar_init(&tempty[a], 8);          // 4 epilogue warps in each CTA
         }
         mbar_init(mma_done, 1);
+        for (int i = 0; i < 8; ++i) mbar_init(&rbars[i], 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -472,37 +758,41 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         const int lg = warp & 3;
         int acc = 0;
         uint32_t acc_phase = 0;
+        WarpStage ws{staging + lg * 2 * SLAB_BYTES, rbars + lg * 2, 0, 0, {}, {}};
         for (int tile = cluster_id; tile < num_tiles; tile += n_clusters) {
             int mb, n_blk;
             const int prob = grouped_tile(g, m_pairs, tiles0, tile, mb, n_blk);
-            const int Mp = prob ? g.M1 : g.M;
-            const int mrow = mb * 256 + (int)rank * 128;
+            const int m0 = mb * 256 + (int)rank * 128 + lg * 32, n0 = n_blk * BN, end = min(n0 + BN, g.N);
+            // the second problem differs in its pointers, rows and maps only
+            const int Mp = prob ? g.M1 : g.M, staged = prob ? g.staged1 : g.staged;
+            const EpiMaps* mp = prob ? &maps1 : &maps;
+            Epi e = g.e;
+            if (prob) {
+                e.bias = g.e1.bias;
+                e.gate = g.e1.gate;
+                e.out = g.e1.out;
+                e.res = g.e1.res;
+                e.row_off = g.e1.row_off;
+            }
+            epilogue_prefetch<FORM>(e.bias, e.gate, staged, &mp->res, Mp, n0, end, m0, ws, lane);
             if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, g.err)) break;
             tc_fence_after();
-            const int m = mrow + lg * 32 + lane;
             const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(acc * BN);
-            for (int c0 = 0; c0 < BN; c0 += 32) {
-                const int col0 = n_blk * BN + c0;
-                if (col0 >= g.N) break;
-                uint32_t r[32];
-                tmem_ld32(taddr + c0, r);
-                tmem_ld_wait();
-                if (m < Mp) {
-                    // two direct calls (each reads its epilogue from the
-                    // kernel parameters; a selected reference would copy it)
-                    if (prob) epilogue_chunk(g.e1, m, col0, r);
-                    else epilogue_chunk(g.e, m, col0, r);
+            auto release = [&] {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    if (rank == 0) mbar_arrive(&tempty[acc]);
+                    else mbar_arrive_remote(acc == 0 ? leader_tempty0 : leader_tempty1);
                 }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                if (rank == 0) mbar_arrive(&tempty[acc]);
-                else mbar_arrive_remote(acc == 0 ? leader_tempty0 : leader_tempty1);
-            }
+            };
+            const bool ok = epilogue_tile<FORM>(e, staged, mp, Mp, m0, n0, end, taddr, ws, abort_flag, g.err, lane, release);
+            if (!ok) break;
             acc ^= 1;
             if (acc == 0) acc_phase ^= 1u;
         }
+        if (lane == 0) bulk_wait_read<0>();    // the slabs stay until their stores have read them
+        epilogue_drain(ws);
     }
     __syncthreads();
     cluster_sync_all();
@@ -546,7 +836,8 @@ bool encode_tmap_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t
 }
 
 bool encode_tmap_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint64_t s1_bytes,
-                    uint64_t s2_bytes, uint32_t b0, uint32_t b1, uint32_t b2, std::string* why, bool f16) {
+                    uint64_t s2_bytes, uint32_t b0, uint32_t b1, uint32_t b2, std::string* why, bool f16,
+                    CUtensorMapSwizzle swizzle) {
     auto fn = get_encode();
     if (!fn) { if (why) *why = "cuTensorMapEncodeTiled unavailable"; return false; }
     cuuint64_t dims[3] = {d0, d1, d2};
@@ -555,8 +846,7 @@ bool encode_tmap_3d(CUtensorMap* map, const void* base, uint64_t d0, uint64_t d1
     cuuint32_t es[3] = {1, 1, 1};
     CUresult r = fn(map, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
                     const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) { if (why) *why = "cuTensorMapEncodeTiled failed: " + std::to_string((int)r); return false; }
     return true;
 }
@@ -576,11 +866,30 @@ wdc_status check_operands(Ctx* c, const void* A, const void* W, const Epi& e) {
     return WDC_OK;
 }
 
+using Kernel1 = void (*)(const CUtensorMap, const CUtensorMap, const EpiMaps, const GemmArgs);
+using Kernel2 = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const EpiMaps,
+                         const EpiMaps, const GemmArgs);
+constexpr Kernel1 kKernel1[kForms] = {gemm_tc_kernel<256, 0>, gemm_tc_kernel<256, 1>, gemm_tc_kernel<256, 2>,
+                                      gemm_tc_kernel<256, 3>, gemm_tc_kernel<256, 4>};
+constexpr Kernel2 kKernel2[kForms] = {gemm_tc2_kernel<0>, gemm_tc2_kernel<1>, gemm_tc2_kernel<2>, gemm_tc2_kernel<3>,
+                                      gemm_tc2_kernel<4>};
+
+int form_of(const Epi& e) {
+    switch (e.mode) {
+        case kEpiResid: return kFormResid;
+        case kEpiQKV: return kFormQKV;
+        case kEpiUnpatch: return kFormUnpatch;
+        default: return e.gelu ? kFormGelu : kFormStore;
+    }
+}
+
 void set_attrs() {
     static bool attr_set = false;
     if (!attr_set) {
-        cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
-        cudaFuncSetAttribute(gemm_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM2_BYTES);
+        for (int f = 0; f < kForms; ++f) {
+            cudaFuncSetAttribute(kKernel1[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmCfg<256>::SMEM);
+            cudaFuncSetAttribute(kKernel2[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM2_BYTES);
+        }
         attr_set = true;
     }
 }
@@ -612,10 +921,34 @@ GemmArgs make_args(Ctx* c, int M, int N, int K, const Epi& e) {
     return g;
 }
 
+// Tensor maps of an epilogue's staged stores and residual loads; 0 when its
+// form takes none (unpatchify; a residual whose rows repeat; a residual row
+// that is not the output's).
+bool encode_epilogue(const Epi& e, int M, int N, EpiMaps* m, int* staged, std::string* why) {
+    *staged = 0;
+    if (e.mode == kEpiUnpatch || (e.mode == kEpiResid && e.res_rows > 0 && M > e.res_rows)) return true;
+    if (e.mode == kEpiQKV) {
+        const uint64_t d = e.d, L = e.L, heads = (uint64_t)e.nb * e.H;
+        if (!encode_tmap_3d(&m->out, e.q, d, L, heads, d * 2, L * d * 2, 64, 32, 1, why) ||
+            !encode_tmap_3d(&m->res, e.k, d, L, heads, d * 2, L * d * 2, 64, 32, 1, why) ||
+            !encode_tmap_3d(&m->vt, e.vt, L, d, heads, (uint64_t)e.ldv * 2, (uint64_t)e.ldv * d * 2, 32, 64, 1, why,
+                            true, CU_TENSOR_MAP_SWIZZLE_64B))
+            return false;
+    } else {
+        if (!encode_tmap_2d(&m->out, e.out, (uint64_t)N, (uint64_t)M, (uint64_t)e.ldo * 2, 64, 32, why)) return false;
+        if (e.mode == kEpiResid &&
+            !encode_tmap_2d(&m->res, e.res, (uint64_t)N, (uint64_t)M, (uint64_t)e.ldo * 2, 64, 32, why))
+            return false;
+    }
+    *staged = 1;
+    return true;
+}
+
 // Pair-kernel launch: a persistent grid of as many CTA pairs as can be
 // resident, capped by the tile count.
 wdc_status launch_pair(Ctx* c, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& ta1,
-                       const CUtensorMap& tb1, const GemmArgs& g, cudaStream_t s) {
+                       const CUtensorMap& tb1, const EpiMaps& maps, const EpiMaps& maps1, const GemmArgs& g,
+                       cudaStream_t s) {
     const int tiles = ((g.m_tiles + 1) / 2) * g.n_tiles + (g.nprob > 1 ? g.m_pairs1 * g.n_tiles : 0);
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kGemmThreads, 1, 1);
@@ -631,7 +964,7 @@ wdc_status launch_pair(Ctx* c, const CUtensorMap& ta, const CUtensorMap& tb, con
     static int max_clusters = 0;
     if (max_clusters == 0) {
         cfg.gridDim = dim3(c->num_sms, 1, 1);
-        if (cudaOccupancyMaxActiveClusters(&max_clusters, gemm_tc2_kernel, &cfg) != cudaSuccess || max_clusters < 1) {
+        if (cudaOccupancyMaxActiveClusters(&max_clusters, kKernel2[0], &cfg) != cudaSuccess || max_clusters < 1) {
             cudaGetLastError();
             max_clusters = c->num_sms / 2;
         }
@@ -639,7 +972,7 @@ wdc_status launch_pair(Ctx* c, const CUtensorMap& ta, const CUtensorMap& tb, con
     int clusters = max_clusters < c->num_sms / 2 ? max_clusters : c->num_sms / 2;
     if (tiles < clusters) clusters = tiles;
     cfg.gridDim = dim3(2 * clusters, 1, 1);
-    cudaLaunchKernelEx(&cfg, gemm_tc2_kernel, ta, tb, ta1, tb1, g);
+    cudaLaunchKernelEx(&cfg, kKernel2[form_of(g.e)], ta, tb, ta1, tb1, maps, maps1, g);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(err));
     return WDC_OK;
@@ -657,11 +990,13 @@ wdc_status tc_gemm(Ctx* c, const void* A, const void* W, int M, int N, int K, co
     if (!encode_tmap_2d(&ta, A, (uint64_t)K, (uint64_t)M, (uint64_t)K * 2, BK, BM, &why) ||
         !encode_tmap_2d(&tb, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * 2, BK, pair ? BN / 2 : BN, &why))
         return fail(c, WDC_ERR_CUDA, why);
-    const GemmArgs g = make_args(c, M, N, K, e);
-    if (pair) return launch_pair(c, ta, tb, ta, tb, g, s);
+    GemmArgs g = make_args(c, M, N, K, e);
+    EpiMaps maps{};
+    if (!encode_epilogue(e, M, N, &maps, &g.staged, &why)) return fail(c, WDC_ERR_CUDA, why);
+    if (pair) return launch_pair(c, ta, tb, ta, tb, maps, maps, g, s);
     const int tiles = g.m_tiles * g.n_tiles;
     const int grid = tiles < c->num_sms ? tiles : c->num_sms;
-    gemm_tc_kernel<<<grid, kGemmThreads, SMEM_BYTES, s>>>(ta, tb, g);
+    kKernel1[form_of(e)]<<<grid, kGemmThreads, GemmCfg<256>::SMEM, s>>>(ta, tb, maps, g);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(err));
     return WDC_OK;
@@ -696,7 +1031,10 @@ wdc_status tc_gemm_grouped(Ctx* c, const void* A0, const void* W0, int M0, const
     g.M1 = M1;
     g.m_pairs1 = (M1 + 255) / 256;
     g.e1 = e1;
-    return launch_pair(c, ta, tb, ta1, tb1, g, s);
+    EpiMaps maps{}, maps1{};
+    if (!encode_epilogue(e0, M0, N, &maps, &g.staged, &why) || !encode_epilogue(e1, M1, N, &maps1, &g.staged1, &why))
+        return fail(c, WDC_ERR_CUDA, why);
+    return launch_pair(c, ta, tb, ta1, tb1, maps, maps1, g, s);
 }
 
 }  // namespace wdc

@@ -1,0 +1,73 @@
+"""The GEMM epilogues where their 32-row x 64-column slabs can go wrong: row
+and column remainders, V^T slabs that do not start on a 16-byte boundary, and
+slabs that hold rows of two samples or of both streams."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import rel_l2
+from oracle import dit
+from oracle.params import DiTConfig
+from paper_2608_01845_gb300 import synth, wdc
+
+pytestmark = pytest.mark.gpu
+
+MODEL = dict(layers=1, hidden=256, heads=4, head_dim=64, mlp=512, temb_dim=256, freq_dim=256, in_ch=16, frames=3,
+             height=14, width=22, patch=2, cond_tokens=16, cond_dim=64, dual_stream=0)
+
+
+def _dev(a, dtype=torch.float32):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda().to(dtype)
+
+
+@pytest.mark.parametrize("M", [1, 31, 33, 127, 128, 255, 256, 257, 289])
+@pytest.mark.parametrize("N", [32, 64, 96, 288])
+@pytest.mark.parametrize("mode", ["store", "gelu", "resid"])
+def test_gemm_rows_and_columns(M, N, mode):
+    """Against fp64: one rounding of the result to bf16 (8 significant bits: at
+    most 2^-8 relative an element, so at most that in the 2-norm) and fp32 sums
+    of K terms; nothing is written past the last row."""
+    K = 72
+    ctx = wdc.Context(wdc.make_config(dtype=wdc.BF16, **MODEL), 2)
+    A, W = synth.bf16_round(synth.normal(1, (M, K))), synth.bf16_round(synth.normal(2, (N, K), 0.1))
+    b = synth.normal(3, (N,), 0.5)
+    want = A.astype(np.float64) @ W.astype(np.float64).T + b
+    buf = torch.full((M + 40, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    C, kw = buf[:M], {}
+    if mode == "gelu":
+        kw["gelu"], want = True, dit.gelu_tanh(want)
+    elif mode == "resid":
+        R, g = synth.bf16_round(synth.normal(4, (M, N))), synth.normal(5, (N,))
+        want = R.astype(np.float64) + g * want
+        kw.update(res=_dev(R, torch.bfloat16), gate=_dev(g))
+    ctx.op_gemm(_dev(A, torch.bfloat16), _dev(W, torch.bfloat16), C, bias=_dev(b), **kw)
+    torch.cuda.synchronize()
+    assert ctx.device_errors() == 0
+    assert rel_l2(C.float().cpu().numpy(), want) <= 2.0 ** -8 + K * 2.0 ** -22
+    assert bool((buf[M:] == 7.0).all())
+
+
+@pytest.mark.parametrize("Lc,dual,d", [(13, 0, 64), (13, 1, 64), (24, 1, 128), (37, 1, 128), (300, 1, 64), (1, 0, 128)])
+def test_forward_slabs_across_samples_and_streams(Lc, dual, d):
+    """A forward against the oracle, and a batch of three bitwise equal to its
+    samples' own forwards, with condition-token counts that leave the video
+    rows' V^T slabs unaligned and put two samples into one slab."""
+    cfgd = dict(MODEL, cond_tokens=Lc, dual_stream=dual, head_dim=d, heads=256 // d)
+    W = synth.dit_weights(cfgd, 7, std=0.06, bias_std=0.05, bf16=True)
+    ctx = wdc.Context(wdc.make_config(dtype=wdc.BF16, max_batch=3, **cfgd), 2)
+    ctx.set_weights(W)
+    z = [synth.latent(20 + b, (16, 3, 14, 22)) for b in range(3)]
+    ct = [synth.cond_tokens(30 + b, Lc, 64) for b in range(3)]
+    zd, cd = [_dev(a.reshape(-1)) for a in z], [_dev(a) for a in ct]
+    one = []
+    for b in range(3):
+        one.append(torch.empty_like(zd[b]))
+        ctx.dit_forward(zd[b], 600.0, cd[b], one[b])
+    many = [torch.empty_like(t) for t in zd]
+    ctx.dit_forward_batch(zd, 600.0, cd, many)
+    torch.cuda.synchronize()
+    assert ctx.device_errors() == 0
+    for b in range(3):
+        assert torch.equal(one[b], many[b])
+    want = dit.forward(W, DiTConfig(**cfgd), z[0], 600.0, ct[0])
+    assert rel_l2(one[0].cpu().numpy(), want) <= 2e-2
