@@ -24,9 +24,9 @@ namespace wdc {
 // tcgen05 paths (gemm_tc.cu, attn_tc.cu); return false when the shape is not
 // supported so the caller can report it.
 bool tc_gemm_supported(int M, int N, int K);
-wdc_status tc_gemm(Ctx* c, const void* A, const void* W, int M, int N, int K, const Epi& e, cudaStream_t s);
-wdc_status tc_gemm_grouped(Ctx* c, const void* A0, const void* W0, int M0, const Epi& e0, const void* A1,
-                           const void* W1, int M1, const Epi& e1, int N, int K, cudaStream_t s);
+wdc_status tc_gemm(Ctx* c, const void* A, const void* W, int M, int N, int K, const Epi& e, int sample, cudaStream_t s);
+wdc_status tc_gemm_grouped(Ctx* c, const void* A0, const void* W0, int M0, int sample0, const Epi& e0, const void* A1,
+                           const void* W1, int M1, int sample1, const Epi& e1, int N, int K, cudaStream_t s);
 bool tc_attention_supported(int L, int d);
 wdc_status tc_attention(Ctx* c, const void* q, const void* k, const void* vt, int ldv, void* o, int H, int L, int d,
                         int Hs, int Lc, cudaStream_t s);
@@ -463,14 +463,16 @@ void launch_ln_mod(const void* x, void* h, int r0, int r1, int D, const float* s
 // ---------------------------------------------------------------- dispatch
 // bf16 runs on the tcgen05 kernels only: a shape outside their limits is an
 // error, not a silent SIMT run.  The SIMT kernels serve the fp32 parity mode.
-static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int N, int K, const Epi& e, cudaStream_t s) {
+// M rows in all, nb samples' worth: the tcgen05 GEMM splits K by one sample's
+// rows, so that a sample's result does not depend on its batch.
+static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int nb, int N, int K, const Epi& e, cudaStream_t s) {
     if (M <= 0 || N <= 0) return WDC_OK;
     if (c->cfg.dtype == WDC_BF16) {
         if (!tc_gemm_supported(M, N, K))
             return fail(c, WDC_ERR_UNSUPPORTED, "bf16 GEMM " + std::to_string(M) + "x" + std::to_string(N) + "x" +
                                                     std::to_string(K) + ": the tcgen05 GEMM needs N % 32 == 0 and K % 8 == 0");
         LaunchScope ls(c, WDC_K_GEMM, s);
-        return tc_gemm(c, A, W, M, N, K, e, s);
+        return tc_gemm(c, A, W, M, N, K, e, M / nb, s);
     }
     LaunchScope ls(c, WDC_K_GEMM, s);
     dim3 grid(blocks_for(N, 64), blocks_for(M, 64));
@@ -485,16 +487,16 @@ static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int N, int K
 // condition rows, each with its own weights and epilogue): one grouped
 // tcgen05 launch in bf16, two SIMT launches in the fp32 parity mode.
 static wdc_status gemm2(Ctx* c, const void* A0, const void* W0, int M0, const Epi& e0, const void* A1,
-                        const void* W1, int M1, const Epi& e1, int N, int K, cudaStream_t s) {
+                        const void* W1, int M1, const Epi& e1, int nb, int N, int K, cudaStream_t s) {
     if (c->cfg.dtype != WDC_BF16) {
-        wdc_status st = gemm(c, A0, W0, M0, N, K, e0, s);
-        return st ? st : gemm(c, A1, W1, M1, N, K, e1, s);
+        wdc_status st = gemm(c, A0, W0, M0, nb, N, K, e0, s);
+        return st ? st : gemm(c, A1, W1, M1, nb, N, K, e1, s);
     }
     if (!tc_gemm_supported(M0 > 0 ? M0 : 1, N, K))
         return fail(c, WDC_ERR_UNSUPPORTED, "bf16 GEMM N=" + std::to_string(N) + " K=" + std::to_string(K) +
                                                 ": the tcgen05 GEMM needs N % 32 == 0 and K % 8 == 0");
     LaunchScope ls(c, WDC_K_GEMM, s);
-    return tc_gemm_grouped(c, A0, W0, M0, e0, A1, W1, M1, e1, N, K, s);
+    return tc_gemm_grouped(c, A0, W0, M0, M0 / nb, e0, A1, W1, M1, M1 / nb, e1, N, K, s);
 }
 
 // V^T rows have stride ldv (>= L).  bf16 runs on the tcgen05 kernel only;
@@ -806,10 +808,10 @@ static wdc_status run_block(Ctx* c, int layer, void* x, const float* mod, int nb
     auto at_row = [&](void* base, int sidx, int width) { return (char*)base + (size_t)r0[sidx] * width * es; };
     auto lin_gemm = [&](const std::vector<Lin>& W, const void* A, int width, int N, Epi* e) -> wdc_status {
         const Lin& w0 = W[layer * S];
-        if (S == 1) return gemm(c, at_row(const_cast<void*>(A), 0, width), w0.w, rows_of(0), N, width, e[0], s);
+        if (S == 1) return gemm(c, at_row(const_cast<void*>(A), 0, width), w0.w, rows_of(0), nb, N, width, e[0], s);
         const Lin& w1 = W[layer * S + 1];
         return gemm2(c, at_row(const_cast<void*>(A), 0, width), w0.w, rows_of(0), e[0],
-                     at_row(const_cast<void*>(A), 1, width), w1.w, rows_of(1), e[1], N, width, s);
+                     at_row(const_cast<void*>(A), 1, width), w1.w, rows_of(1), e[1], nb, N, width, s);
     };
     for (int sidx = 0; sidx < S; ++sidx) ln_mod(c, x, t->h, r0[sidx], r1[sidx], m6[sidx] + 0 * D, m6[sidx] + 1 * D, 0, s);
     {
@@ -904,7 +906,7 @@ wdc_status dit_forward_batch(Ctx* c, int nb, const float* const* z, float t_mode
         }
         Epi e{};
         e.mode = kEpiStore; e.bias = t->cond.b; e.out = t->x; e.ldo = D;
-        if ((st = gemm(c, t->condx, t->cond.w, nb * t->Lc, D, t->Dc, e, s))) return st;
+        if ((st = gemm(c, t->condx, t->cond.w, nb * t->Lc, nb, D, t->Dc, e, s))) return st;
     }
     {
         const long long nt = (long long)t->Lv * t->P * nb;
@@ -918,7 +920,7 @@ wdc_status dit_forward_batch(Ctx* c, int nb, const float* const* z, float t_mode
         Epi e{};
         char* xv = (char*)t->x + (size_t)nb * t->Lc * D * es;
         e.mode = kEpiResid; e.bias = t->patch.b; e.out = xv; e.res = t->pe; e.res_rows = t->Lv; e.ldo = D; e.gate = nullptr;
-        if ((st = gemm(c, t->tok, t->patch.w, nb * t->Lv, D, t->P, e, s))) return st;
+        if ((st = gemm(c, t->tok, t->patch.w, nb * t->Lv, nb, D, t->P, e, s))) return st;
     }
     for (int l = 0; l < t->layers; ++l)
         if ((st = run_block(c, l, t->x, t->mods + (size_t)l * t->S * 6 * D, nb, s))) return st;
@@ -927,7 +929,7 @@ wdc_status dit_forward_batch(Ctx* c, int nb, const float* const* z, float t_mode
     ln_mod(c, t->x, t->h, nb * t->Lc, nb * t->L, fm, fm + D, nb * t->Lc, s);
     Epi e{};
     e.mode = kEpiUnpatch; e.bias = t->fin.b; e.v = v; e.C = g.in_ch; e.F = g.frames; e.Hh = g.height; e.Ww = g.width; e.p = g.patch;
-    if ((st = gemm(c, t->h, t->fin.w, nb * t->Lv, t->P, D, e, s))) return st;
+    if ((st = gemm(c, t->h, t->fin.w, nb * t->Lv, nb, t->P, D, e, s))) return st;
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("forward: ") + cudaGetErrorString(ce));
     return WDC_OK;
@@ -983,7 +985,7 @@ wdc_status op_gemm(Ctx* c, const void* A, const void* W, const float* bias, void
     if (!A || !W || !C || M <= 0 || N <= 0 || K <= 0) return fail(c, WDC_ERR_INVALID_ARG, "bad gemm arguments");
     Epi e{};
     e.mode = res ? kEpiResid : kEpiStore; e.bias = bias; e.gelu = gelu; e.out = C; e.ldo = N; e.res = res; e.gate = gate;
-    wdc_status st = gemm(c, A, W, M, N, K, e, s);
+    wdc_status st = gemm(c, A, W, M, 1, N, K, e, s);
     if (st) return st;
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("gemm: ") + cudaGetErrorString(ce));

@@ -2,24 +2,34 @@
 // the DiT's fused epilogues: C = epilogue(A W^T), A [M, K], W [N, K] bf16,
 // fp32 accumulation in tensor memory.
 //
-// Persistent kernel, one CTA per SM, 6 warps:
-//   warp 0      TMA producer: A (128 x 64) and W (256 x 64) tiles into a
-//               4-stage shared-memory ring (128-byte swizzle), one mbarrier
-//               pair per stage;
-//   warp 1      MMA issuer: one thread issues tcgen05.mma 128x256x16 into one
-//               of two TMEM accumulators (2 x 256 columns), commits the smem
-//               stage back to the producer and the accumulator to the
-//               epilogue;
+// Three kernels, 6 warps a CTA (TMA producer, MMA issuer, 4 epilogue warps):
+//   gemm_tc2_kernel   persistent, CTA pairs, 256 x 256 tiles: shapes with
+//                     tiles for (nearly) every pair;
+//   gemm_tc_kernel    persistent, one CTA a tile of 128 x 128 or 128 x 64:
+//                     shapes that would leave most pairs without a tile;
+//   gemm_split_kernel one 128 x 128 tile a cluster, its CTAs each summing a
+//                     part of K and reducing through distributed shared memory:
+//                     shapes with too few tiles for the SMs and a K to split.
+// choose_gemm picks one by the estimated cycles of each.
+//   warp 0      TMA producer: A and W tiles of 64 columns of K into a
+//               shared-memory ring (128-byte swizzle), one mbarrier pair per
+//               stage;
+//   warp 1      MMA issuer: one thread issues the tcgen05.mma of each stage
+//               into one of two TMEM accumulators, commits the stage back to
+//               the producer and the accumulator to the epilogue;
 //   warps 2-5   epilogue (epilogue_tile): each warp owns its 32-lane TMEM
 //               quarter = 32 rows and works through the tile 64 columns at a
 //               time: tcgen05.ld, bias / GELU / gated residual, bf16 into a
 //               swizzled shared-memory slab, one TMA store per slab; then
 //               release the accumulator so the next tile's MMAs overlap.
-// Tiles are visited N-fastest inside groups of N tiles sized so a group's
-// slab of W stays in L2 (about 40 MB), so W is read from DRAM about once and
-// A once per group.
+// The pair kernel's tiles are visited N-fastest inside groups of N tiles sized
+// so a group's slab of W stays in L2 (about 40 MB), so W is read from DRAM
+// about once and A once per group.
 // Tails: TMA zero-fills rows past M / N and columns past K; the epilogue
 // masks rows >= M.  Every mbarrier wait is bounded.
+// Each output element is accumulated over K in the same order by the pair and
+// the one-CTA kernels, and whether K is split depends on one sample's rows
+// only, so a sample's results are the same bits in any batch.
 #include "dit_kernels.cuh"
 #include "ptx.cuh"
 
@@ -44,7 +54,7 @@ template <int BNT>
 struct GemmCfg {
     static constexpr uint32_t B_BYTES = BNT * BK * 2;
     static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int STAGES = BNT == 256 ? 4 : (BNT == 128 ? 6 : 8);
+    static constexpr int STAGES = BNT == 128 ? 6 : 8;
     static constexpr uint32_t TMEM_COLS = 2 * BNT;
     static constexpr uint32_t IDESC = idesc_bf16(BM, BNT);
     static constexpr size_t SMEM = STAGES * STAGE_BYTES + STAGING_BYTES + 1024 + 256;
@@ -61,19 +71,33 @@ struct EpiMaps {
 
 struct GemmArgs {
     int M, N, K;
-    int m_tiles, n_tiles, k_blocks;
+    int m_tiles, n_tiles, k_blocks;   // 128-row tiles; N tiles of the kernel's width; 64-column K blocks
     int group_n;            // pair kernel: N tiles per raster group
     Epi e;
     unsigned* err;
-    // pair kernel, grouped launch: a second problem with the same N and K
+    // grouped launch: a second problem with the same N and K
     // (its own A, W, M and epilogue) whose tiles follow the first problem's
     int nprob;              // 1 or 2
-    int M1, m_pairs1;
+    int M1, m_tiles1;       // m_tiles1 counts 128-row tiles, as m_tiles
     Epi e1;
     // whether each problem's epilogue has its tensor maps (else every row goes
     // through the direct stores of epilogue_chunk)
     int staged, staged1;
 };
+
+// Epilogue of problem `prob`: the second problem differs from the first in
+// these fields only.
+__device__ __forceinline__ Epi problem_epilogue(const GemmArgs& g, int prob) {
+    Epi e = g.e;
+    if (prob) {
+        e.bias = g.e1.bias;
+        e.gate = g.e1.gate;
+        e.out = g.e1.out;
+        e.res = g.e1.res;
+        e.row_off = g.e1.row_off;
+    }
+    return e;
+}
 
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
@@ -437,7 +461,9 @@ __device__ __forceinline__ bool epilogue_tile(const Epi& e, int staged, const Ep
 template <int BNT, int FORM>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ EpiMaps maps, const __grid_constant__ GemmArgs g) {
+                   const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
+                   const __grid_constant__ EpiMaps maps, const __grid_constant__ EpiMaps maps1,
+                   const __grid_constant__ GemmArgs g) {
     using C = GemmCfg<BNT>;
     constexpr int STAGES = C::STAGES;
     constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES;
@@ -471,6 +497,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     if (warp == 0 && lane == 0) {
         prefetch_tmap(&tmA);
         prefetch_tmap(&tmB);
+        if (g.nprob > 1) {
+            prefetch_tmap(&tmA1);
+            prefetch_tmap(&tmB1);
+        }
     }
     if (warp == 1) {
         tmem_alloc(tmem_slot, C::TMEM_COLS);
@@ -479,39 +509,46 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    const int num_tiles = g.m_tiles * g.n_tiles;
+    // tiles of the first problem, then of the second, N-fastest
+    const int tiles0 = g.m_tiles * g.n_tiles;
+    const int num_tiles = tiles0 + (g.nprob > 1 ? g.m_tiles1 * g.n_tiles : 0);
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             int stage = 0;
             uint32_t phase = 0;
-            uint32_t armed_phase[STAGES];
-            bool armed[STAGES];
-            for (int s = 0; s < STAGES; ++s) armed[s] = false;
+            uint32_t armed = 0, parity = 0;        // per stage: a copy was issued; its phase
             bool ok = true;
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-                const int m_blk = tile / g.n_tiles, n_blk = tile % g.n_tiles;
+                const int prob = tile >= tiles0, r = tile - prob * tiles0;
+                const int m_blk = r / g.n_tiles, n_blk = r % g.n_tiles;
+                const CUtensorMap* mA = prob ? &tmA1 : &tmA;
+                const CUtensorMap* mB = prob ? &tmB1 : &tmB;
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.err)) { ok = false; break; }
-                    mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
-                    uint8_t* sa = smem + stage * STAGE_BYTES;
-                    tma_load_2d(sa, &tmA, &full[stage], kb * BK, m_blk * BM);
-                    tma_load_2d(sa + A_BYTES, &tmB, &full[stage], kb * BK, n_blk * BNT);
-                    armed[stage] = true;
-                    armed_phase[stage] = phase;
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
+                        uint8_t* sa = smem + stage * STAGE_BYTES;
+                        tma_load_2d(sa, mA, &full[stage], kb * BK, m_blk * BM);
+                        tma_load_2d(sa + A_BYTES, mB, &full[stage], kb * BK, n_blk * BNT);
+                    }
+                    __syncwarp();
+                    armed |= 1u << stage;
+                    parity = (parity & ~(1u << stage)) | (phase << stage);
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
             }
             // drain: every issued copy has landed before the CTA may exit
             for (int s = 0; s < STAGES; ++s) {
-                if (!armed[s]) continue;
+                if (!((armed >> s) & 1)) continue;
                 const unsigned long long t0 = globaltimer();
-                while (!mbar_try_wait(&full[s], armed_phase[s]) && globaltimer() - t0 < kWaitLimitNs) {
+                while (!mbar_try_wait(&full[s], (parity >> s) & 1) && globaltimer() - t0 < kWaitLimitNs) {
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
+            const uint64_t da = sdesc_sw128(smem_u32(smem)), db = sdesc_sw128(smem_u32(smem) + A_BYTES);
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
@@ -524,20 +561,23 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
                     if (!mbar_wait(&full[stage], phase, abort_flag, g.err)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t a0 = smem_u32(smem + stage * STAGE_BYTES);
-                    const uint32_t b0 = a0 + A_BYTES;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        tc_mma(d, sdesc_sw128(a0 + k * 32), sdesc_sw128(b0 + k * 32), C::IDESC, (kb | k) != 0);
-                    tc_commit(&empty[stage]);
+                        for (int k = 0; k < BK / 16; ++k)
+                            tc_mma(d, sdesc_at(da, stage * STAGE_BYTES + k * 32), sdesc_at(db, stage * STAGE_BYTES + k * 32),
+                                   C::IDESC, (kb | k) != 0);
+                        tc_commit(&empty[stage]);
+                        if (kb + 1 == g.k_blocks) tc_commit(&tfull[acc]);
+                    }
+                    __syncwarp();
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
-                tc_commit(&tfull[acc]);
                 acc ^= 1;
                 if (acc == 0) acc_phase ^= 1u;
             }
-            // all MMAs issued by this thread have completed before TMEM is freed
-            tc_commit(mma_done);
+            // all MMAs issued by this warp have completed before TMEM is freed
+            if (elect_one()) tc_commit(mma_done);
+            __syncwarp();
             const unsigned long long t0 = globaltimer();
             while (!mbar_try_wait(mma_done, 0) && globaltimer() - t0 < kWaitLimitNs) {
             }
@@ -548,13 +588,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         uint32_t acc_phase = 0;
         WarpStage ws{staging + lg * 2 * SLAB_BYTES, rbars + lg * 2, 0, 0, {}, {}};
         for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x) {
-            const int m_blk = tile / g.n_tiles, n_blk = tile % g.n_tiles;
-            const int m0 = m_blk * BM + lg * 32, n0 = n_blk * BNT, end = min(n0 + BNT, g.N);
-            epilogue_prefetch<FORM>(g.e.bias, g.e.gate, g.staged, &maps.res, g.M, n0, end, m0, ws, lane);
+            const int prob = tile >= tiles0, r = tile - prob * tiles0;
+            const int m0 = (r / g.n_tiles) * BM + lg * 32, n0 = (r % g.n_tiles) * BNT, end = min(n0 + BNT, g.N);
+            const int Mp = prob ? g.M1 : g.M, staged = prob ? g.staged1 : g.staged;
+            const EpiMaps* mp = prob ? &maps1 : &maps;
+            const Epi e = problem_epilogue(g, prob);
+            epilogue_prefetch<FORM>(e.bias, e.gate, staged, &mp->res, Mp, n0, end, m0, ws, lane);
             if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, g.err)) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(acc * BNT);
-            const bool ok = epilogue_tile<FORM>(g.e, g.staged, &maps, g.M, m0, n0, end, taddr, ws, abort_flag, g.err, lane, [&] {
+            const bool ok = epilogue_tile<FORM>(e, staged, mp, Mp, m0, n0, end, taddr, ws, abort_flag, g.err, lane, [&] {
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&tempty[acc]);
@@ -645,7 +688,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const int cluster_id = blockIdx.x >> 1, n_clusters = gridDim.x >> 1;
     const int m_pairs = (g.m_tiles + 1) >> 1;  // 256-row tiles (m_tiles counts 128-row tiles)
     const int tiles0 = m_pairs * g.n_tiles;
-    const int num_tiles = tiles0 + (g.nprob > 1 ? g.m_pairs1 * g.n_tiles : 0);
+    const int num_tiles = tiles0 + (g.nprob > 1 ? ((g.m_tiles1 + 1) >> 1) * g.n_tiles : 0);
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES2; ++s) {
             mbar_init(&full[s], 1);
@@ -682,12 +725,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const uint32_t leader_tempty1 = mapa_shared(smem_u32(&tempty[1]), 0);
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             int stage = 0;
             uint32_t phase = 0;
-            uint32_t armed_phase[STAGES2];
-            bool armed[STAGES2];
-            for (int s = 0; s < STAGES2; ++s) armed[s] = false;
+            uint32_t armed = 0, parity = 0;        // per stage: a copy was issued; its phase
             bool ok = true;
             for (int tile = cluster_id; tile < num_tiles && ok; tile += n_clusters) {
                 int mb, nb;
@@ -698,33 +739,37 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 const int n0 = nb * BN + (int)rank * 128;
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.err)) { ok = false; break; }
-                    if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * STAGE2_BYTES);
-                    const uint32_t fb = mapa_shared(smem_u32(&full[stage]), 0);
-                    uint8_t* sa = smem + stage * STAGE2_BYTES;
-                    tma_load_2d_pair(sa, mA, fb, kb * BK, m0);
-                    tma_load_2d_pair(sa + A2_BYTES, mB, fb, kb * BK, n0);
-                    armed[stage] = true;
-                    armed_phase[stage] = phase;
+                    if (elect_one()) {
+                        if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * STAGE2_BYTES);
+                        const uint32_t fb = mapa_shared(smem_u32(&full[stage]), 0);
+                        uint8_t* sa = smem + stage * STAGE2_BYTES;
+                        tma_load_2d_pair(sa, mA, fb, kb * BK, m0);
+                        tma_load_2d_pair(sa + A2_BYTES, mB, fb, kb * BK, n0);
+                    }
+                    __syncwarp();
+                    armed |= 1u << stage;
+                    parity = (parity & ~(1u << stage)) | (phase << stage);
                     if (++stage == STAGES2) { stage = 0; phase ^= 1u; }
                 }
             }
             // drain: every copy of the pair has landed (even CTA's full) and the
             // MMAs have released every stage (both CTAs' empty)
             for (int s = 0; s < STAGES2; ++s) {
-                if (!armed[s]) continue;
+                if (!((armed >> s) & 1)) continue;
                 if (rank == 0) {
                     const unsigned long long t0 = globaltimer();
-                    while (!mbar_try_wait(&full[s], armed_phase[s]) && globaltimer() - t0 < kWaitLimitNs) {
+                    while (!mbar_try_wait(&full[s], (parity >> s) & 1) && globaltimer() - t0 < kWaitLimitNs) {
                     }
                 }
                 const unsigned long long t1 = globaltimer();
-                while (!mbar_try_wait(&empty[s], armed_phase[s]) && globaltimer() - t1 < kWaitLimitNs) {
+                while (!mbar_try_wait(&empty[s], (parity >> s) & 1) && globaltimer() - t1 < kWaitLimitNs) {
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             // MMA issuer for the pair
+            const uint64_t da = sdesc_sw128(smem_u32(smem)), db = sdesc_sw128(smem_u32(smem) + A2_BYTES);
             int stage = 0;
             uint32_t phase = 0;
             int acc = 0;
@@ -737,19 +782,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
                     if (!mbar_wait(&full[stage], phase, abort_flag, g.err)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t a0 = smem_u32(smem + stage * STAGE2_BYTES);
-                    const uint32_t b0 = a0 + A2_BYTES;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k)
-                        tc_mma2(d, sdesc_sw128(a0 + k * 32), sdesc_sw128(b0 + k * 32), IDESC2, (kb | k) != 0);
-                    tc_commit2_mc(&empty[stage], (uint16_t)0x3);
+                        for (int k = 0; k < BK / 16; ++k)
+                            tc_mma2(d, sdesc_at(da, stage * STAGE2_BYTES + k * 32), sdesc_at(db, stage * STAGE2_BYTES + k * 32),
+                                    IDESC2, (kb | k) != 0);
+                        tc_commit2_mc(&empty[stage], (uint16_t)0x3);
+                        if (kb + 1 == g.k_blocks) tc_commit2_mc(&tfull[acc], (uint16_t)0x3);
+                    }
+                    __syncwarp();
                     if (++stage == STAGES2) { stage = 0; phase ^= 1u; }
                 }
-                tc_commit2_mc(&tfull[acc], (uint16_t)0x3);
                 acc ^= 1;
                 if (acc == 0) acc_phase ^= 1u;
             }
-            tc_commit2_mc(mma_done, (uint16_t)0x1);
+            if (elect_one()) tc_commit2_mc(mma_done, (uint16_t)0x1);
+            __syncwarp();
             const unsigned long long t0 = globaltimer();
             while (!mbar_try_wait(mma_done, 0) && globaltimer() - t0 < kWaitLimitNs) {
             }
@@ -763,17 +811,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             int mb, n_blk;
             const int prob = grouped_tile(g, m_pairs, tiles0, tile, mb, n_blk);
             const int m0 = mb * 256 + (int)rank * 128 + lg * 32, n0 = n_blk * BN, end = min(n0 + BN, g.N);
-            // the second problem differs in its pointers, rows and maps only
             const int Mp = prob ? g.M1 : g.M, staged = prob ? g.staged1 : g.staged;
             const EpiMaps* mp = prob ? &maps1 : &maps;
-            Epi e = g.e;
-            if (prob) {
-                e.bias = g.e1.bias;
-                e.gate = g.e1.gate;
-                e.out = g.e1.out;
-                e.res = g.e1.res;
-                e.row_off = g.e1.row_off;
-            }
+            const Epi e = problem_epilogue(g, prob);
             epilogue_prefetch<FORM>(e.bias, e.gate, staged, &mp->res, Mp, n0, end, m0, ws, lane);
             if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, g.err)) break;
             tc_fence_after();
@@ -799,6 +839,272 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc2(own_base, TMEM2_COLS);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Split-K variant: one 128 x 128 tile a cluster of S = 2, 4 or 8 CTAs.  CTA r
+// sums K blocks [r kb / S, (r + 1) kb / S) into its tensor memory.  Once every
+// CTA is done with its ring, each sends the others their share of its columns
+// (128 / S) into their shared memory, and after a cluster barrier each adds the
+// S partial sums of its columns in rank order and runs the epilogue on them, 8
+// columns a thread at a time.
+// A CTA's main loop is bound by its shared memory: a 64-column block of K puts
+// 32 KB into it and the MMAs read as much, 430-480 cycles whatever the tile's
+// width (482 at 128, 450 at 64), so a small M with a deep K waits for few SMs.
+// Partial sums lie as [source][4 columns][row]: a warp sends one 512-byte run.
+// (Row by row, 16 bytes a packet, sending took 4-8k cycles; fetching instead of
+// sending, one round trip after another, more.)
+constexpr int SPLIT_BN = 128, SPLIT_STAGES = 6, SPLIT_MAX = 8;
+constexpr uint32_t SPLIT_STAGE_BYTES = A_BYTES + SPLIT_BN * BK * 2;
+constexpr size_t SPLIT_SMEM = SPLIT_STAGES * SPLIT_STAGE_BYTES + 1024 + 256;
+static_assert(SPLIT_SMEM <= 227 * 1024, "shared memory per CTA");
+static_assert(BM * SPLIT_BN * 4 <= SPLIT_STAGES * SPLIT_STAGE_BYTES, "partial sums fit the ring");
+// Byte offset of row `row`'s columns 4 c4 .. 4 c4 + 3 of the share of S in
+// source p's partial sums: rows are permuted by the column group, so that
+// lanes on one row and successive 8-column groups meet different banks.
+template <int S>
+__device__ __forceinline__ uint32_t split_at(int p, int c4, int row) {
+    return (uint32_t)((p * (SPLIT_BN / S / 4) + c4) * BM + (row ^ ((c4 >> 1) & 7))) * 16u;
+}
+
+__device__ __forceinline__ uint4 residual8(const Epi& e, int m, int col) {
+    const int rm = e.res_rows > 0 ? m % e.res_rows : m;
+    return *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(e.res) + (size_t)rm * e.ldo + col);
+}
+
+// Bias and gate (0 and 1 where there is none) of 8 columns.
+template <int FORM>
+__device__ __forceinline__ void columns8(const Epi& e, int col, float (&bias)[8], float (&gate)[8]) {
+    auto load = [&](const float* src, float none, float (&x)[8]) {
+        float4 a = make_float4(none, none, none, none), b = a;
+        if (src) {
+            a = __ldg(reinterpret_cast<const float4*>(src + col));
+            b = __ldg(reinterpret_cast<const float4*>(src + col) + 1);
+        }
+        x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
+        x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+    };
+    load(e.bias, 0.f, bias);
+    if (FORM == kFormResid) load(e.gate, 1.f, gate);
+}
+
+// Epilogue of 8 consecutive columns (one 16-byte store) of row m.
+template <int FORM>
+__device__ __forceinline__ void epilogue8(const Epi& e, int m, int col, float (&v)[8], const float (&bias)[8],
+                                          const float (&gate)[8], const uint4& rr) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] += bias[j];
+    if constexpr (FORM == kFormUnpatch) {
+        Epi plain = e;
+        plain.bias = nullptr;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) epi_apply<__nv_bfloat16>(plain, m, col + j, v[j]);
+        return;
+    }
+    if constexpr (FORM == kFormGelu) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = gelu_tanh_f(v[j]);
+    }
+    __nv_bfloat16* dst;
+    if constexpr (FORM == kFormQKV) {
+        const int which = col / e.D, c = col % e.D, dd = c % e.d;
+        int b, tok;
+        batch_token(e.row_off + m, e.nb, e.Lc, e.L, b, tok);
+        const size_t h = (size_t)b * e.H + c / e.d;
+        if (which == 2) {
+            __half* base = reinterpret_cast<__half*>(e.vt) + (h * e.d + dd) * e.ldv + tok;
+            bool sat = false;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) base[(size_t)j * e.ldv] = to_vt_half(v[j], sat);
+            if (sat && e.err) atomicOr(e.err, kErrVSaturated);
+            return;
+        }
+        dst = reinterpret_cast<__nv_bfloat16*>(which == 0 ? e.q : e.k) + (h * e.L + tok) * e.d + dd;
+    } else {
+        dst = reinterpret_cast<__nv_bfloat16*>(e.out) + (size_t)m * e.ldo + col;
+    }
+    if constexpr (FORM == kFormResid) {
+        const uint32_t w[4] = {rr.x, rr.y, rr.z, rr.w};
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const float2 f = unpack_bf16(w[t]);
+            v[2 * t] = fmaf(gate[2 * t], v[2 * t], f.x);
+            v[2 * t + 1] = fmaf(gate[2 * t + 1], v[2 * t + 1], f.y);
+        }
+    }
+    *reinterpret_cast<uint4*>(dst) =
+        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+}
+
+template <int FORM, int S>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+    gemm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                      const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
+                      const __grid_constant__ GemmArgs g) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + SPLIT_STAGES * SPLIT_STAGE_BYTES);
+    uint64_t* empty = full + SPLIT_STAGES;
+    uint64_t* tfull = empty + SPLIT_STAGES;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull + 1);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)cluster_ctarank();
+    const int tile = blockIdx.x / S, tiles0 = g.m_tiles * g.n_tiles;
+    const int prob = tile >= tiles0, r = tile - prob * tiles0;
+    const int m_blk = r / g.n_tiles, n_blk = r % g.n_tiles;
+    const int kb0 = rank * g.k_blocks / S, kb1 = (rank + 1) * g.k_blocks / S;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < SPLIT_STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(tfull, 1);
+        *abort_flag = 0;
+        fence_barrier_init();
+    }
+    if (warp == 1) {
+        tmem_alloc(tmem_slot, SPLIT_BN);
+        tmem_relinquish();
+    }
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    if (warp == 0) {
+        {
+            const CUtensorMap* mA = prob ? &tmA1 : &tmA;
+            const CUtensorMap* mB = prob ? &tmB1 : &tmB;
+            uint32_t armed = 0, parity = 0;        // per stage: a copy was issued; its phase
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.err)) break;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&full[stage], SPLIT_STAGE_BYTES);
+                    uint8_t* sa = smem + stage * SPLIT_STAGE_BYTES;
+                    tma_load_2d(sa, mA, &full[stage], kb * BK, m_blk * BM);
+                    tma_load_2d(sa + A_BYTES, mB, &full[stage], kb * BK, n_blk * SPLIT_BN);
+                }
+                __syncwarp();
+                armed |= 1u << stage;
+                parity = (parity & ~(1u << stage)) | (phase << stage);
+                if (++stage == SPLIT_STAGES) { stage = 0; phase ^= 1u; }
+            }
+            // every issued copy has landed before the ring is reused or the CTA exits
+            for (int s = 0; s < SPLIT_STAGES; ++s) {
+                if (!((armed >> s) & 1)) continue;
+                const unsigned long long t0 = globaltimer();
+                while (!mbar_try_wait(&full[s], (parity >> s) & 1) && globaltimer() - t0 < kWaitLimitNs) {
+                }
+            }
+        }
+    } else if (warp == 1) {
+        {
+            const uint64_t da = sdesc_sw128(smem_u32(smem)), db = sdesc_sw128(smem_u32(smem) + A_BYTES);
+            int stage = 0;
+            uint32_t phase = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!mbar_wait(&full[stage], phase, abort_flag, g.err)) break;
+                tc_fence_after();
+                if (elect_one()) {
+#pragma unroll
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma(tmem_base, sdesc_at(da, stage * SPLIT_STAGE_BYTES + k * 32),
+                               sdesc_at(db, stage * SPLIT_STAGE_BYTES + k * 32), idesc_bf16(BM, SPLIT_BN),
+                               (kb > kb0) || k != 0);
+                    tc_commit(&empty[stage]);
+                }
+                __syncwarp();
+                if (++stage == SPLIT_STAGES) { stage = 0; phase ^= 1u; }
+            }
+            if (elect_one()) tc_commit(tfull);
+            __syncwarp();
+            const unsigned long long t0 = globaltimer();
+            while (!mbar_try_wait(tfull, 0) && globaltimer() - t0 < kWaitLimitNs) {
+            }
+        }
+    }
+    __syncthreads();          // this CTA's copies have landed and its MMAs are done
+    tc_fence_after();
+    const int Mp = prob ? g.M1 : g.M;
+    const Epi e = problem_epilogue(g, prob);
+    // this thread's items: 8-column groups of this CTA's share.  QKV takes one
+    // row (V^T's rows are tokens: consecutive lanes store consecutively), the
+    // other forms one group.
+    constexpr int NG = SPLIT_BN / 8 / S;                      // groups in the share, = items a thread
+    constexpr bool kByRow = FORM == kFormQKV;
+    const int tid = threadIdx.x - 64;
+    const int col_share = n_blk * SPLIT_BN + rank * (SPLIT_BN / S);
+    auto item = [&](int i, int& row, int& grp) {
+        row = kByRow ? tid : i * (BM / NG) + tid / NG;
+        grp = kByRow ? i : tid % NG;
+    };
+    // residual rows, bias and gate are fetched before the barriers
+    uint4 resid[FORM == kFormResid ? NG : 1];
+    if (FORM == kFormResid && warp >= 2) {
+#pragma unroll
+        for (int i = 0; i < NG; ++i) {
+            int row, grp;
+            item(i, row, grp);
+            const int m = m_blk * BM + row, col = col_share + grp * 8;
+            if (m < Mp && col < g.N) resid[i] = residual8(e, m, col);
+        }
+    }
+    float bias[8], gate[8];
+    int col_of;
+    {
+        int row, grp;
+        item(0, row, grp);
+        col_of = min(col_share + grp * 8, g.N - 8);           // (clamped: a share may lie past N)
+    }
+    if (!kByRow && warp >= 2) columns8<FORM>(e, col_of, bias, gate);
+    cluster_sync_all();       // so are the others': every ring is free
+    if (warp >= 2) {
+        const int lg = warp & 3, row = lg * 32 + lane;
+        const uint32_t taddr = tmem_base + ((uint32_t)(lg * 32) << 16);
+        constexpr int C4 = SPLIT_BN / S / 4;                  // 4-column groups in a share
+#pragma unroll
+        for (int c0 = 0; c0 < SPLIT_BN; c0 += 32) {
+            uint32_t v[32];
+            tmem_ld32(taddr + c0, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 32; j += 4) {
+                const int c4 = (c0 + j) / 4;
+                st_shared_cluster_v4(mapa_shared(smem_u32(smem) + split_at<S>(rank, c4 % C4, row), c4 / C4), v[j],
+                                     v[j + 1], v[j + 2], v[j + 3]);
+            }
+        }
+        tc_fence_before();
+    }
+    cluster_sync_all();
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, SPLIT_BN);
+    }
+    if (warp >= 2) {
+#pragma unroll
+        for (int i = 0; i < NG; ++i) {
+            int row, grp;
+            item(i, row, grp);
+            const int m = m_blk * BM + row, col = col_share + grp * 8;
+            float v[8];
+#pragma unroll
+            for (int p = 0; p < S; ++p) {
+                const float4 x = *reinterpret_cast<const float4*>(smem + split_at<S>(p, 2 * grp, row));
+                const float4 y = *reinterpret_cast<const float4*>(smem + split_at<S>(p, 2 * grp + 1, row));
+                if (p == 0) {
+                    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+                    v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+                } else {
+                    v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+                    v[4] += y.x; v[5] += y.y; v[6] += y.z; v[7] += y.w;
+                }
+            }
+            if (kByRow) columns8<FORM>(e, min(col, g.N - 8), bias, gate);
+            if (m < Mp && col < g.N) epilogue8<FORM>(e, m, col, v, bias, gate, resid[FORM == kFormResid ? i : 0]);
+        }
     }
 }
 
@@ -866,13 +1172,20 @@ wdc_status check_operands(Ctx* c, const void* A, const void* W, const Epi& e) {
     return WDC_OK;
 }
 
-using Kernel1 = void (*)(const CUtensorMap, const CUtensorMap, const EpiMaps, const GemmArgs);
-using Kernel2 = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const EpiMaps,
-                         const EpiMaps, const GemmArgs);
-constexpr Kernel1 kKernel1[kForms] = {gemm_tc_kernel<256, 0>, gemm_tc_kernel<256, 1>, gemm_tc_kernel<256, 2>,
-                                      gemm_tc_kernel<256, 3>, gemm_tc_kernel<256, 4>};
-constexpr Kernel2 kKernel2[kForms] = {gemm_tc2_kernel<0>, gemm_tc2_kernel<1>, gemm_tc2_kernel<2>, gemm_tc2_kernel<3>,
-                                      gemm_tc2_kernel<4>};
+using TileKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const EpiMaps,
+                            const EpiMaps, const GemmArgs);
+using SplitKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
+template <int... F>
+struct Tables {
+    static constexpr TileKernel pair[] = {gemm_tc2_kernel<F>...};
+    static constexpr TileKernel one128[] = {gemm_tc_kernel<128, F>...};
+    static constexpr TileKernel one64[] = {gemm_tc_kernel<64, F>...};
+    static constexpr SplitKernel split2[] = {gemm_split_kernel<F, 2>...};
+    static constexpr SplitKernel split4[] = {gemm_split_kernel<F, 4>...};
+    static constexpr SplitKernel split8[] = {gemm_split_kernel<F, 8>...};
+    static SplitKernel split(int S, int f) { return S == 2 ? split2[f] : (S == 4 ? split4[f] : split8[f]); }
+};
+using Kernels = Tables<kFormStore, kFormGelu, kFormResid, kFormQKV, kFormUnpatch>;
 
 int form_of(const Epi& e) {
     switch (e.mode) {
@@ -886,39 +1199,118 @@ int form_of(const Epi& e) {
 void set_attrs() {
     static bool attr_set = false;
     if (!attr_set) {
+        auto smem = [](const void* f, size_t bytes) {
+            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        };
         for (int f = 0; f < kForms; ++f) {
-            cudaFuncSetAttribute(kKernel1[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GemmCfg<256>::SMEM);
-            cudaFuncSetAttribute(kKernel2[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM2_BYTES);
+            smem((const void*)Kernels::pair[f], SMEM2_BYTES);
+            smem((const void*)Kernels::one128[f], GemmCfg<128>::SMEM);
+            smem((const void*)Kernels::one64[f], GemmCfg<64>::SMEM);
+            for (int S = 2; S <= SPLIT_MAX; S *= 2) smem((const void*)Kernels::split(S, f), SPLIT_SMEM);
         }
         attr_set = true;
     }
 }
 
-GemmArgs make_args(Ctx* c, int M, int N, int K, const Epi& e) {
-    GemmArgs g{};
-    g.M = M;
-    g.N = N;
-    g.K = K;
-    g.m_tiles = (M + BM - 1) / BM;
-    g.n_tiles = (N + BN - 1) / BN;
-    g.k_blocks = (K + BK - 1) / BK;
-    // raster groups: a W slab of at most ~40 MB per group (L2 is 126 MB,
-    // shared with the streamed A and the output), as few groups as that
-    // allows.  For deep K (> 4096) a 256-row slab of A is itself large
-    // and re-reading A per group costs more than it saves (measured on the
-    // 17776 x 3072 x 12288 MLP-down GEMM): plain N-fastest order there.
-    g.group_n = g.n_tiles;
-    if (K <= 4096) {
-        const double slab_per_tile = 256.0 * K * 2.0;
-        int gn = (int)(40.0e6 / slab_per_tile);
-        gn = gn < 1 ? 1 : (gn > g.n_tiles ? g.n_tiles : gn);
-        const int groups = (g.n_tiles + gn - 1) / gn;
-        g.group_n = (g.n_tiles + groups - 1) / groups;  // balance the groups
+// One launch: the kernel, its N tile and (split kernel) the CTAs a tile.
+struct Choice {
+    enum Kind { kPair, kOne128, kOne64, kSplit } kind;
+    int split = 1;
+};
+
+// Estimated cycles of a launch with `tiles` tiles on `units` SMs or pairs:
+// `main` cycles of MMAs a tile, `epi` of epilogue behind them.
+double launch_cycles(long long tiles, int units, double main, double epi) {
+    const double waves = (double)((tiles + units - 1) / units);
+    return main + epi + (waves - 1.0) * (main > epi ? main : epi);
+}
+
+// The kernel for a shape is the one with the least estimated cycles; the
+// constants are fits to a sweep (us, store unless said; kb = 64-column blocks):
+//                             pair  one128  one64  split 2 / 4 / 8
+//   272 x 256 x 256 resid      8.8     5.3    4.4    6.1 / 6.5
+//   272 x 256 x 1024 resid    12.1     8.3    7.1    7.4 / 7.2 / 7.4
+//   226 x 3072 x 3072                 15.1   14.2   10.3 / 16.2 / 28.9
+//   64 x 3072 x 8192                  33.7   31.3   17.6 / 12.3 / 18.9
+//   700 x 1024 x 1024 resid   12.2     8.4    7.3    7.6 / 13.8
+//   1600 x 1024 x 4096 resid  25.0    20.1   32.3   23.7 / 28.9
+//   1600 x 3072 x 1024        14.7    15.9   21.9   29.2
+//   6400 x 1024 x 4096 resid  44.6    51.5   90.3   73.8
+// A block of K takes a pair 560 cycles (256 x 256), one CTA 470 (128 x 128) or
+// 450 (128 x 64): a launch of few tiles takes as long in either, so the
+// narrow tile wins where it still fits one wave.  The pair's cluster launch and
+// wider tile cost 1900 more to start; the split kernel's two cluster barriers,
+// exchange and epilogue 4300-6200, and it runs as many clusters at a time as
+// the GPCs hold (76, 36 and 15 of 2, 4 and 8 on this part).
+constexpr double kCyclesPair = 560.0, kCycles128 = 470.0, kCycles64 = 450.0, kCyclesSplit = 440.0, kPairStart = 1900.0;
+
+// Clusters of S split CTAs resident at a time.
+int split_clusters(Ctx* c, int S) {
+    static int cap[SPLIT_MAX + 1] = {};
+    if (cap[S] == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(c->num_sms / S * S, 1, 1);
+        cfg.blockDim = dim3(kGemmThreads, 1, 1);
+        cfg.dynamicSmemBytes = SPLIT_SMEM;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = S;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, Kernels::split(S, 0), &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            n = c->num_sms / S > 0 ? c->num_sms / S : 1;
+        }
+        cap[S] = n;
     }
-    g.e = e;
-    g.err = c->err;
-    g.nprob = 1;
-    return g;
+    return cap[S];
+}
+
+// M, M1: the launch's rows (M1: a second problem's, or 0); sample, sample1:
+// one sample's rows.  Whether and how K is split, which orders the sums,
+// depends on one sample alone; the whole-K kernels sum alike.
+Choice choose_gemm(Ctx* c, int form, int M, int M1, int sample, int sample1, int N, int K) {
+    const int kb = (K + BK - 1) / BK, sms = c->num_sms;
+    const bool plain = form == kFormStore || form == kFormQKV;
+    const double chunk = plain ? 900.0 : 2000.0;              // epilogue of 64 columns
+    auto tiles = [&](int rows, int rows1, int bm, int bn) {
+        return (long long)((rows + bm - 1) / bm + (rows1 + bm - 1) / bm) * ((N + bn - 1) / bn);
+    };
+    auto whole = [&](int rows, int rows1, Choice::Kind* kind) {
+        double best = launch_cycles(tiles(rows, rows1, BM, 64), sms, kb * kCycles64, chunk);
+        *kind = Choice::kOne64;
+        const double one128 = launch_cycles(tiles(rows, rows1, BM, 128), sms, kb * kCycles128, 2 * chunk);
+        if (one128 < best) {
+            best = one128;
+            *kind = Choice::kOne128;
+        }
+        if (rows >= 256 && sms >= 2) {
+            const double pair =
+                kPairStart + launch_cycles(tiles(rows, rows1, 256, BN), sms / 2, kb * kCyclesPair, 4 * chunk);
+            if (pair < best) {
+                best = pair;
+                *kind = Choice::kPair;
+            }
+        }
+        return best;
+    };
+    Choice ch{Choice::kPair};
+    double least = 0.9 * whole(sample, sample1, &ch.kind);    // (a split that gains less is not worth its risk)
+    const long long t = tiles(sample, sample1, BM, SPLIT_BN);
+    for (int S = 2; S <= SPLIT_MAX && 2 * S <= kb; S *= 2) {
+        const int cap = split_clusters(c, S);
+        const double reduce = (S == 8 ? 6200.0 : (S == 4 ? 4550.0 : 4300.0)) + (plain || form == kFormGelu ? 0.0 : 2000.0);
+        const double est = (double)((t + cap - 1) / cap) * (((kb + S - 1) / S) * kCyclesSplit + reduce);
+        if (est < least) {
+            least = est;
+            ch.kind = Choice::kSplit;
+            ch.split = S;
+        }
+    }
+    if (ch.kind != Choice::kSplit) whole(M, M1, &ch.kind);
+    return ch;
 }
 
 // Tensor maps of an epilogue's staged stores and residual loads; 0 when its
@@ -944,35 +1336,108 @@ bool encode_epilogue(const Epi& e, int M, int N, EpiMaps* m, int* staged, std::s
     return true;
 }
 
-// Pair-kernel launch: a persistent grid of as many CTA pairs as can be
-// resident, capped by the tile count.
-wdc_status launch_pair(Ctx* c, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& ta1,
-                       const CUtensorMap& tb1, const EpiMaps& maps, const EpiMaps& maps1, const GemmArgs& g,
-                       cudaStream_t s) {
-    const int tiles = ((g.m_tiles + 1) / 2) * g.n_tiles + (g.nprob > 1 ? g.m_pairs1 * g.n_tiles : 0);
+// A launch's two problems: operands, rows and epilogues (rows1 == 0: one).
+struct Problem {
+    const void *A, *W;
+    int M, sample;
+    const Epi* e;
+};
+
+wdc_status launch_gemm(Ctx* c, const Problem& p0, const Problem* p1, int N, int K, cudaStream_t s) {
+    wdc_status st = check_operands(c, p0.A, p0.W, *p0.e);
+    if (!st && p1) st = check_operands(c, p1->A, p1->W, *p1->e);
+    if (st) return st;
+    set_attrs();
+    const int form = form_of(*p0.e);
+    const Choice ch = choose_gemm(c, form, p0.M, p1 ? p1->M : 0, p0.sample, p1 ? p1->sample : 0, N, K);
+    const int bn = ch.kind == Choice::kPair ? BN : (ch.kind == Choice::kOne64 ? 64 : 128);
+    // W's box: the tile's width, or each CTA's half of it in a pair
+    const uint32_t w_rows = ch.kind == Choice::kPair ? BN / 2 : bn;
+    GemmArgs g{};
+    g.M = p0.M;
+    g.N = N;
+    g.K = K;
+    g.m_tiles = (p0.M + BM - 1) / BM;
+    g.n_tiles = (N + bn - 1) / bn;
+    g.k_blocks = (K + BK - 1) / BK;
+    // raster groups: a W slab of at most ~40 MB per group (L2 is 126 MB,
+    // shared with the streamed A and the output), as few groups as that
+    // allows.  For deep K (> 4096) a 256-row slab of A is itself large
+    // and re-reading A per group costs more than it saves (measured on the
+    // 17776 x 3072 x 12288 MLP-down GEMM): plain N-fastest order there.
+    g.group_n = g.n_tiles;
+    if (K <= 4096) {
+        const double slab_per_tile = 256.0 * K * 2.0;
+        int gn = (int)(40.0e6 / slab_per_tile);
+        gn = gn < 1 ? 1 : (gn > g.n_tiles ? g.n_tiles : gn);
+        const int groups = (g.n_tiles + gn - 1) / gn;
+        g.group_n = (g.n_tiles + groups - 1) / groups;  // balance the groups
+    }
+    g.e = *p0.e;
+    g.err = c->err;
+    g.nprob = p1 ? 2 : 1;
+    std::string why;
+    CUtensorMap ta, tb, ta1, tb1;
+    EpiMaps maps{}, maps1{};
+    auto encode = [&](const Problem& p, CUtensorMap* a, CUtensorMap* b, EpiMaps* m, int* staged) {
+        return encode_tmap_2d(a, p.A, (uint64_t)K, (uint64_t)p.M, (uint64_t)K * 2, BK, BM, &why) &&
+               encode_tmap_2d(b, p.W, (uint64_t)K, (uint64_t)N, (uint64_t)K * 2, BK, w_rows, &why) &&
+               (ch.kind == Choice::kSplit || encode_epilogue(*p.e, p.M, N, m, staged, &why));
+    };
+    if (!encode(p0, &ta, &tb, &maps, &g.staged)) return fail(c, WDC_ERR_CUDA, why);
+    if (p1) {
+        g.M1 = p1->M;
+        g.m_tiles1 = (p1->M + BM - 1) / BM;
+        g.e1 = *p1->e;
+        if (!encode(*p1, &ta1, &tb1, &maps1, &g.staged1)) return fail(c, WDC_ERR_CUDA, why);
+    } else {
+        ta1 = ta;
+        tb1 = tb;
+    }
+    const int tiles128 = (g.m_tiles + g.m_tiles1) * g.n_tiles;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kGemmThreads, 1, 1);
-    cfg.dynamicSmemBytes = SMEM2_BYTES;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    attr[0].val.clusterDim.x = attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    static int max_clusters = 0;
-    if (max_clusters == 0) {
-        cfg.gridDim = dim3(c->num_sms, 1, 1);
-        if (cudaOccupancyMaxActiveClusters(&max_clusters, kKernel2[0], &cfg) != cudaSuccess || max_clusters < 1) {
-            cudaGetLastError();
-            max_clusters = c->num_sms / 2;
+    switch (ch.kind) {
+        case Choice::kPair: {
+            // a persistent grid of as many CTA pairs as can be resident,
+            // capped by the tile count
+            cfg.numAttrs = 1;
+            attr[0].val.clusterDim.x = 2;
+            cfg.dynamicSmemBytes = SMEM2_BYTES;
+            static int max_clusters = 0;
+            if (max_clusters == 0) {
+                cfg.gridDim = dim3(c->num_sms, 1, 1);
+                if (cudaOccupancyMaxActiveClusters(&max_clusters, Kernels::pair[0], &cfg) != cudaSuccess ||
+                    max_clusters < 1) {
+                    cudaGetLastError();
+                    max_clusters = c->num_sms / 2;
+                }
+            }
+            const int tiles = ((g.m_tiles + 1) / 2 + (g.m_tiles1 + 1) / 2) * g.n_tiles;
+            int clusters = max_clusters < c->num_sms / 2 ? max_clusters : c->num_sms / 2;
+            if (tiles < clusters) clusters = tiles;
+            cfg.gridDim = dim3(2 * clusters, 1, 1);
+            cudaLaunchKernelEx(&cfg, Kernels::pair[form], ta, tb, ta1, tb1, maps, maps1, g);
+            break;
         }
+        case Choice::kSplit:
+            cfg.numAttrs = 1;
+            attr[0].val.clusterDim.x = ch.split;
+            cfg.dynamicSmemBytes = SPLIT_SMEM;
+            cfg.gridDim = dim3(tiles128 * ch.split, 1, 1);
+            cudaLaunchKernelEx(&cfg, Kernels::split(ch.split, form), ta, tb, ta1, tb1, g);
+            break;
+        default:
+            cfg.dynamicSmemBytes = bn == 64 ? GemmCfg<64>::SMEM : GemmCfg<128>::SMEM;
+            cfg.gridDim = dim3(tiles128 < c->num_sms ? tiles128 : c->num_sms, 1, 1);
+            cudaLaunchKernelEx(&cfg, bn == 64 ? Kernels::one64[form] : Kernels::one128[form], ta, tb, ta1, tb1, maps,
+                               maps1, g);
     }
-    int clusters = max_clusters < c->num_sms / 2 ? max_clusters : c->num_sms / 2;
-    if (tiles < clusters) clusters = tiles;
-    cfg.gridDim = dim3(2 * clusters, 1, 1);
-    cudaLaunchKernelEx(&cfg, kKernel2[form_of(g.e)], ta, tb, ta1, tb1, maps, maps1, g);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(err));
     return WDC_OK;
@@ -980,61 +1445,20 @@ wdc_status launch_pair(Ctx* c, const CUtensorMap& ta, const CUtensorMap& tb, con
 
 }  // namespace
 
-wdc_status tc_gemm(Ctx* c, const void* A, const void* W, int M, int N, int K, const Epi& e, cudaStream_t s) {
-    wdc_status st = check_operands(c, A, W, e);
-    if (st) return st;
-    set_attrs();
-    const bool pair = M >= 256 && c->num_sms >= 2;
-    CUtensorMap ta, tb;
-    std::string why;
-    if (!encode_tmap_2d(&ta, A, (uint64_t)K, (uint64_t)M, (uint64_t)K * 2, BK, BM, &why) ||
-        !encode_tmap_2d(&tb, W, (uint64_t)K, (uint64_t)N, (uint64_t)K * 2, BK, pair ? BN / 2 : BN, &why))
-        return fail(c, WDC_ERR_CUDA, why);
-    GemmArgs g = make_args(c, M, N, K, e);
-    EpiMaps maps{};
-    if (!encode_epilogue(e, M, N, &maps, &g.staged, &why)) return fail(c, WDC_ERR_CUDA, why);
-    if (pair) return launch_pair(c, ta, tb, ta, tb, maps, maps, g, s);
-    const int tiles = g.m_tiles * g.n_tiles;
-    const int grid = tiles < c->num_sms ? tiles : c->num_sms;
-    kKernel1[form_of(e)]<<<grid, kGemmThreads, GemmCfg<256>::SMEM, s>>>(ta, tb, maps, g);
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(err));
-    return WDC_OK;
+// `sample`: the rows of one sample of a batch (M alone), see choose_gemm.
+wdc_status tc_gemm(Ctx* c, const void* A, const void* W, int M, int N, int K, const Epi& e, int sample, cudaStream_t s) {
+    return launch_gemm(c, Problem{A, W, M, sample, &e}, nullptr, N, K, s);
 }
 
-// Two GEMMs with the same N and K in one launch of the pair kernel (the
-// dual-stream blocks' video rows and condition rows): problem 1's tiles
-// follow problem 0's, filling the pairs problem 0 leaves idle in its last
-// wave.  When problem 0 is too short for the pair kernel the two run as two
-// launches on the stream.
-wdc_status tc_gemm_grouped(Ctx* c, const void* A0, const void* W0, int M0, const Epi& e0, const void* A1,
-                           const void* W1, int M1, const Epi& e1, int N, int K, cudaStream_t s) {
-    if (M1 <= 0) return tc_gemm(c, A0, W0, M0, N, K, e0, s);
-    if (M0 <= 0) return tc_gemm(c, A1, W1, M1, N, K, e1, s);
-    if (M0 < 256 || c->num_sms < 2) {
-        wdc_status st = tc_gemm(c, A0, W0, M0, N, K, e0, s);
-        return st ? st : tc_gemm(c, A1, W1, M1, N, K, e1, s);
-    }
-    wdc_status st = check_operands(c, A0, W0, e0);
-    if (!st) st = check_operands(c, A1, W1, e1);
-    if (st) return st;
-    set_attrs();
-    CUtensorMap ta, tb, ta1, tb1;
-    std::string why;
-    if (!encode_tmap_2d(&ta, A0, (uint64_t)K, (uint64_t)M0, (uint64_t)K * 2, BK, BM, &why) ||
-        !encode_tmap_2d(&tb, W0, (uint64_t)K, (uint64_t)N, (uint64_t)K * 2, BK, BN / 2, &why) ||
-        !encode_tmap_2d(&ta1, A1, (uint64_t)K, (uint64_t)M1, (uint64_t)K * 2, BK, BM, &why) ||
-        !encode_tmap_2d(&tb1, W1, (uint64_t)K, (uint64_t)N, (uint64_t)K * 2, BK, BN / 2, &why))
-        return fail(c, WDC_ERR_CUDA, why);
-    GemmArgs g = make_args(c, M0, N, K, e0);
-    g.nprob = 2;
-    g.M1 = M1;
-    g.m_pairs1 = (M1 + 255) / 256;
-    g.e1 = e1;
-    EpiMaps maps{}, maps1{};
-    if (!encode_epilogue(e0, M0, N, &maps, &g.staged, &why) || !encode_epilogue(e1, M1, N, &maps1, &g.staged1, &why))
-        return fail(c, WDC_ERR_CUDA, why);
-    return launch_pair(c, ta, tb, ta1, tb1, maps, maps1, g, s);
+// Two GEMMs with the same N and K in one launch (the dual-stream blocks' video
+// rows and condition rows): problem 1's tiles follow problem 0's, filling the
+// SMs problem 0 leaves idle in its last wave.
+wdc_status tc_gemm_grouped(Ctx* c, const void* A0, const void* W0, int M0, int sample0, const Epi& e0, const void* A1,
+                           const void* W1, int M1, int sample1, const Epi& e1, int N, int K, cudaStream_t s) {
+    if (M1 <= 0) return tc_gemm(c, A0, W0, M0, N, K, e0, sample0, s);
+    if (M0 <= 0) return tc_gemm(c, A1, W1, M1, N, K, e1, sample1, s);
+    const Problem p1{A1, W1, M1, sample1, &e1};
+    return launch_gemm(c, Problem{A0, W0, M0, sample0, &e0}, &p1, N, K, s);
 }
 
 }  // namespace wdc

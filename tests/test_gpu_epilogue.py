@@ -71,3 +71,55 @@ def test_forward_slabs_across_samples_and_streams(Lc, dual, d):
         assert torch.equal(one[b], many[b])
     want = dit.forward(W, DiTConfig(**cfgd), z[0], 600.0, ct[0])
     assert rel_l2(one[0].cpu().numpy(), want) <= 2e-2
+
+
+@pytest.mark.parametrize("M,N,K", [(226, 3072, 3072), (64, 1056, 8192), (128, 512, 12288), (1, 9216, 3072), (257, 160, 4104),
+                                   (130, 32, 2056), (700, 1024, 1024), (1600, 1024, 2048)])
+@pytest.mark.parametrize("mode", ["store", "gelu", "resid"])
+def test_gemm_few_tiles(M, N, K, mode):
+    """Shapes of the narrow-tile and split-K kernels (2, 4 and 8 CTAs a tile,
+    shares past N, K blocks that do not divide evenly), bound as above."""
+    ctx = wdc.Context(wdc.make_config(dtype=wdc.BF16, **MODEL), 2)
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    r = lambda *s: torch.randn(*s, device="cuda", generator=g)
+    A, W, b = r(M, K).bfloat16(), (r(N, K) * K ** -0.5).bfloat16(), r(N)
+    want, kw = A.double() @ W.double().T + b.double(), {}
+    buf = torch.full((M + 40, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    if mode == "gelu":
+        kw["gelu"] = True
+        want = 0.5 * want * (1 + torch.tanh((2 / np.pi) ** 0.5 * (want + 0.044715 * want ** 3)))
+    elif mode == "resid":
+        R, gate = r(M, N).bfloat16(), r(N)
+        want = R.double() + gate.double() * want
+        kw.update(res=R, gate=gate)
+    ctx.op_gemm(A, W, buf[:M], bias=b, **kw)
+    torch.cuda.synchronize()
+    assert ctx.device_errors() == 0
+    assert float((buf[:M].double() - want).norm() / want.norm()) <= 2.0 ** -8 + K * 2.0 ** -22
+    assert bool((buf[M:] == 7.0).all())
+
+
+@pytest.mark.parametrize("Lc,dual,d", [(5, 0, 64), (5, 1, 128), (140, 1, 64)])
+def test_forward_split_k(Lc, dual, d):
+    """A wide model on few tokens (every GEMM of its block splits K) against the
+    oracle, and a batch of three bitwise equal to its samples' own forwards."""
+    cfgd = dict(MODEL, hidden=2048, heads=2048 // d, head_dim=d, mlp=4096, frames=1, height=8, width=10, cond_tokens=Lc,
+                cond_dim=2048, dual_stream=dual)
+    W = synth.dit_weights(cfgd, 9, std=0.02, bias_std=0.05, bf16=True)
+    ctx = wdc.Context(wdc.make_config(dtype=wdc.BF16, max_batch=3, **cfgd), 2)
+    ctx.set_weights(W)
+    z = [synth.latent(20 + b, (16, 1, 8, 10)) for b in range(3)]
+    ct = [synth.cond_tokens(30 + b, Lc, 2048) for b in range(3)]
+    zd, cd = [_dev(a.reshape(-1)) for a in z], [_dev(a) for a in ct]
+    one = []
+    for b in range(3):
+        one.append(torch.empty_like(zd[b]))
+        ctx.dit_forward(zd[b], 600.0, cd[b], one[b])
+    many = [torch.empty_like(t) for t in zd]
+    ctx.dit_forward_batch(zd, 600.0, cd, many)
+    torch.cuda.synchronize()
+    assert ctx.device_errors() == 0
+    for b in range(3):
+        assert torch.equal(one[b], many[b])
+    want = dit.forward(W, DiTConfig(**cfgd), z[0], 600.0, ct[0])
+    assert rel_l2(one[0].cpu().numpy(), want) <= 2e-2
