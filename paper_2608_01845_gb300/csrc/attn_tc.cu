@@ -8,7 +8,7 @@
 //   warpgroup 0 (control, registers lowered to 40 per thread)
 //     warp 0    TMA producer: the two 128-row Q tiles once, then K / V^T
 //               tiles of BK keys into a shared-memory ring (128-byte swizzle);
-//     warps 1, 2 MMA issuers, one thread per query tile t:
+//     warps 1, 2 MMA issuers, one warp per query tile t:
 //               S(t) = Q(t) K^T into TMEM (BK fp32 columns) and
 //               O(t) += P(t) V into TMEM;
 //   warpgroups 1, 2 (softmax of query tile 0, 1; registers raised to 232)
@@ -37,6 +37,17 @@
 //     S(t, j), PV(t, j-1)
 // and the MMA of S(t, j+1) overlaps the softmax of step j instead of
 // waiting behind PV(t, j).
+// What bounds a step (128 keys at d = 64, about 1850 cycles): the two tiles'
+// MMAs take about 1540 back to back (an S product is fed from shared memory at
+// 128 bytes a clock, 340 instead of 256), the softmax's two warps on an SM
+// sub-partition 1230 (the exponentials alone 1050).  A warp alone forms its 64
+// numerator pairs in 700 cycles, both at once take 1130, and then neither has
+// any while both wait for S, store P and hand over; so tile 1's first product
+// waits for tile 0's first P (`stagger`) and the two warps stay about half a
+// step apart (3.08 -> 2.88 ms at 48 heads x 17776).  Producer and issuers run
+// with all lanes and issue from an elected one (3.17 -> 3.08 ms; 1.49 -> 1.36
+// at 24 x 13568 x 128).  Tiles half a step apart hold a stage of K and V
+// longer: five stages instead of three, 227 -> 203 us at 48 x 4276 x 64.
 // Grid: one CTA per (head, 256-query) unit, one CTA per SM.  The units of a
 // sample's last, partial round are split over the key range instead: each
 // part runs the same pipeline over its steps and writes its unnormalised O,
@@ -69,7 +80,7 @@ struct AttnCfg {
     static constexpr uint32_t K_TILE = BK * D * 2;
     static constexpr uint32_t V_TILE = D * BK * 2;
     static constexpr uint32_t STAGE = K_TILE + V_TILE;      // 32 KB for both head sizes
-    static constexpr int STAGES = D == 64 ? 3 : 5;
+    static constexpr int STAGES = 5;
     static constexpr uint32_t SMEM = 2 * Q_TILE + STAGES * STAGE + 1024 + 256;
     static constexpr uint32_t TMEM_COLS = 512;
     static constexpr uint32_t REGS_CONTROL = 40;
@@ -169,7 +180,8 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
     uint64_t* p_full = s_free + 2;                            // [2]
     uint64_t* p_free = p_full + 2;                            // [2]
     uint64_t* o_final = p_free + 2;                           // [2]
-    uint64_t* mma_done = o_final + 2;
+    uint64_t* stagger = o_final + 2;                          // tile 0 has stored its first P
+    uint64_t* mma_done = stagger + 1;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -204,6 +216,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
             mbar_init(&p_free[w], 1);
             mbar_init(&o_final[w], 1);
         }
+        mbar_init(stagger, 4);
         mbar_init(mma_done, C::ISSUERS);
         *abort_flag = 0;
         fence_barrier_init();
@@ -225,26 +238,29 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
     if (wg == 0) {
       setmaxnreg_dec<C::REGS_CONTROL>();
       if (warp == 0) {
-        if (lane == 0) {
             // Q: two tiles x ATOMS boxes of [128 rows x 64 d]
-            mbar_arrive_expect_tx(q_full, 2 * C::Q_TILE);
-            for (int t = 0; t < 2; ++t)
-                for (int a = 0; a < C::ATOMS; ++a)
-                    tma_load_3d(sq + t * C::Q_TILE + a * (BQ * 128), &tq, q_full, 64 * a, q0 + t * BQ, h);
+            if (elect_one()) {
+                mbar_arrive_expect_tx(q_full, 2 * C::Q_TILE);
+                for (int t = 0; t < 2; ++t)
+                    for (int a = 0; a < C::ATOMS; ++a)
+                        tma_load_3d(sq + t * C::Q_TILE + a * (BQ * 128), &tq, q_full, 64 * a, q0 + t * BQ, h);
+            }
+            __syncwarp();
             int stage = 0;
             uint32_t phase = 0;
-            bool armed[C::STAGES];
-            uint32_t armed_phase[C::STAGES];
-            for (int s = 0; s < C::STAGES; ++s) armed[s] = false;
+            uint32_t armed = 0, parity = 0;        // per stage: a copy was issued; its phase
             for (int j = j0; j < j0 + nj; ++j) {
                 if (!mbar_wait(&kv_empty[stage], phase ^ 1u, abort_flag, g.err)) break;
-                mbar_arrive_expect_tx(&kv_full[stage], C::STAGE);
-                uint8_t* sk = skv + stage * C::STAGE;
-                uint8_t* sv = sk + C::K_TILE;
-                for (int a = 0; a < C::ATOMS; ++a) tma_load_3d(sk + a * (BKV * 128), &tk, &kv_full[stage], 64 * a, j * BKV, h);
-                for (int a = 0; a < BKV / 64; ++a) tma_load_3d(sv + a * (D * 128), &tv, &kv_full[stage], j * BKV + 64 * a, 0, h);
-                armed[stage] = true;
-                armed_phase[stage] = phase;
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&kv_full[stage], C::STAGE);
+                    uint8_t* sk = skv + stage * C::STAGE;
+                    uint8_t* sv = sk + C::K_TILE;
+                    for (int a = 0; a < C::ATOMS; ++a) tma_load_3d(sk + a * (BKV * 128), &tk, &kv_full[stage], 64 * a, j * BKV, h);
+                    for (int a = 0; a < BKV / 64; ++a) tma_load_3d(sv + a * (D * 128), &tv, &kv_full[stage], j * BKV + 64 * a, 0, h);
+                }
+                __syncwarp();
+                armed |= 1u << stage;
+                parity = (parity & ~(1u << stage)) | (phase << stage);
                 if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
             }
             {
@@ -253,75 +269,86 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
                 }
             }
             for (int s = 0; s < C::STAGES; ++s) {
-                if (!armed[s]) continue;
+                if (!((armed >> s) & 1)) continue;
                 const unsigned long long t0 = globaltimer();
-                while (!mbar_try_wait(&kv_full[s], armed_phase[s]) && globaltimer() - t0 < kWaitLimitNs) {
+                while (!mbar_try_wait(&kv_full[s], (parity >> s) & 1) && globaltimer() - t0 < kWaitLimitNs) {
                 }
             }
-        }
       } else if (warp == 1 || warp == 2) {
-        if (lane == 0) {
             constexpr uint32_t idesc_s = idesc_bf16(BQ, BKV);
             constexpr uint32_t idesc_o = idesc_f16(BQ, D);       // P (fp16, TMEM) x V (fp16, shared memory)
-            const uint32_t sq0 = smem_u32(sq);
+            // this warp issues the MMAs of query tile t only; the other tile
+            // has its own issuer, so neither waits behind the other's softmax
+            const int t = warp - 1;
+            const uint64_t dq = sdesc_sw128(smem_u32(sq) + t * C::Q_TILE);
+            const uint64_t dk = sdesc_sw128(smem_u32(skv)), dv = sdesc_sw128(smem_u32(skv) + C::K_TILE);
             bool ok = mbar_wait(q_full, 0, abort_flag, g.err);
             int stage = 0, prev = 0;
             uint32_t phase = 0;
             // S(t) = Q(t) K^T into TMEM (BK fp32 columns)
-            auto issue_s = [&](int t, int st) {
-                const uint32_t kb = smem_u32(skv + st * C::STAGE);
-                const uint32_t qb = sq0 + t * C::Q_TILE;
+            auto issue_s = [&](int st) {
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
                     const uint32_t off = (ks >> 2) * (BQ * 128) + (ks & 3) * 32;
                     const uint32_t koff = (ks >> 2) * (BKV * 128) + (ks & 3) * 32;
-                    tc_mma(tmem + C::s_col(t), sdesc_sw128(qb + off), sdesc_sw128(kb + koff), idesc_s, ks != 0);
+                    tc_mma(tmem + C::s_col(t), sdesc_at(dq, off), sdesc_at(dk, st * C::STAGE + koff), idesc_s, ks != 0);
                 }
             };
             // O(t) (+)= P(t) V, A = P in TMEM (16 bf16 = 8 columns per K step)
-            auto issue_pv = [&](int t, int st, bool acc) {
-                const uint32_t vb = smem_u32(skv + st * C::STAGE + C::K_TILE);
+            auto issue_pv = [&](int st, bool acc) {
 #pragma unroll
                 for (int ks = 0; ks < BKV / 16; ++ks) {
                     const uint32_t voff = (ks >> 2) * (D * 128) + (ks & 3) * 32;
-                    tc_mma_ts(tmem + C::o_col(t), tmem + C::p_col(t) + ks * 8, sdesc_sw128(vb + voff), idesc_o,
+                    tc_mma_ts(tmem + C::o_col(t), tmem + C::p_col(t) + ks * 8, sdesc_at(dv, st * C::STAGE + voff), idesc_o,
                               (acc || ks != 0) ? 1u : 0u);
                 }
             };
-            // this thread issues the MMAs of query tile t only; the other
-            // tile has its own issuer, so neither waits behind the other's
-            // softmax
-            const int t = warp - 1;
+            if (ok && t == 1) ok = mbar_wait(stagger, 0, abort_flag, g.err);
+            if (ok) ok = mbar_wait(&kv_full[0], 0, abort_flag, g.err);
             for (int j = 0; j < nj && ok; ++j) {
-                if (!mbar_wait(&kv_full[stage], phase, abort_flag, g.err)) { ok = false; break; }
+                // here K(j) has landed, and S(t, j - 1) is in the softmax's registers
                 tc_fence_after();
-                if (j > 0) {
-                    if (!mbar_wait(&s_free[t], (j - 1) & 1, abort_flag, g.err)) { ok = false; break; }
-                    tc_fence_after();
+                if (elect_one()) {
+                    issue_s(stage);
+                    tc_commit(&s_full[t]);
                 }
-                issue_s(t, stage);
-                tc_commit(&s_full[t]);
+                __syncwarp();
+                const int cur = stage;
+                if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+                // the next step's K: awaited before P(t, j - 1) at d = 128
+                // (1.34 -> 1.31 ms at 24 x 13568), after it at d = 64, where
+                // waiting first keeps the two tiles' steps in phase (2.89 ->
+                // 2.95 ms at 48 x 17776)
+                auto next_k = [&]() { return j + 1 >= nj || mbar_wait(&kv_full[stage], phase, abort_flag, g.err); };
+                if (D == 128 && !next_k()) { ok = false; break; }
                 if (j > 0) {
                     if (!mbar_wait(&p_full[t], (j - 1) & 1, abort_flag, g.err)) { ok = false; break; }
                     tc_fence_after();
-                    issue_pv(t, prev, j > 1);
-                    tc_commit(&p_free[t]);
-                    tc_commit(&kv_empty[prev]);
+                    if (elect_one()) {
+                        issue_pv(prev, j > 1);
+                        tc_commit(&p_free[t]);
+                        tc_commit(&kv_empty[prev]);
+                    }
+                    __syncwarp();
                 }
-                prev = stage;
-                if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+                prev = cur;
+                if (D == 64 && !next_k()) { ok = false; break; }
+                if (j + 1 < nj && !mbar_wait(&s_free[t], j & 1, abort_flag, g.err)) { ok = false; break; }
             }
             if (ok && mbar_wait(&p_full[t], (nj - 1) & 1, abort_flag, g.err)) {
                 tc_fence_after();
-                issue_pv(t, prev, nj > 1);
-                tc_commit(&kv_empty[prev]);
-                tc_commit(&o_final[t]);
+                if (elect_one()) {
+                    issue_pv(prev, nj > 1);
+                    tc_commit(&kv_empty[prev]);
+                    tc_commit(&o_final[t]);
+                }
+                __syncwarp();
             }
-            tc_commit(mma_done);
+            if (elect_one()) tc_commit(mma_done);
+            __syncwarp();
             const unsigned long long t0 = globaltimer();
             while (!mbar_try_wait(mma_done, 0) && globaltimer() - t0 < kWaitLimitNs) {
             }
-        }
       }
     } else {
         setmaxnreg_inc<C::REGS_SOFTMAX>();
@@ -337,9 +364,9 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
         const int mask_step = (j0 + nj == n_kv && last_valid < BKV) ? nj - 1 : -1;   // this CTA's ragged step
         float m_run = -INFINITY, l_run = 0.f;
         const uint64_t scale2 = pair(g.scale_log2, g.scale_log2);
-        bool ok = true;
+        bool ok = true, s_ready = false;
         for (int j = 0; j < nj; ++j) {                  // j counts this CTA's steps
-            if (!mbar_wait(&s_full[t], j & 1, abort_flag, g.err)) { ok = false; break; }
+            if (!s_ready && !mbar_wait(&s_full[t], j & 1, abort_flag, g.err)) { ok = false; break; }
             tc_fence_after();
             float s[BKV];
 #pragma unroll
@@ -378,6 +405,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
             };
             float base = (j == 0) ? tile_max() * g.scale_log2 : m_run;
             float sum;
+            bool moved = false;                         // some row of the warp moved its base
             // A numerator above 2^8 implies a row sum above 2^8 (so does a
             // non-finite one): only then take the tile max, move the base and
             // recompute, as a second pass of the same code.
@@ -386,9 +414,9 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
                 sum = numerators(base);
                 const bool redo = pass == 0 && !(sum <= 256.0f);
                 if (!__any_sync(0xffffffffu, redo)) break;
+                moved = true;
                 if (redo) base = fmaxf(base, tile_max() * g.scale_log2);
             }
-            const bool moved = base != m_run;
             const float corr = ex2(m_run - base);     // 1 when the base stays; 0 before the first tile
             l_run = l_run * corr + sum;
             m_run = base;
@@ -397,7 +425,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
                 if (!mbar_wait(&p_free[t], (j - 1) & 1, abort_flag, g.err)) { ok = false; break; }
                 tc_fence_after();
             }
-            if (j > 0 && __any_sync(0xffffffffu, moved)) {
+            if (j > 0 && moved) {
                 // PV(t, j-1) is complete: rescale O in place
 #pragma unroll
                 for (int c = 0; c < D; c += 32) {
@@ -417,10 +445,16 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
             // P (BK / 2 columns of fp16 pairs)
 #pragma unroll
             for (int c = 0; c < BKV / 2; c += 16) tmem_st16(p_addr + c, *reinterpret_cast<uint32_t(*)[16]>(&p[c]));
+            // d = 64: a look at S(t, j + 1) while the store completes (2.99 -> 2.94 ms)
+            const bool next = D == 64 && mbar_test(&s_full[t], (j + 1) & 1);
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&p_full[t]);
+            if (lane == 0) {
+                mbar_arrive(&p_full[t]);
+                if (j == 0 && t == 0) mbar_arrive(stagger);
+            }
+            if (D == 64) s_ready = __all_sync(0xffffffffu, next);
         }
         if (ok && is_part && mbar_wait(&o_final[t], 0, abort_flag, g.err)) {
             // a part of a split unit: unnormalised O with its base and row
