@@ -158,7 +158,7 @@ const float* anchor_ptr(const Ctx* c) { return c->n_bank > 0 ? c->bank[newest_sl
 PassArgs base_args(Ctx* c, int k) {
     PassArgs a;
     std::memset(&a, 0, sizeof(a));
-    a.n = (long long)c->n;
+    set_numel(a, c->n);
     a.k = k;
     a.T = c->sched.T;
     a.age = c->age;
@@ -178,7 +178,7 @@ void set_cond(PassArgs& a, const wdc_cond* cd) {
     }
 }
 
-// Skip pass + async copy of the step record into `dst` (pinned); no sync.
+// Skip pass; its last CTA writes the step record into `dst` (pinned).  No sync.
 bool needs_disp(const Ctx* c) { return c->prm.flags & (WDC_ABL_SECANT | WDC_OBS_RESIDUAL); }
 
 // z_cur (the current latent) is read only by the secant and the residual reading.
@@ -204,10 +204,8 @@ wdc_status enqueue_skip(Ctx* c, int k, const wdc_cond* cd, const float* z_cur, f
     }
     a.anchor = anchor_ptr(c);
     a.out = z_hat;
-    wdc_status st = launch_pass(c, mode, a, s);
-    if (st) return st;
-    WDC_CUDA_TRY(c, cudaMemcpyAsync(dst, &c->st->out, sizeof(StepOut), cudaMemcpyDeviceToHost, s));
-    return WDC_OK;
+    a.host_out = dst;
+    return launch_pass(c, mode, a, s);
 }
 
 wdc_status enqueue_anchor(Ctx* c, int k, const wdc_cond* cd, const float* z_t, const float* v, const float* z_cf,
@@ -223,9 +221,9 @@ wdc_status enqueue_anchor(Ctx* c, int k, const wdc_cond* cd, const float* z_t, c
     a.out = c->bank[ins];
     a.out2 = needs_disp(c) ? c->disp[ins] : nullptr;
     a.ins_slot = ins;
+    a.host_out = dst;                  // d_cf, R, eta and r of it
     wdc_status st = launch_pass(c, kModeAnchor, a, s);
     if (st) return st;
-    if (dst) WDC_CUDA_TRY(c, cudaMemcpyAsync(dst, &c->st->out, sizeof(StepOut), cudaMemcpyDeviceToHost, s));
     if (c->n_bank < K) c->n_bank++;
     else c->head = (c->head + 1) % K;
     c->age = 0;

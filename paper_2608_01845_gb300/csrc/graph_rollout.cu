@@ -329,7 +329,7 @@ wdc_status graph_rollout(Ctx* c, const float* z_T, bool z_dev, const wdc_cond* c
     // this rollout's constants (parameters and descriptors may change between rollouts)
     PlanArgs p;
     std::memset(&p, 0, sizeof(p));
-    p.tmpl.n = (long long)c->n;
+    set_numel(p.tmpl, c->n);
     p.tmpl.T = T;
     p.tmpl.prm = to_dev_params(c->prm);
     p.tmpl.st = c->st;

@@ -57,8 +57,6 @@ __device__ __forceinline__ float signed_term(uint32_t idx, uint32_t seed, float 
     return __int_as_float(__float_as_int(x) ^ (int)h);
 }
 
-// Butterfly sum over the 32 lanes (a fixed-order tree: every lane ends with
-// the same value).
 // Bulk prefetch of `bytes` (a multiple of 16, 16-byte aligned) into L2.
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -66,6 +64,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
 // Runs per warp whose bank reads are prefetched while warp 0 forms the head.
 constexpr int kPrefetchRuns = 4;
 
+// Butterfly sum over the 32 lanes (a fixed-order tree: every lane ends with
+// the same value).
 __device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -121,36 +121,37 @@ __device__ __forceinline__ void reduce256d(double (&v)[NV], double* scratch, dou
     __syncthreads();
 }
 
-// The part of the device state a pass reads, copied into shared memory by all
-// threads at the start in one batch of independent loads; the head and the
-// tails then work from shared memory.  (Read in place, the head and the
-// controller tail were chains of dependent L2 round trips -- the state may sit
-// in the other die's half of L2 -- that cost about 10 us per launch.)
-struct alignas(16) StateIn {
-    float cur_S[kSketch], anchor_S[kSketch];
-    float s_phi[kSummary];                 // anchor pass: the pre-insertion summary
-    float n_in[kMaxBank], n_out[kMaxBank]; // records by age (oldest first)
-    float q_in[kMaxBank], dq[kMaxBank], r[kMaxBank];
-    float cur_sumsq, cur_sumsq_anchor, anchor_sumsq, R, eta, q_a_out, q_a_dq, cand_p;
-    float cam_a[4], depth_a[4];
-    int cand_k, cand_supported, cand_finite;
+// The vectors and scalars of the device state a pass reads, copied into shared
+// memory by all threads at the start in one batch of independent loads, beside
+// the launch arguments; the head and the tails then work from shared memory.
+// (Read in place, the head and the controller tail were chains of dependent L2
+// round trips -- the state may sit in the other die's half of L2 -- that cost
+// about 10 us per launch.)
+constexpr int kMisc = kSummary - 2 * kSketch;      // a summary's last entries: cam, depth, phase, history
+struct alignas(16) StateIn : DevScalars {
+    alignas(16) float cur_S[kSketch];
+    alignas(16) float anchor_S[kSketch];
+    alignas(16) float s_phi[kSummary];     // anchor pass: the pre-insertion summary
+    float misc[kMisc];                     // skip passes: s(phi_k)'s last entries
+    float dist2[2], norm2[2];              // camera, depth: squared distance to the anchor's descriptors, squared norm
+    float n_in[kMaxBank], n_out[kMaxBank], q_in[kMaxBank];   // records by age (oldest first)
 };
-// The records' summaries by age; shares storage with the stream's bucket
-// rows, which are used only after the head.
+// The records' summaries by age (linear observation only); shares storage with
+// the stream's bucket rows, which that variant zeroes after its head.
 struct alignas(16) RecSummaries {
     float s_in[kMaxBank][kSummary], s_out[kMaxBank][kSummary], s_dphi[kMaxBank][kSummary];
 };
 
 struct HeadShared {
-    float phi[kSummary];
-    float hat[kSummary];
+    alignas(16) float phi[kSummary];
+    alignas(16) float hat[kSummary];
     float scratch[8 * (kMaxBank + 1)];
     float red[kMaxBank + 1];
+    float dot_in[kMaxBank + 1], dot_out[kMaxBank + 1];   // phi . s_in_i and |phi|^2; s_hat . s_out_i and |s_hat|^2
     double dscratch[8 * kMaxBank];          // linear observation: fp64 reduction scratch
     double gram[kMaxBank + 1][kMaxBank];    // linear observation: the records' Gram matrix, then S_out s_hat
-    float sim_in[kMaxBank], sim_out[kMaxBank], pi[kMaxBank], kappa[kMaxBank];
+    float pi[kMaxBank], kappa[kMaxBank];
     float alpha;
-    int compat[kMaxBank];
     int n_compat, supported;
 };
 
@@ -221,147 +222,168 @@ __device__ __noinline__ void linear_readout(const PassArgs& a, const RecSummarie
     }
 }
 
-// Skip-pass head, Eq. 2-5 scalar part, in fp32, run by one warp of every CTA
-// (so no CTA waits for another): lane l owns the summary entries l, l+32, ...,
-// every dot product is a lane-local sum followed by a butterfly, and every
-// lane then holds the totals, so each lane evaluates the small softmaxes of
-// Eq. 3 and 5 itself and no block barrier is needed.  (Spread over 256
-// threads with block reductions, the same head took ~9k cycles, most of it in
-// barriers.)  The head and the controller tails are one chain of dependent
-// scalar steps per launch, so they use the fast division and exponential
-// intrinsics (a few ulp; the tolerances are 1e-5).  Writes hs.phi, hs.hat,
-// hs.alpha and, for K > 0, hs.sim_in/sim_out/compat/pi/kappa/n_compat/
-// supported; the caller synchronises the block afterwards.
+// Skip-pass head, Eq. 2-5 scalar part, in fp32, run by the first 9 warps of
+// every CTA (so no CTA waits for another).  Thread t < 256 owns summary entry
+// t; warp i <= K takes the dot product with record i (warp K: the norm), 8
+// entries a lane and a butterfly.  The records' rows are in registers since the
+// kernel's start (HeadRegs).  Lane i of a warp evaluates record i's terms of the
+// softmaxes of Eq. 3 and 5.
+// Code that a launch runs once, like the head and the tails, costs about 11
+// cycles an instruction, whatever it computes (clock stamps: its instructions
+// come from L2): spread over threads but with the records' terms unrolled the
+// head took as long, 8k cycles, as in one warp.  So it is written for few
+// instructions: one record a lane, entries prepared where they are loaded,
+// fast division and exponential (a few ulp; the tolerances are 1e-5).  The
+// softmaxes magnify rounding by 1 / temperature, so their sums and the dot
+// products keep one fixed order.  8.0k -> 3.4k cycles; a pass at 1.12M elements
+// and 4 records 20.7 -> 17.4 us between events, of which an empty launch is 5.
+constexpr int kHeadThreads = (kMaxBank + 1) * 32;
+
+// What a thread of the head holds of the records: its lane's entries l, l + 32,
+// ... of its warp's record's lifted input and output, and entry t of every
+// increment.
+constexpr int kLaneEntries = kSummary / 32;
 template <int K>
-__device__ void skip_head_warp(const PassArgs& a, const StateIn& S, const RecSummaries& rs, HeadShared& hs) {
-    constexpr int J = kSummary / 32;                  // entries per lane
-    const int lane = threadIdx.x & 31;
-    const float N = (float)a.n;
-    const float sc = sqrtf(__fdividef((float)kSketch, N));
-    const float eps_nu = a.prm.eps_nu;
-    const bool no_cond = a.prm.flags & WDC_ABL_NO_COND;
-    const float inv_cur = __fdividef(sc, sqrtf(__fdividef(S.cur_sumsq, N)) + eps_nu);
-    const float inv_dz = __fdividef(sc, sqrtf(__fdividef(S.cur_sumsq_anchor, N)) + eps_nu);
-    // s(phi_k): current-state summary (Eq. 2 through the linear sketch)
-    float ph[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const int t = lane + 32 * j;
-        float val;
-        if (t < kSketch) {
-            val = S.cur_S[t] * inv_cur;
-        } else if (t < 2 * kSketch) {
-            const int b = t - kSketch;
-            val = (S.cur_S[b] - S.anchor_S[b]) * inv_dz;
-        } else if (t < kOffDepth) {
-            val = no_cond ? 0.f : a.cam[t - kOffCam];
-        } else if (t < kOffQ) {
-            val = no_cond ? 0.f : a.depth[t - kOffDepth];
-        } else if (t == kOffQ) {
-            val = a.sk.q_k;
-        } else {
-            // h(H): [r_1..3, T*(q_in - q_out)_1..3, n_bank/K], newest record first
-            const int h = t - kOffH;
-            val = 0.f;
-            if (h < 3) {
-                if (h < a.nsrc) val = S.r[a.nsrc - 1 - h];
-            } else if (h < 6) {
-                if (h - 3 < a.nsrc) val = -(float)a.T * S.dq[a.nsrc - 1 - (h - 3)];
-            } else {
-                val = __fdividef((float)a.nsrc, (float)a.prm.K);
-            }
-        }
-        ph[j] = val;
-        hs.phi[t] = val;
-    }
-    // Eq. 4: alpha = clip(|q_{t-1}-q_t| / (|q_{a-1}-q_a| + eps), alpha_min, alpha_max)
-    const float alpha =
-        fminf(fmaxf(__fdividef(fabsf(a.sk.dq), fabsf(S.q_a_dq) + a.prm.eps), a.prm.alpha_min), a.prm.alpha_max);
-    if (lane == 0) hs.alpha = alpha;
+struct HeadRegs {
+    float in[kLaneEntries], out[kLaneEntries];
+    float dphi[K > 0 ? K : 1];
+};
+
+template <int K>
+__device__ __forceinline__ void load_head(const PassArgs& a, HeadRegs<K>& r) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if constexpr (K > 0) {
-        // Eq. 3: similarities with the records' lifted inputs
-        float d[K + 1];
+        if (warp < K) {
+            const DevRecord& R = a.st->rec[a.slot[warp]];
 #pragma unroll
-        for (int i = 0; i <= K; ++i) d[i] = 0.f;
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const int t = lane + 32 * j;
-#pragma unroll
-            for (int i = 0; i < K; ++i) d[i] = fmaf(ph[j], rs.s_in[i][t], d[i]);
-            d[K] = fmaf(ph[j], ph[j], d[K]);
-        }
-#pragma unroll
-        for (int i = 0; i <= K; ++i) d[i] = warp_sum_f(d[i]);
-        const float nphi = sqrtf(d[K]);
-        const bool filter = !(a.prm.flags & WDC_ABL_NO_SUPPORT);   // w/o support: N_t = whole bank
-        const float gq = a.prm.gamma_q, inv_tin = __fdividef(1.0f, a.prm.tau_in);
-        int nc = 0;
-        float mx = -INFINITY, ell[K], pi[K], sim[K];
-        bool compat[K];
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            sim[i] = (nphi == 0.f || S.n_in[i] == 0.f) ? 0.f : __fdividef(d[i], nphi * S.n_in[i]);
-            const float dq = a.sk.q_k - S.q_in[i];
-            compat[i] = !filter || ((sim[i] >= a.prm.sim_min) && (fabsf(dq) <= a.prm.q_gap_max));
-            ell[i] = (sim[i] - gq * dq * dq) * inv_tin;
-            if (compat[i]) { ++nc; mx = fmaxf(mx, ell[i]); }
-        }
-        float tot = 0.f;
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            pi[i] = compat[i] ? __expf(ell[i] - mx) : 0.f;
-            tot += pi[i];
-        }
-        const float inv_tot = nc > 0 ? __fdividef(1.0f, tot) : 0.f;
-#pragma unroll
-        for (int i = 0; i < K; ++i) pi[i] *= inv_tot;
-        // Eq. 4 in summary space, then Eq. 5 similarities with the lifted outputs
-        float e[K + 1];
-#pragma unroll
-        for (int i = 0; i <= K; ++i) e[i] = 0.f;
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-            const int t = lane + 32 * j;
-            float acc = 0.f;
-#pragma unroll
-            for (int i = 0; i < K; ++i)
-                if (pi[i] != 0.f) acc = fmaf(pi[i], rs.s_dphi[i][t], acc);
-            const float hv = fmaf(alpha, acc, ph[j]);
-            hs.hat[t] = hv;
-#pragma unroll
-            for (int i = 0; i < K; ++i) e[i] = fmaf(hv, rs.s_out[i][t], e[i]);
-            e[K] = fmaf(hv, hv, e[K]);
-        }
-#pragma unroll
-        for (int i = 0; i <= K; ++i) e[i] = warp_sum_f(e[i]);
-        const float nh = sqrtf(e[K]);
-        const float inv_tau = __fdividef(1.0f, a.prm.tau_obs);
-        float so[K];
-        float mo = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-            so[i] = (nh == 0.f || S.n_out[i] == 0.f) ? 0.f : __fdividef(e[i], nh * S.n_out[i]);
-            e[i] = so[i] * inv_tau;
-            mo = fmaxf(mo, e[i]);
-        }
-        float to = 0.f;
-#pragma unroll
-        for (int i = 0; i < K; ++i) { e[i] = __expf(e[i] - mo); to += e[i]; }
-        const float inv = __fdividef(1.0f, to);
-        if (lane == 0) {
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                hs.sim_in[i] = sim[i];
-                hs.compat[i] = compat[i];
-                hs.pi[i] = pi[i];
-                hs.sim_out[i] = so[i];
-                hs.kappa[i] = e[i] * inv;
+            for (int j = 0; j < kLaneEntries; ++j) {
+                r.in[j] = __ldcg(&R.s_in[lane + 32 * j]);
+                r.out[j] = __ldcg(&R.s_out[lane + 32 * j]);
             }
-            hs.n_compat = nc;
-            hs.supported = filter ? (nc >= a.prm.min_support) : 1;
+        }
+        if (t < kSummary) {
+#pragma unroll
+            for (int i = 0; i < K; ++i) r.dphi[i] = __ldcg(&a.st->rec[a.slot[i]].s_dphi[t]);
         }
     }
 }
+
+__device__ __forceinline__ void head_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kHeadThreads) : "memory"); }
+
+// Dot product of the summary x with the warp's row (or with itself), the same
+// in every lane.
+__device__ __forceinline__ float summary_dot(const float* x, const float (&row)[kLaneEntries], bool self) {
+    float s = 0.f;
+#pragma unroll
+    for (int j = 0; j < kLaneEntries; ++j) {
+        const float v = x[(threadIdx.x & 31) + 32 * j];
+        s = fmaf(v, self ? v : row[j], s);
+    }
+    return warp_sum_f(s);
+}
+// Maximum over lanes 8 g .. 8 g + 7, and the sum over lanes 0 .. K - 1 in order.
+__device__ __forceinline__ float max8(float v) {
+#pragma unroll
+    for (int o = 4; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+template <int K>
+__device__ __forceinline__ float sum_records(float v) {
+    float s = 0.f;
+#pragma unroll
+    for (int r = 0; r < K; ++r) s += __shfl_sync(0xffffffffu, v, r);
+    return s;
+}
+// Similarity of a record with its dot product and norm; 0 where a norm is.
+__device__ __forceinline__ float similarity(float dot, float n_rec, float n_self) {
+    return n_self == 0.f || n_rec == 0.f ? 0.f : __fdividef(dot, n_self * n_rec);
+}
+
+// Fills hs.phi, hs.alpha and, for K > 0, hs.hat, hs.pi, hs.n_compat,
+// hs.supported and hs.dot_out; the caller synchronises the block afterwards.
+template <int K>
+__device__ __forceinline__ void skip_head(const PassArgs& a, const StateIn& S, const HeadRegs<K>& rg, HeadShared& hs) {
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    // Eq. 4: alpha = clip(|q_{t-1}-q_t| / (|q_{a-1}-q_a| + eps), alpha_min, alpha_max)
+    const float alpha =
+        fminf(fmaxf(__fdividef(fabsf(a.sk.dq), fabsf(S.q_a_dq) + a.prm.eps), a.prm.alpha_min), a.prm.alpha_max);
+    float ph = 0.f;
+    if (t < kSummary) {
+        // s(phi_k): current-state summary (Eq. 2 through the linear sketch)
+        const bool dz = t >= kSketch;
+        const int b = dz ? min(t - kSketch, kSketch - 1) : t;
+        float x = S.cur_S[b];
+        if (dz) x -= S.anchor_S[b];
+        const float sc = sqrtf(__fdividef((float)kSketch, a.n_f));
+        ph = x * __fdividef(sc, sqrtf(__fdividef(dz ? S.cur_sumsq_anchor : S.cur_sumsq, a.n_f)) + a.prm.eps_nu);
+        if (t >= 2 * kSketch) ph = S.misc[t - 2 * kSketch];
+        hs.phi[t] = ph;
+        if (t == 0) hs.alpha = alpha;
+    }
+    if constexpr (K > 0) {
+        const int i = lane & 7;              // this lane's record
+        const bool in = i < K;
+        head_sync();
+        if (warp <= K) {
+            // Eq. 3: similarities with the records' lifted inputs
+            const float d = summary_dot(hs.phi, rg.in, warp == K);
+            if (lane == 0) hs.dot_in[warp] = d;
+        }
+        head_sync();
+        if (t < kSummary) {
+            const bool filter = !(a.prm.flags & WDC_ABL_NO_SUPPORT);   // w/o support: N_t = whole bank
+            const float gq = a.prm.gamma_q, inv_tin = __fdividef(1.0f, a.prm.tau_in);
+            const float sim = similarity(hs.dot_in[i], S.n_in[i], sqrtf(hs.dot_in[K]));
+            const float dq = a.sk.q_k - S.q_in[i];
+            const bool compat = in && (!filter || (sim >= a.prm.sim_min && fabsf(dq) <= a.prm.q_gap_max));
+            const float ell = compat ? (sim - gq * dq * dq) * inv_tin : -INFINITY;
+            const int nc = __popc(__ballot_sync(0xffffffffu, compat) & 0xff);
+            const float top = max8(ell);
+            const float e = compat ? __expf(ell - top) : 0.f;
+            const float tot = sum_records<K>(e);
+            const float pi = nc > 0 ? e * __fdividef(1.0f, tot) : 0.f;
+            // Eq. 4 in summary space
+            float acc = 0.f;
+#pragma unroll
+            for (int r = 0; r < K; ++r) {
+                const float w = __shfl_sync(0xffffffffu, pi, r);
+                if (w != 0.f) acc = fmaf(w, rg.dphi[r], acc);
+            }
+            hs.hat[t] = fmaf(alpha, acc, ph);
+            if (t < K) hs.pi[t] = pi;
+            if (t == 0) {
+                hs.n_compat = nc;
+                hs.supported = filter ? (nc >= a.prm.min_support) : 1;
+            }
+        }
+        head_sync();
+        if (warp <= K) {
+            // Eq. 5 similarities with the lifted outputs
+            const float d = summary_dot(hs.hat, rg.out, warp == K);
+            if (lane == 0) hs.dot_out[warp] = d;
+        }
+    }
+}
+
+// Eq. 5: the observation weights (a softmax over every record), by each warp
+// after the block's barrier.
+template <int K>
+__device__ __forceinline__ void observation_weights(const PassArgs& a, const StateIn& S, const HeadShared& hs,
+                                                    float (&kap)[K]) {
+    const int i = threadIdx.x & 7;
+    const float inv_tau = __fdividef(1.0f, a.prm.tau_obs);
+    const float x = i < K ? similarity(hs.dot_out[i], S.n_out[i], sqrtf(hs.dot_out[K])) * inv_tau : -INFINITY;
+    const float e = __expf(x - max8(x));
+    const float w = e * __fdividef(1.0f, sum_records<K>(e));
+#pragma unroll
+    for (int r = 0; r < K; ++r) kap[r] = __shfl_sync(0xffffffffu, w, r);
+}
+
+constexpr int kScalarWords = sizeof(DevScalars) / 4;
+static_assert(sizeof(DevScalars) % 4 == 0 && kScalarWords <= 32, "one warp copies the scalars");
+static_assert(kMisc == 16 && kOffQ - kOffCam == 8 && kOffH - kOffCam == 9, "layout of a summary's last entries");
+constexpr int kStepOutWords = sizeof(StepOut) / 4;
+static_assert(sizeof(StepOut) % 4 == 0 && kStepOutWords <= 128, "the step record is copied word by word");
 
 // Per-block scalar slots: the stream's five sums and the non-finite count.
 constexpr int kScalars = 6;
@@ -376,21 +398,18 @@ struct alignas(16) PassShared {
     };
     float blk[kWarps][kScalars];
     float fin[kPartials];
-    StateIn S;
+    alignas(16) StateIn S;
     int last;
 };
 
 static_assert(alignof(PassShared) >= 16 && alignof(StateIn) >= 16 && alignof(RecSummaries) >= 16,
               "float4 snapshot stores need 16-byte aligned shared arrays");
-static_assert(offsetof(PassShared, S) % 16 == 0 && offsetof(PassShared, rs) == 0, "snapshot offsets");
 static_assert(sizeof(PassArgs) % 8 == 0 && alignof(PassArgs) <= 16, "the argument copy moves whole words");
-static_assert(offsetof(StateIn, cur_S) % 16 == 0 && offsetof(StateIn, anchor_S) % 16 == 0 &&
-              offsetof(StateIn, s_phi) % 16 == 0, "snapshot vector offsets");
 static_assert((kSummary * sizeof(float)) % 16 == 0, "summary rows stay 16-byte aligned");
 static_assert(offsetof(DevRecord, s_in) % 16 == 0 && offsetof(DevRecord, s_out) % 16 == 0 &&
               offsetof(DevRecord, s_dphi) % 16 == 0 && sizeof(DevRecord) % 16 == 0, "record layout");
-static_assert(offsetof(DevState, rec) % 16 == 0 && offsetof(DevState, cur_S) % 16 == 0 &&
-              offsetof(DevState, anchor_S) % 16 == 0 && offsetof(DevState, s_phi) % 16 == 0, "state layout");
+// (DevState's and StateIn's vectors are declared alignas(16))
+static_assert(alignof(DevState) >= 16, "state layout");
 
 // Copies what this mode reads of the device state into shared memory (one
 // batch of independent loads spread over the block's threads).
@@ -400,7 +419,7 @@ __device__ __forceinline__ void load_state(const PassArgs& a, PassShared& ps) {
     const int t = threadIdx.x;
     StateIn& S = ps.S;
     const bool head = MODE == kModeSkip || MODE == kModeResidual || MODE == kModeSecant;
-    if (MODE == kModeSkip || MODE == kModeResidual) {
+    if ((MODE == kModeSkip || MODE == kModeResidual) && (a.prm.flags & WDC_ABL_LINEAR_OBS)) {
         // summaries of the nsrc records by age: 3 arrays x 64 float4 each
         for (int idx = t; idx < a.nsrc * 192; idx += kThreads) {
             const int i = idx / 192, rem = idx - i * 192, which = rem >> 6, c = rem & 63;
@@ -411,37 +430,67 @@ __device__ __forceinline__ void load_state(const PassArgs& a, PassShared& ps) {
         }
     }
     if (head || MODE == kModeAnchor) {
-        const int u = t - 384;                   // threads 384.. take the vectors and scalars
-        if (u >= 0 && u < 30) reinterpret_cast<float4*>(S.cur_S)[u] = __ldcg(reinterpret_cast<const float4*>(st->cur_S) + u);
-        else if (u >= 32 && u < 62)
-            reinterpret_cast<float4*>(S.anchor_S)[u - 32] = __ldcg(reinterpret_cast<const float4*>(st->anchor_S) + (u - 32));
-        else if (MODE == kModeAnchor && u >= 64 && u < 128)
-            reinterpret_cast<float4*>(S.s_phi)[u - 64] = __ldcg(reinterpret_cast<const float4*>(st->s_phi) + (u - 64));
-        else if (u >= 128 && u < 128 + kMaxBank) {
-            const int i = u - 128;
-            if (i < a.nsrc) {
-                const DevRecord& R = st->rec[a.slot[i]];
-                S.n_in[i] = __ldcg(&R.n_in);
-                S.n_out[i] = __ldcg(&R.n_out);
-                S.q_in[i] = __ldcg(&R.q_in);
-                S.dq[i] = __ldcg(&R.dq);
-                S.r[i] = __ldcg(&R.r);
-            }
-        } else if (u >= 160 && u < 168) {
-            const int j = u - 160;
-            if (j < 4) S.cam_a[j] = __ldcg(&st->cam_a[j]);
-            else S.depth_a[j - 4] = __ldcg(&st->depth_a[j - 4]);
-        } else if (u == 168) S.cur_sumsq = __ldcg(&st->cur_sumsq);
-        else if (u == 169) S.cur_sumsq_anchor = __ldcg(&st->cur_sumsq_anchor);
-        else if (u == 170) S.anchor_sumsq = __ldcg(&st->anchor_sumsq);
-        else if (u == 171) S.R = __ldcg(&st->R);
-        else if (u == 172) S.eta = __ldcg(&st->eta);
-        else if (u == 173) S.q_a_dq = __ldcg(&st->q_a_dq);
-        else if (u == 174) S.q_a_out = __ldcg(&st->q_a_out);
-        else if (u == 175) S.cand_p = __ldcg(&st->cand_p);
-        else if (u == 176) S.cand_k = __ldcg(&st->cand_k);
-        else if (u == 177) S.cand_supported = __ldcg(&st->cand_supported);
-        else if (u == 178) S.cand_finite = __ldcg(&st->cand_finite);
+        // warps past the head's, one array each
+        const int lane = t & 31;
+        auto copy4 = [&](float* dst, const float* src, int i) {
+            reinterpret_cast<float4*>(dst)[i] = __ldcg(reinterpret_cast<const float4*>(src) + i);
+        };
+        switch (t >> 5) {
+            case 12: if (lane < kSketch / 4) copy4(S.cur_S, st->cur_S, lane); break;
+            case 13: if (lane < kSketch / 4) copy4(S.anchor_S, st->anchor_S, lane); break;
+            case 14:
+                if (lane < kScalarWords)
+                    reinterpret_cast<uint32_t*>(static_cast<DevScalars*>(&S))[lane] =
+                        __ldcg(reinterpret_cast<const uint32_t*>(static_cast<const DevScalars*>(st)) + lane);
+                break;
+            case 15:
+                if (head && lane < a.nsrc) {
+                    const DevRecord& R = st->rec[a.slot[lane]];
+                    S.n_in[lane] = __ldcg(&R.n_in);
+                    S.n_out[lane] = __ldcg(&R.n_out);
+                    S.q_in[lane] = __ldcg(&R.q_in);
+                }
+                break;
+            case 16:
+                if (head && lane < kMisc) {
+                    // camera, depth, phase, then h(H): [r_1..3, T*(q_in - q_out)_1..3,
+                    // n_bank/K], newest record first
+                    const int h = lane - 9, rec = h < 3 ? h : h - 3;
+                    float x = 0.f;
+                    if (lane < 8) {
+                        if (!(a.prm.flags & WDC_ABL_NO_COND)) x = lane < 4 ? a.cam[lane] : a.depth[lane - 4];
+                    } else if (lane == 8) {
+                        x = a.sk.q_k;
+                    } else if (h == 6) {
+                        x = __fdividef((float)a.nsrc, (float)a.prm.K);
+                    } else if (rec < a.nsrc) {
+                        const DevRecord& R = st->rec[a.slot[a.nsrc - 1 - rec]];
+                        x = h < 3 ? __ldcg(&R.r) : -(float)a.T * __ldcg(&R.dq);
+                    }
+                    S.misc[lane] = x;
+                }
+                break;
+            case 19:
+                // lane 0: camera, lane 1: depth
+                if (head && lane < 2) {
+                    const float* c = lane ? a.depth : a.cam;
+                    const float* ca = lane ? st->depth_a : st->cam_a;
+                    float d = 0.f, u = 0.f;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float x = c[j], y = x - __ldcg(ca + j);
+                        d = fmaf(y, y, d);
+                        u = fmaf(x, x, u);
+                    }
+                    S.dist2[lane] = d;
+                    S.norm2[lane] = u;
+                }
+                break;
+            case 17: case 18:
+                if (MODE == kModeAnchor) copy4(S.s_phi, st->s_phi, t - 17 * 32);
+                break;
+            default: break;
+        }
     }
 }
 
@@ -468,8 +517,19 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
     // launch, measured).
     __shared__ __align__(16) uint32_t s_args[(sizeof(PassArgs) + 3) / 4];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    for (int i = t; i < (int)((sizeof(PassArgs) + 3) / 4); i += kThreads)
+    // copied from the far end of the block, whose threads have the least to do here
+    for (int i = kThreads - 1 - t; i < (int)((sizeof(PassArgs) + 3) / 4); i += kThreads)
         s_args[i] = reinterpret_cast<const uint32_t*>(&a_in)[i];
+    constexpr bool kHead = MODE == kModeSkip || MODE == kModeResidual;
+    HeadRegs<kHead ? K : 0> regs;
+    if constexpr (kHead) load_head<K>(a_in, regs);
+    load_state<MODE>(a_in, ps);
+    const bool linear = kHead && K > 0 && (a_in.prm.flags & WDC_ABL_LINEAR_OBS);
+    constexpr int kSketches = MODE == kModeStats ? 2 : 1;    // reduced by this mode
+    auto zero_rows = [&]() {
+        for (int i = t; i < kSketches * kWarps * kSketch; i += kThreads) (&ps.wb[0][0][0])[i] = 0.f;
+    };
+    if (!linear) zero_rows();        // (the linear observation's summaries share their storage)
     __syncthreads();
     const PassArgs& a = *reinterpret_cast<const PassArgs*>(s_args);
     const uint32_t seed = a.prm.seed;
@@ -477,17 +537,14 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
     const long long nruns = (n + kRun - 1) / kRun;
     const long long full = n / kRun;
 
-    load_state<MODE>(a, ps);
-    __syncthreads();
-
     bool do_stream = true;
     float kap[K > 0 ? K : 1];
     float alpha_f = 0.f;
     if constexpr ((MODE == kModeSkip || MODE == kModeResidual || MODE == kModeObserve) && K > 0) {
-        // while warp 0 forms the head, the other warps start the HBM reads of
+        // while the first warps form the head, the others start the HBM reads of
         // their first runs (into L2): lane i < K takes bank record i, lane K
         // the anchor (observe / residual) or the current latent (residual)
-        if (warp != 0 && lane <= K) {
+        if ((MODE == kModeObserve ? warp != 0 : t >= kHeadThreads) && lane <= K) {
             const float* src = lane < K ? a.src[lane] : (MODE == kModeSkip ? nullptr : a.anchor);
             const long long gw = (long long)blockIdx.x * kWarps + warp;
             const long long stride = (long long)gridDim.x * kWarps;
@@ -500,15 +557,26 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
             }
         }
     }
-    if (MODE == kModeSkip || MODE == kModeResidual) {
-        if (warp == 0) skip_head_warp<K>(a, ps.S, ps.rs, hs);
+    if constexpr (kHead) {
+        if (t < kHeadThreads) skip_head<K>(a, ps.S, regs, hs);
         __syncthreads();
-        if (a.prm.flags & WDC_ABL_LINEAR_OBS) linear_readout<K>(a, ps.rs, hs);
-        do_stream = (K > 0) && hs.supported;
+        if constexpr (K > 0) {
+            observation_weights<K>(a, ps.S, hs, kap);
+            if (linear) {
+                linear_readout<K>(a, ps.rs, hs);
 #pragma unroll
-        for (int i = 0; i < K; ++i) kap[i] = hs.kappa[i];
+                for (int i = 0; i < K; ++i) kap[i] = hs.kappa[i];
+                __syncthreads();
+                zero_rows();
+                __syncthreads();
+            } else if (t == 0) {
+#pragma unroll
+                for (int i = 0; i < K; ++i) hs.kappa[i] = kap[i];    // for the tail
+            }
+        }
+        do_stream = (K > 0) && hs.supported;
     } else if (MODE == kModeSecant) {
-        if (warp == 0) skip_head_warp<0>(a, ps.S, ps.rs, hs);   // lift summary and alpha only: no retrieval
+        if (t < kHeadThreads) skip_head<0>(a, ps.S, HeadRegs<0>{}, hs);   // lift summary and alpha only: no retrieval
         __syncthreads();
         do_stream = a.nsrc > 0;
         alpha_f = hs.alpha;
@@ -516,9 +584,6 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
 #pragma unroll
         for (int i = 0; i < K; ++i) kap[i] = a.kappa[i];
     }
-    // the bucket rows share storage with the record summaries the head read
-    for (int i = t; i < 2 * kWarps * kSketch; i += kThreads) (&ps.wb[0][0][0])[i] = 0.f;
-    __syncthreads();
 
     // per-thread accumulators: plain fp32 over up to 16 runs (64 terms), then
     // a compensated fp32 outer sum
@@ -785,11 +850,11 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
     }
     __syncthreads();
     // partials are value-major, [kPartials][gridDim.x], so the last block
-    // reads each value's per-block entries with coalesced loads
+    // reads each value's per-block entries with coalesced loads; a block alone
+    // has its totals at once
     const int G = gridDim.x;
-    float* part = a.partials + blockIdx.x;
-    const int nsk = (MODE == kModeStats) ? 2 : 1;       // sketches reduced by this mode
-    if (t < nsk * kSketch) {
+    float* part = G == 1 ? ps.fin : a.partials + blockIdx.x;
+    if (t < kSketches * kSketch) {
         part[(size_t)t * G] = sum_warp_rows(ps.wb[t / kSketch], t % kSketch);
     } else if (warp == kWarps - 1) {
         // the last warp: one lane per warp row, a butterfly per scalar
@@ -799,22 +864,27 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
             if (lane == 0) part[(size_t)(2 * kSketch + j) * G] = v;
         }
     }
-    __threadfence();
     __syncthreads();
-    if (t == 0) {
-        const unsigned prev = atomicAdd(a.counter, 1u);
-        ps.last = (prev == gridDim.x - 1);
+    if (G > 1) {
+        // the barrier orders the block's partial sums before this thread's
+        // fence, and the fence before its count (and, for the last block, the
+        // others' counts before its reads)
+        if (t == 0) {
+            __threadfence();
+            const unsigned prev = atomicAdd(a.counter, 1u);
+            ps.last = (prev == gridDim.x - 1);
+            __threadfence();
+        }
+        __syncthreads();
+        if (!ps.last) return;
     }
-    __syncthreads();
-    if (!ps.last) return;
-    __threadfence();
 
     // final reduction over the blocks, fixed order: each warp takes values
     // w, w + 32, ...; lane l sums blocks l, l + 32, ... (G <= kMaxPassBlocks),
     // then a butterfly.  All of a warp's loads for four values are issued
     // before any is added (one L2 round trip per four values).
-    {
-        const int nv = nsk * kSketch;             // sketch values, then the scalars at 2 * kSketch
+    if (G > 1) {
+        const int nv = kSketches * kSketch;       // sketch values, then the scalars at 2 * kSketch
         const int total = nv + kScalars;
         for (int v0 = warp; v0 < total; v0 += 4 * kWarps) {
             float x[4][kMaxPassBlocks / 32];
@@ -841,7 +911,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
         }
         __syncthreads();
     }
-    if (t == 0) *a.counter = 0u;
+    if (G > 1 && t == 0) *a.counter = 0u;
 
     if (MODE == kModeObserve) {
         // raw signed bucket sums of z_hat, sum z_hat^2, sum (z_hat - z_a)^2, non-finite count
@@ -855,7 +925,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
     }
 
     DevState* st = a.st;
-    const float N = (float)n;
+    const float N = a.n_f;
     const float* fin = ps.fin;
     const int sc0 = 2 * kSketch;   // scalar sums start here
 
@@ -878,6 +948,12 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
         const int supported = (MODE == kModeSecant) ? (a.nsrc > 0) : ((K > 0) && hs.supported);
         const int finite = supported && (fin[sc0 + 5] == 0.f);
         __shared__ int s_dec;
+        __shared__ StepOut s_out;
+        if (t >= 32 && t < 32 + kMaxBank) {
+            const int i = t - 32;
+            s_out.kappa[i] = i < K ? hs.kappa[i] : 0.f;
+            s_out.pi[i] = i < K ? hs.pi[i] : 0.f;
+        }
         if (t == 0) {
             // controller tail in fp32; the stored risk R stays fp64
             const ParamsDev& p = a.prm;
@@ -886,21 +962,12 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
             const float d_z = __fdividef(sqrtf(__fdividef(S.cur_sumsq_anchor, N)), sqrtf(__fdividef(S.anchor_sumsq, N)) + eps);
             const float d_age = (float)a.age;
             const float d_phase = fabsf(a.sk.q_next - S.q_a_out);
-            float dc = 0.f, dd = 0.f, uc = 0.f, ud = 0.f;
-            for (int j = 0; j < 4; ++j) {
-                const float cj = a.cam[j], dj = a.depth[j];
-                const float ca = S.cam_a[j], da = S.depth_a[j];
-                dc = fmaf(cj - ca, cj - ca, dc);
-                dd = fmaf(dj - da, dj - da, dd);
-                uc = fmaf(cj, cj, uc);
-                ud = fmaf(dj, dj, ud);
-            }
-            const float pt = p.w_z * d_z + p.w_age * d_age + p.w_phase * d_phase + p.w_cam * sqrtf(dc) +
-                             p.w_depth * sqrtf(dd);
+            const float pt = p.w_z * d_z + p.w_age * d_age + p.w_phase * d_phase + p.w_cam * sqrtf(S.dist2[0]) +
+                             p.w_depth * sqrtf(S.dist2[1]);
             const float d_hat = S.eta * pt;
             const float w = (p.flags & WDC_ABL_NO_IMPACT)
                                 ? 1.f
-                                : fminf(2.f, 1.f + p.a_cam * sqrtf(uc) + p.a_depth * sqrtf(ud) + p.a_phase * a.sk.q_k);
+                                : fminf(2.f, 1.f + p.a_cam * sqrtf(S.norm2[0]) + p.a_depth * sqrtf(S.norm2[1]) + p.a_phase * a.sk.q_k);
             const float delta = w * d_hat;
             const float R_cand = fmaf(p.lam, S.R, delta);
             const bool avail = (a.nsrc > 0) && (a.age <= p.max_age) &&
@@ -909,7 +976,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
             // Eq. 10, or periodic placement (ablation): at most period - 1 surrogate steps in a row
             const bool accept = (p.flags & WDC_ABL_PERIODIC) ? (a.age + 1 < p.period) : (R_cand <= p.tau_risk);
             const int dec = (avail && accept) ? 1 : 0;
-            StepOut& o = st->out;
+            StepOut& o = s_out;
             o.decision = dec;
             o.finite = finite;
             o.supported = supported;
@@ -924,10 +991,6 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
             o.d_cf = __int_as_float(0x7fc00000);   // NaN: no exact step yet
             o.d_z = d_z;
             o.r = 0.f;
-            for (int i = 0; i < kMaxBank; ++i) {
-                o.kappa[i] = (i < K) ? hs.kappa[i] : 0.f;
-                o.pi[i] = (i < K) ? hs.pi[i] : 0.f;
-            }
             const float R_new = dec ? R_cand : S.R;
             if (dec) st->R = R_cand;
             if (a.graph) {
@@ -946,6 +1009,14 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
             s_dec = dec;
         }
         __syncthreads();
+        // the step record, to the state and (host-driven steps) to the host's
+        // pinned copy, which the end of the launch makes visible: no copy
+        // of its own behind the launch
+        if (t >= 128 && t < 128 + kStepOutWords) {
+            const uint32_t w = reinterpret_cast<const uint32_t*>(&s_out)[t - 128];
+            reinterpret_cast<uint32_t*>(&st->out)[t - 128] = w;
+            if (a.host_out) reinterpret_cast<uint32_t*>(a.host_out)[t - 128] = w;
+        }
         if (t < kSketch) {
             st->cand_S[t] = fin[t];
             if (s_dec) st->cur_S[t] = fin[t];
@@ -979,8 +1050,14 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
         st->out.d_cf = d_cf;
         st->out.R = R;
         st->out.eta = eta;
+        if (a.host_out) {            // an exact step's part of the record
+            a.host_out->d_cf = d_cf;
+            a.host_out->R = R;
+            a.host_out->eta = eta;
+        }
         const float r = __fdividef(sqrtf(__fdividef(fin[sc0 + 4], N)), sqrtf(__fdividef(S.cur_sumsq, N)) + eps);
         st->out.r = r;
+        if (a.host_out) a.host_out->r = r;
         st->rec[a.ins_slot].r = r;
         s_rms[0] = sqrtf(__fdividef(fin[sc0 + 2], N));
         s_rms[1] = sqrtf(__fdividef(fin[sc0 + 3], N));
@@ -1161,14 +1238,17 @@ wdc_status launch_pair_stats(Ctx* c, const float* a, const float* b, const float
     return WDC_OK;
 }
 
-int pass_grid(const Ctx* c) {
-    const long long nruns = ((long long)c->n + kRun - 1) / kRun;
+// Blocks of a pass over n elements: a warp a run, up to one block an SM.
+int pass_blocks(long long n, int num_sms, int most) {
+    const long long nruns = (n + kRun - 1) / kRun;
     long long g = (nruns + kWarps - 1) / kWarps;
-    if (g > c->num_sms) g = c->num_sms;
-    if (g > kMaxPassBlocks) g = kMaxPassBlocks;
+    if (g > num_sms) g = num_sms;
+    if (g > most) g = most;
     if (g < 1) g = 1;
     return (int)g;
 }
+
+int pass_grid(const Ctx* c) { return pass_blocks((long long)c->n, c->num_sms, kMaxPassBlocks); }
 
 // Pointer-argument launch (graph capture); K selects the bank-size
 // specialisation of the skip / residual passes.
@@ -1232,6 +1312,11 @@ wdc_status launch_pass(Ctx* c, int mode, const PassArgs& a, cudaStream_t s) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("latent pass launch: ") + cudaGetErrorString(e));
     return WDC_OK;
+}
+
+void set_numel(PassArgs& a, size_t n) {
+    a.n = (long long)n;
+    a.n_f = (float)n;
 }
 
 ParamsDev to_dev_params(const wdc_cache_params& p) {
@@ -1344,7 +1429,7 @@ extern "C" wdc_status wdc_observe_noalloc(const float* const* z_out, int K, cons
     }
     PassArgs a;
     std::memset(&a, 0, sizeof(a));
-    a.n = (long long)n;
+    set_numel(a, n);
     a.nsrc = K;
     for (int i = 0; i < K; ++i) {
         a.src[i] = z_out[i];
@@ -1356,23 +1441,19 @@ extern "C" wdc_status wdc_observe_noalloc(const float* const* z_out, int K, cons
     a.partials = reinterpret_cast<float*>(d.scratch);
     a.counter = reinterpret_cast<unsigned*>(d.scratch + kNoAllocPartialBytes);
     a.stats_out = stats;
-    const long long nruns = ((long long)n + kRun - 1) / kRun;
-    long long grid = (nruns + kWarps - 1) / kWarps;
-    if (grid > d.num_sms) grid = d.num_sms;
-    if (grid > kNoAllocMaxBlocks) grid = kNoAllocMaxBlocks;
-    if (grid < 1) grid = 1;
+    const int grid = pass_blocks((long long)n, d.num_sms, kNoAllocMaxBlocks);
     cudaStream_t s = (cudaStream_t)stream;
     // the last-CTA counter must start at zero (a failed earlier call may have left it set)
     if (cudaMemsetAsync(a.counter, 0, sizeof(unsigned), s) != cudaSuccess) { cudaGetLastError(); return WDC_ERR_CUDA; }
     switch (K) {
-        case 1: launch_observe<1>(a, (int)grid, s); break;
-        case 2: launch_observe<2>(a, (int)grid, s); break;
-        case 3: launch_observe<3>(a, (int)grid, s); break;
-        case 4: launch_observe<4>(a, (int)grid, s); break;
-        case 5: launch_observe<5>(a, (int)grid, s); break;
-        case 6: launch_observe<6>(a, (int)grid, s); break;
-        case 7: launch_observe<7>(a, (int)grid, s); break;
-        default: launch_observe<8>(a, (int)grid, s); break;
+        case 1: launch_observe<1>(a, grid, s); break;
+        case 2: launch_observe<2>(a, grid, s); break;
+        case 3: launch_observe<3>(a, grid, s); break;
+        case 4: launch_observe<4>(a, grid, s); break;
+        case 5: launch_observe<5>(a, grid, s); break;
+        case 6: launch_observe<6>(a, grid, s); break;
+        case 7: launch_observe<7>(a, grid, s); break;
+        default: launch_observe<8>(a, grid, s); break;
     }
     if (cudaGetLastError() != cudaSuccess) return WDC_ERR_CUDA;
     return WDC_OK;

@@ -57,20 +57,24 @@ struct StepScalars {
     float t_model;                // 1000 sigma_k
 };
 
-// Continuous controller/memory state (discrete state -- bank ring, age -- is
-// owned by the host and passed per launch).
-struct DevState {
+// Scalars of the state, in one block so that a pass copies them at once.
+struct DevScalars {
     float R, eta;
     float q_a_in, q_a_out, q_a_dq;  // latest exact interval and its length
     float cam_a[4], depth_a[4];
-    DevRecord rec[kMaxBank];                       // indexed by ring slot
-    alignas(16) float cur_S[kSketch];              // raw signed bucket sums over the current latent
-    float cur_sumsq, cur_sumsq_anchor;             // sum z^2, sum (z - z_a)^2
-    alignas(16) float anchor_S[kSketch];
+    float cur_sumsq, cur_sumsq_anchor;             // sum z^2, sum (z - z_a)^2 of the current latent
     float anchor_sumsq;
-    alignas(16) float s_phi[kSummary];             // summary of the current state (this step)
     int cand_k, cand_supported, cand_finite;
     float cand_p;
+};
+
+// Continuous controller/memory state (discrete state -- bank ring, age -- is
+// owned by the host and passed per launch).
+struct DevState : DevScalars {
+    DevRecord rec[kMaxBank];                       // indexed by ring slot
+    alignas(16) float cur_S[kSketch];              // raw signed bucket sums over the current latent
+    alignas(16) float anchor_S[kSketch];
+    alignas(16) float s_phi[kSummary];             // summary of the current state (this step)
     alignas(16) float cand_S[kSketch];
     float cand_sumsq, cand_sumsq_anchor;
     StepOut out;
@@ -95,6 +99,7 @@ enum StreamMode { kModeStats = 0, kModeSkip = 1, kModeAnchor = 2, kModeObserve =
 // Launch arguments of the fused latent-pass kernels (passed by value).
 struct PassArgs {
     long long n;
+    float n_f;                         // n in fp32
     int nsrc;                          // skip: records in age order (oldest first)
     const float* src[kMaxBank];        // skip: bank latents by age; anchor/stats: src[0] = z_k;
                                        // secant: src[0] = z_k, src[1] = z_a - z_a,in;
@@ -114,6 +119,7 @@ struct PassArgs {
     float* partials;                   // [kPartials][gridDim.x] (value-major)
     unsigned* counter;
     unsigned* err;
+    StepOut* host_out;                 // the step record's pinned host copy, or nullptr
     float kappa[kMaxBank];             // observe: caller-given weights
     double* stats_out;                 // observe: caller-given statistics output
     // graph rollout (device-side control flow)
@@ -213,6 +219,7 @@ int pass_grid(const Ctx* c);
 wdc_status launch_pass(Ctx* c, int mode, const PassArgs& a, cudaStream_t s);
 wdc_status launch_pass_ptr(Ctx* c, int mode, int K, const PassArgs* pa, cudaStream_t s);
 ParamsDev to_dev_params(const wdc_cache_params& p);
+void set_numel(PassArgs& a, size_t n);         // n and n_f
 // wdc_latent_pair_stats: five sums over three latents into out_dev (device, 5 doubles)
 wdc_status launch_pair_stats(Ctx* c, const float* a, const float* b, const float* cz, double* out_dev,
                              cudaStream_t s);
