@@ -326,8 +326,107 @@ __global__ void normal_init_kernel(T* __restrict__ dst, long long n, unsigned lo
 }
 
 // ---------------------------------------------------------------- SIMT GEMM
-// C = epilogue(A W^T), A [M, K], W [N, K]; 64x64 tiles, 4x4 per thread,
-// sequential-k fp32 accumulation.
+// C = epilogue(A W^T), A [M, K], W [N, K], fp32, each element one chain of
+// fused multiply-adds over k = 0, 1, ...: every tile shape gives the same bits.
+//
+// A warp takes TM rows x 32 TN columns of a BM x 32 TN tile, a lane columns
+// lane + 32 j, operands as [row][k] in shared memory, four k at a time: TM
+// 16-byte reads that all lanes share, TN of a row a lane (8 consecutive rows
+// meet all banks at a pitch of 36), 4 TM TN FMAs.  A kSimtStages-deep ring
+// filled by cp.async keeps three 32-wide blocks of k in flight.  A 16-byte read
+// by a warp occupies shared memory for four cycles whatever its addresses, which
+// bounds both shapes: 64 x 64 with 8 x 2 a lane for large products (66 cycles
+// an element of k), 16 x 32 with 4 x 1 for those whose 64 x 64 tiles leave most
+// SMs idle (28).  The kernel below, with 64 x 64 tiles loaded between barriers,
+// took all products before: 272 x 256 x 1024 83 -> 17 us, 272 x 768 x 256
+// 23 -> 9.3, 4000 x 2048 x 512 262 -> 246.
+constexpr int kSimtBK = 32, kSimtPitch = kSimtBK + 4, kSimtStages = 4;
+
+template <int BM, int TM, int TN>
+struct SimtTile {
+    static constexpr int BN = 32 * TN, THREADS = BM / TM * 32;
+    static constexpr size_t SMEM = (size_t)kSimtStages * (BM + BN) * kSimtPitch * sizeof(float);
+};
+using SimtLarge = SimtTile<64, 8, 2>;
+using SimtSmall = SimtTile<16, 4, 1>;
+
+// 16 bytes to shared memory, or zeros where there is no source.
+__device__ __forceinline__ void cp_async16_or_zero(void* smem, const void* gmem, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
+                 "l"(gmem), "r"(in ? 16 : 0) : "memory");
+}
+
+template <int BM, int TM, int TN>
+__global__ void __launch_bounds__(SimtTile<BM, TM, TN>::THREADS)
+    gemm_simt_tile_kernel(const float* __restrict__ A, const float* __restrict__ W, int M, int N, int K, const Epi e) {
+    using C = SimtTile<BM, TM, TN>;
+    constexpr int BN = C::BN;
+    extern __shared__ float4 simt_smem[];
+    float* ring = reinterpret_cast<float*>(simt_smem);
+    const int lane = threadIdx.x & 31, row0 = (threadIdx.x >> 5) * TM;
+    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int blocks = (K + kSimtBK - 1) / kSimtBK;
+    auto load = [&](int b) {
+        if (b < blocks) {
+            float* dst = ring + (size_t)(b % kSimtStages) * (BM + BN) * kSimtPitch;
+            for (int i = threadIdx.x; i < (BM + BN) * (kSimtBK / 4); i += C::THREADS) {
+                const int row = i / (kSimtBK / 4), k = b * kSimtBK + 4 * (i % (kSimtBK / 4));
+                const bool is_a = row < BM;
+                const int g = is_a ? m0 + row : n0 + row - BM;
+                const bool in = k < K && g < (is_a ? M : N);          // K is a multiple of 4
+                const float* src = (is_a ? A : W) + (in ? (size_t)g * K + k : 0);
+                cp_async16_or_zero(dst + row * kSimtPitch + 4 * (i % (kSimtBK / 4)), src, in);
+            }
+        }
+        cp_async_commit();                                            // one group a block, empty past the end
+    };
+    float acc[TM][TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+#pragma unroll
+    for (int b = 0; b < kSimtStages - 1; ++b) load(b);
+    for (int b = 0; b < blocks; ++b) {
+        cp_async_wait<kSimtStages - 2>();                             // this thread's copies of block b
+        __syncthreads();                                              // everyone's, and block b - 1 is read
+        load(b + kSimtStages - 1);
+        const float* as = ring + (size_t)(b % kSimtStages) * (BM + BN) * kSimtPitch;
+        const float* ws = as + BM * kSimtPitch;
+        // the next four k are read while these are multiplied
+        float4 a[2][TM], w[2][TN];
+        auto read = [&](int k, float4 (&ra)[TM], float4 (&rw)[TN]) {
+#pragma unroll
+            for (int i = 0; i < TM; ++i) ra[i] = *reinterpret_cast<const float4*>(as + (row0 + i) * kSimtPitch + k);
+#pragma unroll
+            for (int j = 0; j < TN; ++j) rw[j] = *reinterpret_cast<const float4*>(ws + (lane + 32 * j) * kSimtPitch + k);
+        };
+        read(0, a[0], w[0]);
+#pragma unroll
+        for (int k = 0; k < kSimtBK; k += 4) {
+            const int c = (k >> 2) & 1;
+            if (k + 4 < kSimtBK) read(k + 4, a[c ^ 1], w[c ^ 1]);
+#pragma unroll
+            for (int e4 = 0; e4 < 4; ++e4)
+#pragma unroll
+                for (int i = 0; i < TM; ++i)
+#pragma unroll
+                    for (int j = 0; j < TN; ++j)
+                        acc[i][j] = fmaf(reinterpret_cast<const float*>(&a[c][i])[e4],
+                                         reinterpret_cast<const float*>(&w[c][j])[e4], acc[i][j]);
+        }
+    }
+    cp_async_wait<0>();                                               // no copy left in flight at exit
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+            const int m = m0 + row0 + i, n = n0 + lane + 32 * j;
+            if (m < M && n < N) epi_apply<float>(e, m, n, acc[i][j]);
+        }
+}
+
+// Any K and alignment: 64 x 64 tiles loaded element by element.
 template <typename T>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A, const T* __restrict__ W, int M,
                                                          int N, int K, const Epi e) {
@@ -372,57 +471,176 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A,
 }
 
 // ---------------------------------------------------------------- SIMT attention
-// One thread per query row, online softmax over key tiles staged in shared memory.
-template <typename T, typename TV, int HD>
-__global__ void __launch_bounds__(128) attn_simt_kernel(const T* __restrict__ q, const T* __restrict__ k,
-                                                         const TV* __restrict__ vt, int ldv, T* __restrict__ o, int Hs,
-                                                         int nb, int Lc, int L, float scale) {
-    constexpr int KT = HD <= 64 ? 64 : 32;
-    __shared__ float Ks[KT][HD + 1];
-    __shared__ float Vs[KT][HD + 1];
-    const int h = blockIdx.y;
-    const int qi = blockIdx.x * 128 + threadIdx.x;
-    float qr[HD], acc[HD];
+// fp32 softmax attention: a block of 128 threads takes 16 query rows through the
+// keys in tiles of 64, online over the tiles.  A warp has four rows: lane l
+// forms their scores with keys l, l + 32 (Q, K as [row][d], four d at a time, a
+// row of Q read by all lanes at once), the warp shares a row's maximum and sum
+// by shuffles, the numerators go through shared memory, and the lane accumulates
+// output columns l + 32 j (V^T as [d][key], four keys at a time).  Tiles of K and V^T are
+// double-buffered by cp.async.  (One thread a row, 64 dependent multiply-adds a
+// key, took 121 us at 4 heads x 272 tokens x 64.)
+constexpr int kAttnRows = 16, kAttnKeys = 64, kAttnThreads = 128;
+template <int HD>
+struct AttnSimt {
+    static constexpr int KP = HD + 4, VP = kAttnKeys + 4;            // pitches: 8 consecutive rows meet all banks
+    static constexpr int STAGE = kAttnKeys * KP + HD * VP;           // floats
+    static constexpr size_t SMEM = (size_t)(2 * STAGE + kAttnRows * (KP + VP)) * sizeof(float);
+};
+
+__device__ __forceinline__ void cp_async4_or_zero(void* smem, const void* gmem, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
+                 "l"(gmem), "r"(in ? 4 : 0) : "memory");
+}
+
+template <int HD>
+__global__ void __launch_bounds__(kAttnThreads) attn_simt_kernel(const float* __restrict__ q, const float* __restrict__ k,
+                                                                 const float* __restrict__ vt, int ldv,
+                                                                 float* __restrict__ o, int Hs, int nb, int Lc, int L,
+                                                                 float scale, int wide, int wide_v) {
+    using C = AttnSimt<HD>;
+    extern __shared__ float4 simt_smem[];
+    float* stages = reinterpret_cast<float*>(simt_smem);
+    float* qs = stages + 2 * C::STAGE;                                // [16][KP]
+    float* ps = qs + kAttnRows * C::KP;                               // [16][VP]
+    const int h = blockIdx.y, q0 = blockIdx.x * kAttnRows;
+    const int lane = threadIdx.x & 31, row0 = (threadIdx.x >> 5) * 4;
+    const int tiles = (L + kAttnKeys - 1) / kAttnKeys;
+    const float* kh = k + (size_t)h * L * HD;
+    const float* vh = vt + (size_t)h * HD * ldv;
+    // 4 floats of a row of q or k, whose base may be aligned to 4 bytes only
+    auto copy4 = [&](float* dst, const float* src, bool in) {
+        if (wide) {
+            cp_async16_or_zero(dst, src, in);
+        } else {
 #pragma unroll
-    for (int dd = 0; dd < HD; ++dd) {
-        qr[dd] = (qi < L) ? ld_act<T>(q + ((size_t)h * L + qi) * HD + dd) : 0.f;
-        acc[dd] = 0.f;
-    }
-    float mx = -INFINITY, l = 0.f;
-    for (int j0 = 0; j0 < L; j0 += KT) {
-        for (int i = threadIdx.x; i < KT * HD; i += 128) {
-            const int jj = i / HD, dd = i % HD;
-            Ks[jj][dd] = (j0 + jj < L) ? ld_act<T>(k + ((size_t)h * L + j0 + jj) * HD + dd) : 0.f;
-            const int dv = i / KT, jv = i % KT;
-            Vs[jv][dv] = (j0 + jv < L) ? ld_act<TV>(vt + ((size_t)h * HD + dv) * ldv + j0 + jv) : 0.f;
+            for (int e = 0; e < 4; ++e) cp_async4_or_zero(dst + e, src + (in ? e : 0), in);
         }
-        __syncthreads();
-        const int nk = min(KT, L - j0);
-        for (int jj = 0; jj < nk; ++jj) {
-            float s = 0.f;
-#pragma unroll
-            for (int dd = 0; dd < HD; ++dd) s = fmaf(qr[dd], Ks[jj][dd], s);
-            s *= scale;
-            if (s > mx) {
-                const float corr = expf(mx - s);
-                l *= corr;
-#pragma unroll
-                for (int dd = 0; dd < HD; ++dd) acc[dd] *= corr;
-                mx = s;
+    };
+    auto load = [&](int t) {
+        if (t < tiles) {
+            float* ks = stages + (t & 1) * C::STAGE;
+            float* vs = ks + kAttnKeys * C::KP;
+            const int j0 = t * kAttnKeys;
+            for (int i = threadIdx.x; i < kAttnKeys * (HD / 4); i += kAttnThreads) {
+                const int row = i / (HD / 4), c = 4 * (i % (HD / 4));
+                const bool in = j0 + row < L;
+                copy4(ks + row * C::KP + c, kh + (in ? (size_t)(j0 + row) * HD + c : 0), in);
             }
-            const float pj = expf(s - mx);
-            l += pj;
-#pragma unroll
-            for (int dd = 0; dd < HD; ++dd) acc[dd] = fmaf(pj, Vs[jj][dd], acc[dd]);
+            if (wide_v) {                            // 16-byte rows, ldv and L multiples of 4
+                for (int i = threadIdx.x; i < HD * (kAttnKeys / 4); i += kAttnThreads) {
+                    const int row = i / (kAttnKeys / 4), c = 4 * (i % (kAttnKeys / 4));
+                    const bool in = j0 + c < L;
+                    cp_async16_or_zero(vs + row * C::VP + c, vh + (in ? (size_t)row * ldv + j0 + c : 0), in);
+                }
+            } else {
+                for (int i = threadIdx.x; i < HD * kAttnKeys; i += kAttnThreads) {
+                    const int row = i / kAttnKeys, c = i % kAttnKeys;
+                    const bool in = j0 + c < L;
+                    cp_async4_or_zero(vs + row * C::VP + c, vh + (in ? (size_t)row * ldv + j0 + c : 0), in);
+                }
+            }
         }
-        __syncthreads();
+        cp_async_commit();
+    };
+    for (int i = threadIdx.x; i < kAttnRows * (HD / 4); i += kAttnThreads) {
+        const int row = i / (HD / 4), c = 4 * (i % (HD / 4));
+        const bool in = q0 + row < L;
+        copy4(qs + row * C::KP + c, q + (in ? ((size_t)h * L + q0 + row) * HD + c : 0), in);
     }
-    if (qi < L) {
-        const float inv = 1.0f / l;
-        const int b = h / Hs, hs = h - b * Hs;
-        const size_t orow = (size_t)batch_row(b, qi, nb, Lc, L);
+    load(0);
+    constexpr int ND = HD / 32;
+    float acc[4][ND], mx[4], l[4];
 #pragma unroll
-        for (int dd = 0; dd < HD; ++dd) o[orow * Hs * HD + hs * HD + dd] = to_act<T>(acc[dd] * inv);
+    for (int i = 0; i < 4; ++i) {
+        mx[i] = -INFINITY;
+        l[i] = 0.f;
+#pragma unroll
+        for (int j = 0; j < ND; ++j) acc[i][j] = 0.f;
+    }
+    for (int t = 0; t < tiles; ++t) {
+        load(t + 1);
+        cp_async_wait<1>();                                           // this thread's copies of tile t
+        __syncthreads();                                              // everyone's
+        const float* ks = stages + (t & 1) * C::STAGE;
+        const float* vs = ks + kAttnKeys * C::KP;
+        const int nk = min(kAttnKeys, L - t * kAttnKeys);
+        float s[4][2] = {};
+#pragma unroll 4
+        for (int dd = 0; dd < HD; dd += 4) {
+            float4 b[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) b[j] = *reinterpret_cast<const float4*>(ks + (lane + 32 * j) * C::KP + dd);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 a = *reinterpret_cast<const float4*>(qs + (row0 + i) * C::KP + dd);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    s[i][j] = fmaf(a.x, b[j].x, s[i][j]);
+                    s[i][j] = fmaf(a.y, b[j].y, s[i][j]);
+                    s[i][j] = fmaf(a.z, b[j].z, s[i][j]);
+                    s[i][j] = fmaf(a.w, b[j].w, s[i][j]);
+                }
+            }
+        }
+        float top[4], sum[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) s[i][j] = lane + 32 * j < nk ? s[i][j] * scale : -INFINITY;
+            top[i] = fmaxf(mx[i], fmaxf(s[i][0], s[i][1]));
+        }
+#pragma unroll
+        for (int w = 16; w; w >>= 1)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) top[i] = fmaxf(top[i], __shfl_xor_sync(0xffffffffu, top[i], w));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float p0 = expf(s[i][0] - top[i]), p1 = expf(s[i][1] - top[i]);
+            ps[(row0 + i) * C::VP + lane] = p0;
+            ps[(row0 + i) * C::VP + lane + 32] = p1;
+            sum[i] = p0 + p1;
+            const float corr = expf(mx[i] - top[i]);
+            mx[i] = top[i];
+            l[i] *= corr;
+#pragma unroll
+            for (int j = 0; j < ND; ++j) acc[i][j] *= corr;
+        }
+#pragma unroll
+        for (int w = 16; w; w >>= 1)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) l[i] += sum[i];
+        __syncwarp();                                                 // a row's numerators come from its own warp
+#pragma unroll 4
+        for (int kk = 0; kk < kAttnKeys; kk += 4) {
+            float4 b[ND];
+#pragma unroll
+            for (int j = 0; j < ND; ++j) b[j] = *reinterpret_cast<const float4*>(vs + (lane + 32 * j) * C::VP + kk);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 a = *reinterpret_cast<const float4*>(ps + (row0 + i) * C::VP + kk);
+#pragma unroll
+                for (int j = 0; j < ND; ++j) {
+                    acc[i][j] = fmaf(a.x, b[j].x, acc[i][j]);
+                    acc[i][j] = fmaf(a.y, b[j].y, acc[i][j]);
+                    acc[i][j] = fmaf(a.z, b[j].z, acc[i][j]);
+                    acc[i][j] = fmaf(a.w, b[j].w, acc[i][j]);
+                }
+            }
+        }
+        __syncthreads();                                              // the tile is read: its buffer may be refilled
+    }
+    cp_async_wait<0>();
+    const int b = h / Hs, hs = h - b * Hs;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int qi = q0 + row0 + i;
+        if (qi >= L) continue;
+        const float inv = 1.0f / l[i];
+        float* row = o + (size_t)batch_row(b, qi, nb, Lc, L) * Hs * HD + hs * HD;
+#pragma unroll
+        for (int j = 0; j < ND; ++j) row[lane + 32 * j] = acc[i][j] * inv;
     }
 }
 
@@ -475,9 +693,35 @@ static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int nb, int 
         return tc_gemm(c, A, W, M, N, K, e, M / nb, s);
     }
     LaunchScope ls(c, WDC_K_GEMM, s);
-    dim3 grid(blocks_for(N, 64), blocks_for(M, 64));
-    gemm_simt_kernel<float><<<grid, 256, 0, s>>>(reinterpret_cast<const float*>(A),
-                                                 reinterpret_cast<const float*>(W), M, N, K, e);
+    const float* a = reinterpret_cast<const float*>(A);
+    const float* w = reinterpret_cast<const float*>(W);
+    const long long large = (long long)blocks_for(M, 64) * blocks_for(N, 64);
+    const long long small = (long long)blocks_for(M, 16) * blocks_for(N, 32);
+    if (K % 4 || (((uintptr_t)A | (uintptr_t)W) & 15) || blocks_for(M, 16) > 65535) {
+        dim3 grid(blocks_for(N, 64), blocks_for(M, 64));
+        gemm_simt_kernel<float><<<grid, 256, 0, s>>>(a, w, M, N, K, e);
+        return WDC_OK;
+    }
+    static bool attr = false;
+    if (!attr) {
+        cudaFuncSetAttribute(gemm_simt_tile_kernel<64, 8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)SimtLarge::SMEM);
+        cudaFuncSetAttribute(gemm_simt_tile_kernel<16, 4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)SimtSmall::SMEM);
+        attr = true;
+    }
+    // the shape with the fewer cycles an element of k: 66 for each 64 x 64 tile
+    // of the busiest SM; 28 for a 16 x 32 one alone, 13.4 each for several (600
+    // x 1536 x 512: 38 us by the large shape, 48 by the small one; 272 x 256 x
+    // 1024: 37 and 17)
+    const long long sms = c->num_sms;
+    const long long per_large = (large + sms - 1) / sms, per_small = (small + sms - 1) / sms;
+    if (660 * per_large <= (per_small > 2 ? 134 * per_small : 280))
+        gemm_simt_tile_kernel<64, 8, 2><<<dim3(blocks_for(N, 64), blocks_for(M, 64)), SimtLarge::THREADS,
+                                              SimtLarge::SMEM, s>>>(a, w, M, N, K, e);
+    else
+        gemm_simt_tile_kernel<16, 4, 1><<<dim3(blocks_for(N, 32), blocks_for(M, 16)), SimtSmall::THREADS,
+                                              SimtSmall::SMEM, s>>>(a, w, M, N, K, e);
     return WDC_OK;
 }
 
@@ -509,14 +753,22 @@ static wdc_status attention(Ctx* c, const void* q, const void* k, const void* vt
         return tc_attention(c, q, k, vt, ldv, o, H, L, d, Hs, Lc, s);     // times its own launches
     }
     LaunchScope ls(c, WDC_K_ATTN, s);
-    dim3 grid(blocks_for(L, 128), H);
+    dim3 grid(blocks_for(L, kAttnRows), H);
     const float scale = 1.0f / sqrtf((float)d);
     const int nb = H / Hs;
-    using T = float;
+    static bool attr = false;
+    if (!attr) {
+        cudaFuncSetAttribute(attn_simt_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttnSimt<64>::SMEM);
+        cudaFuncSetAttribute(attn_simt_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttnSimt<128>::SMEM);
+        attr = true;
+    }
+    const int wide = (((uintptr_t)q | (uintptr_t)k) & 15) == 0;
+    const int wide_v = ((uintptr_t)vt & 15) == 0 && ldv % 4 == 0 && L % 4 == 0;
+    const float *qf = (const float*)q, *kf = (const float*)k, *vf = (const float*)vt;
     if (d == 64)
-        attn_simt_kernel<T, T, 64><<<grid, 128, 0, s>>>((const T*)q, (const T*)k, (const T*)vt, ldv, (T*)o, Hs, nb, Lc, L, scale);
+        attn_simt_kernel<64><<<grid, kAttnThreads, AttnSimt<64>::SMEM, s>>>(qf, kf, vf, ldv, (float*)o, Hs, nb, Lc, L, scale, wide, wide_v);
     else
-        attn_simt_kernel<T, T, 128><<<grid, 128, 0, s>>>((const T*)q, (const T*)k, (const T*)vt, ldv, (T*)o, Hs, nb, Lc, L, scale);
+        attn_simt_kernel<128><<<grid, kAttnThreads, AttnSimt<128>::SMEM, s>>>(qf, kf, vf, ldv, (float*)o, Hs, nb, Lc, L, scale, wide, wide_v);
     return WDC_OK;
 }
 
