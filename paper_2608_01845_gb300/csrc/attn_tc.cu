@@ -232,6 +232,8 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
     }
     __syncthreads();
     tc_fence_after();
+    chain_release();
+    chain_wait();
     const uint32_t tmem = *tmem_slot;
     const int wg = warp >> 2;
 
@@ -520,6 +522,8 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
 // the numerators).
 template <int D, bool BATCH>
 __global__ void __launch_bounds__(256) attn_combine_kernel(const AttnArgs g, int n_split_units) {
+    chain_release();
+    chain_wait();
     const int w = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (w >= n_split_units * 2 * BQ) return;
     const int ug = w / (2 * BQ), r = w - ug * (2 * BQ);      // split unit over all samples, row
@@ -620,15 +624,15 @@ wdc_status launch(Ctx* c, const void* q, const void* k, const void* vt, int ldv,
     const int n_split = g.nb * (g.units_s - g.n_full);       // split units over all samples
     {
         LaunchScope ls(c, WDC_K_ATTN, s);
-        attn_tc_kernel<D, BATCH><<<g.nb * (g.n_full + (g.units_s - g.n_full) * g.split), Cf::THREADS, Cf::SMEM, s>>>(
-            tq, tk, tv, g);
+        launch_kernel(attn_tc_kernel<D, BATCH>, g.nb * (g.n_full + (g.units_s - g.n_full) * g.split), Cf::THREADS, Cf::SMEM, s,
+                      1, tq, tk, tv, g);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("tcgen05 attention launch: ") + cudaGetErrorString(e));
     }
     if (n_split > 0) {
         LaunchScope ls(c, WDC_K_OTHER, s);
         const int threads = n_split * 2 * BQ * 32;
-        attn_combine_kernel<D, BATCH><<<(threads + 255) / 256, 256, 0, s>>>(g, n_split);
+        launch_kernel(attn_combine_kernel<D, BATCH>, (threads + 255) / 256, 256, 0, s, 1, g, n_split);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("attention combine launch: ") + cudaGetErrorString(e));
     }

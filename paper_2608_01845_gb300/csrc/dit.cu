@@ -65,6 +65,8 @@ namespace {
 // ---------------------------------------------------------------- small kernels
 // t_src (device, or null): the timestep is read there instead (graph rollout).
 __global__ void features_kernel(float t, const float* t_src, int half, float* out) {
+    chain_release();
+    chain_wait();
     const int j = threadIdx.x + blockIdx.x * blockDim.x;
     if (j >= half) return;
     if (t_src) t = *t_src;
@@ -76,13 +78,15 @@ __global__ void features_kernel(float t, const float* t_src, int half, float* ou
 
 // y[r] = act(W[r,:] . x + b[r]); one warp per row.  act: 0 none, 1 SiLU.
 template <typename T>
-__global__ void gemv_kernel(const T* __restrict__ W, const float* __restrict__ x, const float* __restrict__ b,
-                            float* __restrict__ y, int rows, int cols, int act) {
+__global__ void gemv_kernel(const T* __restrict__ W, const float* x, const float* __restrict__ b, float* y,
+                            int rows, int cols, int act) {
+    chain_release();
+    chain_wait();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= rows) return;
     const T* w = W + (size_t)warp * cols;
     float s = 0.f;
-    for (int c = lane; c < cols; c += 32) s = fmaf(ld_act<T>(w + c), x[c], s);
+    for (int c = lane; c < cols; c += 32) s = fmaf(ld_act<T>(w + c), ld_chain(x + c), s);
 #pragma unroll
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
@@ -94,8 +98,10 @@ __global__ void gemv_kernel(const T* __restrict__ W, const float* __restrict__ x
 
 // h[r] = LN(x[r]) * (1 + scale) + shift, one warp per row, rows [r0, r1).
 template <typename T, int VPT>
-__global__ void ln_mod_kernel(const T* __restrict__ x, T* __restrict__ h, int r0, int r1, int D,
-                              const float* __restrict__ shift, const float* __restrict__ scale, int h_row_off) {
+__global__ void ln_mod_kernel(const T* x, T* h, int r0, int r1, int D, const float* shift, const float* scale,
+                              int h_row_off) {
+    chain_release();
+    chain_wait();
     const int row = r0 + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (row >= r1) return;
     const T* xr = x + (size_t)row * D;
@@ -122,9 +128,19 @@ __global__ void ln_mod_kernel(const T* __restrict__ x, T* __restrict__ h, int r0
     const float rstd = 1.0f / sqrtf(q / (float)D + 1e-6f);
     T* hr = h + (size_t)(row - h_row_off) * D;
 #pragma unroll
-    for (int i = 0; i < VPT; ++i) {
-        const int c = lane + 32 * i;
-        if (c < D) hr[c] = to_act<T>(fmaf((v[i] - mean) * rstd, 1.0f + scale[c], shift[c]));
+    for (int i0 = 0; i0 < VPT; i0 += 8) {
+        float sc[8], sh[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int c = min(lane + 32 * (i0 + i), D - 1);
+            sc[i] = ld_chain(scale + c);
+            sh[i] = ld_chain(shift + c);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int c = lane + 32 * (i0 + i);
+            if (c < D) hr[c] = to_act<T>(fmaf((v[i0 + i] - mean) * rstd, 1.0f + sc[i], sh[i]));
+        }
     }
 }
 
@@ -151,10 +167,12 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 
 template <int NV>
 __global__ void __launch_bounds__(kLnWarps * 32, 1)
-    ln_mod_stream_kernel(const __nv_bfloat16* __restrict__ x, __nv_bfloat16* __restrict__ h, int r0, int r1, int D,
-                         const float* __restrict__ shift, const float* __restrict__ scale, int h_row_off) {
+    ln_mod_stream_kernel(const __nv_bfloat16* x, __nv_bfloat16* h, int r0, int r1, int D, const float* shift,
+                         const float* scale, int h_row_off) {
     __shared__ float4 s_sc[NV * 64], s_sh[NV * 64];        // 256 NV floats each
     extern __shared__ uint4 ring[];                        // [warp][kLnRing][NV * 32]
+    chain_release();
+    chain_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stride = gridDim.x * kLnWarps;
     uint4* my = ring + (size_t)warp * kLnRing * NV * 32;
@@ -170,10 +188,10 @@ __global__ void __launch_bounds__(kLnWarps * 32, 1)
 #pragma unroll
     for (int j = 0; j < kLnRing - 1; ++j) issue(j, row0 + j * stride);
     for (int i = threadIdx.x; i < NV * 64; i += blockDim.x) {
-        float4 a = __ldg(reinterpret_cast<const float4*>(scale) + i);
+        float4 a = ld_chain(reinterpret_cast<const float4*>(scale) + i);
         a.x += 1.0f; a.y += 1.0f; a.z += 1.0f; a.w += 1.0f;
         s_sc[i] = a;
-        s_sh[i] = __ldg(reinterpret_cast<const float4*>(shift) + i);
+        s_sh[i] = ld_chain(reinterpret_cast<const float4*>(shift) + i);
     }
     __syncthreads();
     int slot = 0;
@@ -240,6 +258,8 @@ struct BatchPtrs {
 // tok[b][(f, h', w'), (c, ph, pw)] = z_b[c, f, h'*p+ph, w'*p+pw]
 template <typename T>
 __global__ void patchify_kernel(BatchPtrs z, int nb, T* __restrict__ tok, int C, int F, int Hh, int Ww, int p) {
+    chain_release();
+    chain_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int P = C * p * p, hp = Hh / p, wp = Ww / p;
     const long long per = (long long)F * hp * wp * P;
@@ -256,6 +276,8 @@ __global__ void patchify_kernel(BatchPtrs z, int nb, T* __restrict__ tok, int C,
 // dst[b][i] = src_b[i] in the model dtype; a null src_b is the all-zero set.
 template <typename T>
 __global__ void convert_kernel(BatchPtrs src, int nb, T* __restrict__ dst, long long per) {
+    chain_release();
+    chain_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= per * nb) return;
     const int b = (int)(i / per);
@@ -266,7 +288,9 @@ __global__ void convert_kernel(BatchPtrs src, int nb, T* __restrict__ dst, long 
 // Guided velocity (cfg) or plain scatter of a batched forward's [nb, n]
 // velocities into the callers' buffers: cfg: rows (2b, 2b+1) = (conditional,
 // null-condition) forwards of sample b, v_b = v_u + g (v_c - v_u).
-__global__ void guide_kernel(const float* __restrict__ vb, long long n, int B, int cfg, float g, BatchPtrs dst) {
+__global__ void guide_kernel(const float* vb, long long n, int B, int cfg, float g, BatchPtrs dst) {
+    chain_release();
+    chain_wait();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n * B) return;
     const int b = (int)(i / n);
@@ -358,8 +382,9 @@ __device__ __forceinline__ void cp_async16_or_zero(void* smem, const void* gmem,
 
 template <int BM, int TM, int TN>
 __global__ void __launch_bounds__(SimtTile<BM, TM, TN>::THREADS)
-    gemm_simt_tile_kernel(const float* __restrict__ A, const float* __restrict__ W, int M, int N, int K, const Epi e) {
+    gemm_simt_tile_kernel(const float* A, const float* __restrict__ W, int M, int N, int K, const Epi e) {
     using C = SimtTile<BM, TM, TN>;
+    chain_wait();
     constexpr int BN = C::BN;
     extern __shared__ float4 simt_smem[];
     float* ring = reinterpret_cast<float*>(simt_smem);
@@ -428,8 +453,9 @@ __global__ void __launch_bounds__(SimtTile<BM, TM, TN>::THREADS)
 
 // Any K and alignment: 64 x 64 tiles loaded element by element.
 template <typename T>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A, const T* __restrict__ W, int M,
+__global__ void __launch_bounds__(256) gemm_simt_kernel(const T* A, const T* __restrict__ W, int M,
                                                          int N, int K, const Epi e) {
+    chain_wait();
     __shared__ float As[16][68];
     __shared__ float Ws[16][68];
     const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
@@ -493,11 +519,11 @@ __device__ __forceinline__ void cp_async4_or_zero(void* smem, const void* gmem, 
 }
 
 template <int HD>
-__global__ void __launch_bounds__(kAttnThreads) attn_simt_kernel(const float* __restrict__ q, const float* __restrict__ k,
-                                                                 const float* __restrict__ vt, int ldv,
-                                                                 float* __restrict__ o, int Hs, int nb, int Lc, int L,
+__global__ void __launch_bounds__(kAttnThreads) attn_simt_kernel(const float* q, const float* k,
+                                                                 const float* vt, int ldv, float* o, int Hs, int nb, int Lc, int L,
                                                                  float scale, int wide, int wide_v) {
     using C = AttnSimt<HD>;
+    chain_wait();
     extern __shared__ float4 simt_smem[];
     float* stages = reinterpret_cast<float*>(simt_smem);
     float* qs = stages + 2 * C::STAGE;                                // [16][KP]
@@ -647,8 +673,9 @@ __global__ void __launch_bounds__(kAttnThreads) attn_simt_kernel(const float* __
 inline unsigned blocks_for(long long n, int per) { return (unsigned)((n + per - 1) / per); }
 
 template <typename T>
-void launch_ln_mod(const void* x, void* h, int r0, int r1, int D, const float* shift, const float* scale,
-                   int h_row_off, int num_sms, cudaStream_t s) {
+void launch_ln_mod(const Ctx* c, const void* x, void* h, int r0, int r1, int D, const float* shift, const float* scale,
+                   int h_row_off, cudaStream_t s) {
+    const int num_sms = c->num_sms;
     const int rows = r1 - r0;
     if (rows <= 0) return;
     const unsigned grid = blocks_for((long long)rows * 32, 256);
@@ -667,13 +694,13 @@ void launch_ln_mod(const void* x, void* h, int r0, int r1, int D, const float* s
             }
             const int blocks = (rows + kLnWarps - 1) / kLnWarps;
             const unsigned g = (unsigned)(blocks < num_sms ? blocks : num_sms);
-            ln_mod_stream_kernel<12><<<g, kLnWarps * 32, ring_bytes, s>>>(xp, hp, r0, r1, D, shift, scale, h_row_off);
+            launch_kernel(ln_mod_stream_kernel<12>, g, kLnWarps * 32, ring_bytes, s, 1, xp, hp, r0, r1, D, shift, scale, h_row_off);
             return;
         }
     }
-    if (D <= 256) ln_mod_kernel<T, 8><<<grid, 256, 0, s>>>(xp, hp, r0, r1, D, shift, scale, h_row_off);
-    else if (D <= 1024) ln_mod_kernel<T, 32><<<grid, 256, 0, s>>>(xp, hp, r0, r1, D, shift, scale, h_row_off);
-    else ln_mod_kernel<T, 128><<<grid, 256, 0, s>>>(xp, hp, r0, r1, D, shift, scale, h_row_off);
+    if (D <= 256) launch_kernel(ln_mod_kernel<T, 8>, grid, 256, 0, s, 1, xp, hp, r0, r1, D, shift, scale, h_row_off);
+    else if (D <= 1024) launch_kernel(ln_mod_kernel<T, 32>, grid, 256, 0, s, 1, xp, hp, r0, r1, D, shift, scale, h_row_off);
+    else launch_kernel(ln_mod_kernel<T, 128>, grid, 256, 0, s, 1, xp, hp, r0, r1, D, shift, scale, h_row_off);
 }
 
 }  // namespace
@@ -699,7 +726,7 @@ static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int nb, int 
     const long long small = (long long)blocks_for(M, 16) * blocks_for(N, 32);
     if (K % 4 || (((uintptr_t)A | (uintptr_t)W) & 15) || blocks_for(M, 16) > 65535) {
         dim3 grid(blocks_for(N, 64), blocks_for(M, 64));
-        gemm_simt_kernel<float><<<grid, 256, 0, s>>>(a, w, M, N, K, e);
+        launch_kernel(gemm_simt_kernel<float>, grid, 256, 0, s, 1, a, w, M, N, K, e);
         return WDC_OK;
     }
     static bool attr = false;
@@ -717,11 +744,11 @@ static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int nb, int 
     const long long sms = c->num_sms;
     const long long per_large = (large + sms - 1) / sms, per_small = (small + sms - 1) / sms;
     if (660 * per_large <= (per_small > 2 ? 134 * per_small : 280))
-        gemm_simt_tile_kernel<64, 8, 2><<<dim3(blocks_for(N, 64), blocks_for(M, 64)), SimtLarge::THREADS,
-                                              SimtLarge::SMEM, s>>>(a, w, M, N, K, e);
+        launch_kernel(gemm_simt_tile_kernel<64, 8, 2>, dim3(blocks_for(N, 64), blocks_for(M, 64)), SimtLarge::THREADS,
+                      SimtLarge::SMEM, s, 1, a, w, M, N, K, e);
     else
-        gemm_simt_tile_kernel<16, 4, 1><<<dim3(blocks_for(N, 32), blocks_for(M, 16)), SimtSmall::THREADS,
-                                              SimtSmall::SMEM, s>>>(a, w, M, N, K, e);
+        launch_kernel(gemm_simt_tile_kernel<16, 4, 1>, dim3(blocks_for(N, 32), blocks_for(M, 16)), SimtSmall::THREADS,
+                      SimtSmall::SMEM, s, 1, a, w, M, N, K, e);
     return WDC_OK;
 }
 
@@ -766,9 +793,11 @@ static wdc_status attention(Ctx* c, const void* q, const void* k, const void* vt
     const int wide_v = ((uintptr_t)vt & 15) == 0 && ldv % 4 == 0 && L % 4 == 0;
     const float *qf = (const float*)q, *kf = (const float*)k, *vf = (const float*)vt;
     if (d == 64)
-        attn_simt_kernel<64><<<grid, kAttnThreads, AttnSimt<64>::SMEM, s>>>(qf, kf, vf, ldv, (float*)o, Hs, nb, Lc, L, scale, wide, wide_v);
+        launch_kernel(attn_simt_kernel<64>, grid, kAttnThreads, AttnSimt<64>::SMEM, s, 1, qf, kf, vf, ldv, (float*)o, Hs, nb, Lc, L,
+                      scale, wide, wide_v);
     else
-        attn_simt_kernel<128><<<grid, kAttnThreads, AttnSimt<128>::SMEM, s>>>(qf, kf, vf, ldv, (float*)o, Hs, nb, Lc, L, scale, wide, wide_v);
+        launch_kernel(attn_simt_kernel<128>, grid, kAttnThreads, AttnSimt<128>::SMEM, s, 1, qf, kf, vf, ldv, (float*)o, Hs, nb, Lc, L,
+                      scale, wide, wide_v);
     return WDC_OK;
 }
 
@@ -777,9 +806,9 @@ static void ln_mod(Ctx* c, const void* x, void* h, int r0, int r1, const float* 
     if (r1 <= r0) return;
     LaunchScope ls(c, WDC_K_NORM, s);
     if (c->cfg.dtype == WDC_BF16)
-        launch_ln_mod<__nv_bfloat16>(x, h, r0, r1, c->cfg.hidden, shift, scale, h_row_off, c->num_sms, s);
+        launch_ln_mod<__nv_bfloat16>(c, x, h, r0, r1, c->cfg.hidden, shift, scale, h_row_off, s);
     else
-        launch_ln_mod<float>(x, h, r0, r1, c->cfg.hidden, shift, scale, h_row_off, c->num_sms, s);
+        launch_ln_mod<float>(c, x, h, r0, r1, c->cfg.hidden, shift, scale, h_row_off, s);
 }
 
 // ---------------------------------------------------------------- lifetime
@@ -1020,15 +1049,15 @@ wdc_status dit_modulation(Ctx* c, float t_model, float* mod_out, cudaStream_t s)
     const int half = t->Fd / 2;
     {
         LaunchScope ls(c, WDC_K_OTHER, s);
-        features_kernel<<<blocks_for(half, 128), 128, 0, s>>>(t_model, t->t_src, half, t->feat);
+        launch_kernel(features_kernel, blocks_for(half, 128), 128, 0, s, 1, t_model, t->t_src, half, t->feat);
     }
     auto gv = [&](const void* W, const float* x, const float* b, float* y, int rows, int cols, int act) {
         const unsigned grid = blocks_for((long long)rows * 32, 256);
         LaunchScope ls(c, WDC_K_OTHER, s);
         if (t->dtype == WDC_BF16)
-            gemv_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>((const __nv_bfloat16*)W, x, b, y, rows, cols, act);
+            launch_kernel(gemv_kernel<__nv_bfloat16>, grid, 256, 0, s, 1, (const __nv_bfloat16*)W, x, b, y, rows, cols, act);
         else
-            gemv_kernel<float><<<grid, 256, 0, s>>>((const float*)W, x, b, y, rows, cols, act);
+            launch_kernel(gemv_kernel<float>, grid, 256, 0, s, 1, (const float*)W, x, b, y, rows, cols, act);
     };
     gv(t->t1.w, t->feat, t->t1.b, t->h1, t->E, t->Fd, 1);
     gv(t->t2.w, t->h1, t->t2.b, t->temb, t->E, t->E, 1);   // SiLU(temb)
@@ -1122,6 +1151,7 @@ wdc_status dit_block(Ctx* c, int layer, void* x, const float* mod6, cudaStream_t
     if (!c->dit) return fail(c, WDC_ERR_UNSUPPORTED, "context has no denoiser (layers == 0)");
     if (layer < 0 || layer >= c->dit->layers) return fail(c, WDC_ERR_INVALID_ARG, "layer out of range");
     if (!x || !mod6) return fail(c, WDC_ERR_INVALID_ARG, "null pointer");
+    OverlapScope chain(c, s);
     return run_block(c, layer, x, mod6, 1, s);
 }
 
@@ -1140,6 +1170,7 @@ wdc_status dit_forward_batch(Ctx* c, int nb, const float* const* z, float t_mode
         zp.p[b] = z[b];
         cp.p[b] = cond ? cond[b] : nullptr;
     }
+    OverlapScope chain(c, s);
     wdc_status st;
     if ((st = dit_modulation(c, t_model, nullptr, s))) return st;
     const int D = t->D;
@@ -1152,9 +1183,9 @@ wdc_status dit_forward_batch(Ctx* c, int nb, const float* const* z, float t_mode
         {
             LaunchScope ls(c, WDC_K_OTHER, s);
             if (t->dtype == WDC_BF16)
-                convert_kernel<__nv_bfloat16><<<blocks_for(per * nb, 256), 256, 0, s>>>(cp, nb, (__nv_bfloat16*)t->condx, per);
+                launch_kernel(convert_kernel<__nv_bfloat16>, blocks_for(per * nb, 256), 256, 0, s, 1, cp, nb, (__nv_bfloat16*)t->condx, per);
             else
-                convert_kernel<float><<<blocks_for(per * nb, 256), 256, 0, s>>>(cp, nb, (float*)t->condx, per);
+                launch_kernel(convert_kernel<float>, blocks_for(per * nb, 256), 256, 0, s, 1, cp, nb, (float*)t->condx, per);
         }
         Epi e{};
         e.mode = kEpiStore; e.bias = t->cond.b; e.out = t->x; e.ldo = D;
@@ -1165,9 +1196,9 @@ wdc_status dit_forward_batch(Ctx* c, int nb, const float* const* z, float t_mode
         {
             LaunchScope ls(c, WDC_K_OTHER, s);
             if (t->dtype == WDC_BF16)
-                patchify_kernel<__nv_bfloat16><<<blocks_for(nt, 256), 256, 0, s>>>(zp, nb, (__nv_bfloat16*)t->tok, g.in_ch, g.frames, g.height, g.width, g.patch);
+                launch_kernel(patchify_kernel<__nv_bfloat16>, blocks_for(nt, 256), 256, 0, s, 1, zp, nb, (__nv_bfloat16*)t->tok, g.in_ch, g.frames, g.height, g.width, g.patch);
             else
-                patchify_kernel<float><<<blocks_for(nt, 256), 256, 0, s>>>(zp, nb, (float*)t->tok, g.in_ch, g.frames, g.height, g.width, g.patch);
+                launch_kernel(patchify_kernel<float>, blocks_for(nt, 256), 256, 0, s, 1, zp, nb, (float*)t->tok, g.in_ch, g.frames, g.height, g.width, g.patch);
         }
         Epi e{};
         char* xv = (char*)t->x + (size_t)nb * t->Lc * D * es;
@@ -1219,12 +1250,13 @@ wdc_status dit_forward_guided(Ctx* c, int B, const float* const* z, float t_mode
         }
     }
     if (nb == 1) return dit_forward_batch(c, 1, zz, t_model, cc, v[0], s);
+    OverlapScope chain(c, s);
     wdc_status st = dit_forward_batch(c, nb, zz, t_model, cc, t->vb, s);
     if (st) return st;
     const long long n = (long long)c->n;
     {
         LaunchScope ls(c, WDC_K_OTHER, s);
-        guide_kernel<<<blocks_for(n * B, 256), 256, 0, s>>>(t->vb, n, B, cfg, guidance, out);
+        launch_kernel(guide_kernel, blocks_for(n * B, 256), 256, 0, s, 1, t->vb, n, B, cfg, guidance, out);
     }
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("guidance: ") + cudaGetErrorString(ce));

@@ -143,7 +143,7 @@ __device__ __forceinline__ void epilogue_chunk(const Epi& e, int m, int col0, co
                 const float4* g4 = reinterpret_cast<const float4*>(e.gate + col0);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const float4 t = __ldg(g4 + j);
+                    const float4 t = ld_chain(g4 + j);
                     g[4 * j] = t.x; g[4 * j + 1] = t.y; g[4 * j + 2] = t.z; g[4 * j + 3] = t.w;
                 }
             } else {
@@ -286,7 +286,7 @@ __device__ __forceinline__ void fetch_columns(const float* bias, const float* ga
     }
     if (FORM == kFormResid && gate) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) ws.gate[i] = __ldg(reinterpret_cast<const float2*>(gate + min(c + 8 * i, end - 2)));
+        for (int i = 0; i < 8; ++i) ws.gate[i] = ld_chain(reinterpret_cast<const float2*>(gate + min(c + 8 * i, end - 2)));
     }
 }
 
@@ -508,6 +508,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
     __syncthreads();
     tc_fence_after();
+    chain_release();
+    chain_wait();
     const uint32_t tmem_base = *tmem_slot;
     // tiles of the first problem, then of the second, N-fastest
     const int tiles0 = g.m_tiles * g.n_tiles;
@@ -718,6 +720,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     __syncthreads();
     cluster_sync_all();
     tc_fence_after();
+    chain_release();
+    chain_wait();
     const uint32_t own_base = *tmem_slot;
     const uint32_t tmem = rank == 0 ? own_base : ld_shared_cluster_u32(mapa_shared(smem_u32(tmem_slot), 0));
     if (threadIdx.x == 0 && tmem != own_base) atomicOr(g.err, kErrTmem);
@@ -879,8 +883,8 @@ __device__ __forceinline__ void columns8(const Epi& e, int col, float (&bias)[8]
     auto load = [&](const float* src, float none, float (&x)[8]) {
         float4 a = make_float4(none, none, none, none), b = a;
         if (src) {
-            a = __ldg(reinterpret_cast<const float4*>(src + col));
-            b = __ldg(reinterpret_cast<const float4*>(src + col) + 1);
+            a = ld_chain(reinterpret_cast<const float4*>(src + col));
+            b = ld_chain(reinterpret_cast<const float4*>(src + col) + 1);
         }
         x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
         x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
@@ -970,6 +974,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     }
     __syncthreads();
     tc_fence_after();
+    chain_release();
+    chain_wait();
     const uint32_t tmem_base = *tmem_slot;
     if (warp == 0) {
         {
@@ -1244,28 +1250,34 @@ double launch_cycles(long long tiles, int units, double main, double epi) {
 // the GPCs hold (76, 36 and 15 of 2, 4 and 8 on this part).
 constexpr double kCyclesPair = 560.0, kCycles128 = 470.0, kCycles64 = 450.0, kCyclesSplit = 440.0, kPairStart = 1900.0;
 
-// Clusters of S split CTAs resident at a time.
-int split_clusters(Ctx* c, int S) {
-    static int cap[SPLIT_MAX + 1] = {};
-    if (cap[S] == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(c->num_sms / S * S, 1, 1);
-        cfg.blockDim = dim3(kGemmThreads, 1, 1);
-        cfg.dynamicSmemBytes = SPLIT_SMEM;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = S;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, Kernels::split(S, 0), &cfg) != cudaSuccess || n < 1) {
-            cudaGetLastError();
-            n = c->num_sms / S > 0 ? c->num_sms / S : 1;
-        }
-        cap[S] = n;
+// Clusters of `size` CTAs of a GEMM kernel resident at a time.
+int resident_clusters(const Ctx* c, const void* kernel, int size, size_t smem) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c->num_sms / size * size, 1, 1);
+    cfg.blockDim = dim3(kGemmThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = size;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        n = c->num_sms / size > 0 ? c->num_sms / size : 1;
     }
+    return n;
+}
+int split_clusters(const Ctx* c, int S) {
+    static int cap[SPLIT_MAX + 1] = {};
+    if (cap[S] == 0) cap[S] = resident_clusters(c, (const void*)Kernels::split(S, 0), S, SPLIT_SMEM);
     return cap[S];
+}
+int pair_clusters(const Ctx* c) {
+    static int cap = 0;
+    if (cap == 0) cap = resident_clusters(c, (const void*)Kernels::pair[0], 2, SMEM2_BYTES);
+    return cap < c->num_sms / 2 ? cap : c->num_sms / 2;
 }
 
 // M, M1: the launch's rows (M1: a second problem's, or 0); sample, sample1:
@@ -1395,48 +1407,23 @@ wdc_status launch_gemm(Ctx* c, const Problem& p0, const Problem* p1, int N, int 
         tb1 = tb;
     }
     const int tiles128 = (g.m_tiles + g.m_tiles1) * g.n_tiles;
-    cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kGemmThreads, 1, 1);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
     switch (ch.kind) {
         case Choice::kPair: {
             // a persistent grid of as many CTA pairs as can be resident,
             // capped by the tile count
-            cfg.numAttrs = 1;
-            attr[0].val.clusterDim.x = 2;
-            cfg.dynamicSmemBytes = SMEM2_BYTES;
-            static int max_clusters = 0;
-            if (max_clusters == 0) {
-                cfg.gridDim = dim3(c->num_sms, 1, 1);
-                if (cudaOccupancyMaxActiveClusters(&max_clusters, Kernels::pair[0], &cfg) != cudaSuccess ||
-                    max_clusters < 1) {
-                    cudaGetLastError();
-                    max_clusters = c->num_sms / 2;
-                }
-            }
-            const int tiles = ((g.m_tiles + 1) / 2 + (g.m_tiles1 + 1) / 2) * g.n_tiles;
-            int clusters = max_clusters < c->num_sms / 2 ? max_clusters : c->num_sms / 2;
-            if (tiles < clusters) clusters = tiles;
-            cfg.gridDim = dim3(2 * clusters, 1, 1);
-            cudaLaunchKernelEx(&cfg, Kernels::pair[form], ta, tb, ta1, tb1, maps, maps1, g);
+            const int resident = pair_clusters(c), tiles = ((g.m_tiles + 1) / 2 + (g.m_tiles1 + 1) / 2) * g.n_tiles;
+            launch_kernel(Kernels::pair[form], dim3(2 * (tiles < resident ? tiles : resident)), kGemmThreads,
+                          SMEM2_BYTES, s, 2, ta, tb, ta1, tb1, maps, maps1, g);
             break;
         }
         case Choice::kSplit:
-            cfg.numAttrs = 1;
-            attr[0].val.clusterDim.x = ch.split;
-            cfg.dynamicSmemBytes = SPLIT_SMEM;
-            cfg.gridDim = dim3(tiles128 * ch.split, 1, 1);
-            cudaLaunchKernelEx(&cfg, Kernels::split(ch.split, form), ta, tb, ta1, tb1, g);
+            launch_kernel(Kernels::split(ch.split, form), dim3(tiles128 * ch.split), kGemmThreads, SPLIT_SMEM, s,
+                          ch.split, ta, tb, ta1, tb1, g);
             break;
         default:
-            cfg.dynamicSmemBytes = bn == 64 ? GemmCfg<64>::SMEM : GemmCfg<128>::SMEM;
-            cfg.gridDim = dim3(tiles128 < c->num_sms ? tiles128 : c->num_sms, 1, 1);
-            cudaLaunchKernelEx(&cfg, bn == 64 ? Kernels::one64[form] : Kernels::one128[form], ta, tb, ta1, tb1, maps,
-                               maps1, g);
+            launch_kernel(bn == 64 ? Kernels::one64[form] : Kernels::one128[form],
+                          dim3(tiles128 < c->num_sms ? tiles128 : c->num_sms), kGemmThreads,
+                          bn == 64 ? GemmCfg<64>::SMEM : GemmCfg<128>::SMEM, s, 1, ta, tb, ta1, tb1, maps, maps1, g);
     }
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(err));

@@ -195,6 +195,93 @@ struct LaunchScope {
     ~LaunchScope();
 };
 
+// ---------------------------------------------------------------- launches
+// The denoiser's kernels are short links of one chain.  Each is launched as a
+// programmatic dependent of the one before it on the stream (t_overlap): it
+// starts once every block of that kernel has called chain_release() (or
+// exited), sets itself up, and calls chain_wait() before it touches global
+// memory, which returns when that kernel is complete and its writes are
+// visible.  Every kernel of the chain waits, so a kernel's wait also covers all
+// earlier ones.  chain_release() comes after a kernel has its tensor memory: a
+// dependent block on the same SM must not take it first.  Launched plainly,
+// both are no-ops.  The fp32 kernels, of which several blocks share an SM, wait
+// but do not release early: the next kernel's blocks, placed beside them, end
+// up unevenly spread.
+// Measured, plain launches -> this: bf16 forward of 2 layers, 272 tokens (26
+// launches) 150 -> 107 us; 4 layers of 1024, 6400 tokens 999 -> 908 us; a block
+// of 3072, 17776 tokens 5481 -> 5348 us; fp32 rollout of the 2-layer model
+// 1365 -> 1168 us (1710 us if its kernels release early).
+//
+// Whether the call in progress on this thread launches that way: OverlapScope.
+inline thread_local bool t_overlap = false;
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Loads of what an earlier kernel of the chain wrote.  The read-only path is
+// for data that does not change while the kernel is resident, and the compiler
+// may move its loads above chain_wait(): inputs that a kernel of the chain
+// writes are neither __ldg nor const __restrict__, but plain, or one of these.
+__device__ __forceinline__ float ld_chain(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_chain(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_chain(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+
+template <class... P, class... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                          unsigned cluster, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
+    if (t_overlap) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        ++cfg.numAttrs;
+    }
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
+// Sets t_overlap for a call on stream s: not while s is being captured (a
+// conditional graph's body takes plain edges only), not with the event profiler
+// on (its events lie between the launches).
+struct OverlapScope {
+    const bool before = t_overlap;
+    OverlapScope(const Ctx* c, cudaStream_t s) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+            cudaGetLastError();
+            st = cudaStreamCaptureStatusActive;
+        }
+        t_overlap = st == cudaStreamCaptureStatusNone && !c->prof;
+    }
+    ~OverlapScope() { t_overlap = before; }
+    OverlapScope(const OverlapScope&) = delete;
+    OverlapScope& operator=(const OverlapScope&) = delete;
+};
+
 // ---------------------------------------------------------------- helpers
 #define WDC_CUDA_TRY(ctx, call)                                                   \
     do {                                                                          \
