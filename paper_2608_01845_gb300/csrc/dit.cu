@@ -63,30 +63,48 @@ struct DiT {
 namespace {
 
 // ---------------------------------------------------------------- small kernels
-// t_src (device, or null): the timestep is read there instead (graph rollout).
-__global__ void features_kernel(float t, const float* t_src, int half, float* out) {
-    chain_release();
-    chain_wait();
-    const int j = threadIdx.x + blockIdx.x * blockDim.x;
-    if (j >= half) return;
-    if (t_src) t = *t_src;
-    const double w = exp(-log(10000.0) * (double)j / (double)half);
-    const double a = (double)t * w;
-    out[j] = (float)cos(a);
-    out[half + j] = (float)sin(a);
-}
-
 // y[r] = act(W[r,:] . x + b[r]); one warp per row.  act: 0 none, 1 SiLU.
+// Bound by the latency of its loads (E x E) or by reading W (the modulation).
+// With whole 16-byte vectors in a row (vec) each lane loads up to four of W's
+// before the wait for x: W is constant, so its reads run under the kernels
+// before.  Alone, 26624 x 512 bf16 (27 MB, cold) takes 10 us as with 2-byte
+// loads; the gain is in the chain (with prep_kernel's, see there).
 template <typename T>
-__global__ void gemv_kernel(const T* __restrict__ W, const float* x, const float* __restrict__ b, float* y,
-                            int rows, int cols, int act) {
+__global__ void __launch_bounds__(256) gemv_kernel(const T* __restrict__ W, const float* x, const float* __restrict__ b,
+                                                   float* y, int rows, int cols, int act, int vec) {
+    constexpr int VEC = 16 / (int)sizeof(T), PRE = 4;
     chain_release();
-    chain_wait();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const T* w = W + (size_t)min(warp, rows - 1) * cols;
+    const uint4* w4 = reinterpret_cast<const uint4*>(w);
+    const int nv = vec ? cols / VEC : 0;
+    uint4 u[PRE];
+#pragma unroll
+    for (int i = 0; i < PRE; ++i)
+        if (lane + 32 * i < nv) u[i] = w4[lane + 32 * i];
+    chain_wait();
     if (warp >= rows) return;
-    const T* w = W + (size_t)warp * cols;
     float s = 0.f;
-    for (int c = lane; c < cols; c += 32) s = fmaf(ld_act<T>(w + c), ld_chain(x + c), s);
+    auto add = [&](const uint4& q, int v) {                // the terms of vector v
+        const float4* xv = reinterpret_cast<const float4*>(x + (size_t)v * VEC);
+        const T* t = reinterpret_cast<const T*>(&q);
+#pragma unroll
+        for (int k = 0; k < VEC / 4; ++k) {
+            const float4 f = ld_chain(xv + k);
+            s = fmaf(ld_act<T>(t + 4 * k), f.x, s);
+            s = fmaf(ld_act<T>(t + 4 * k + 1), f.y, s);
+            s = fmaf(ld_act<T>(t + 4 * k + 2), f.z, s);
+            s = fmaf(ld_act<T>(t + 4 * k + 3), f.w, s);
+        }
+    };
+    if (vec) {
+#pragma unroll
+        for (int i = 0; i < PRE; ++i)
+            if (lane + 32 * i < nv) add(u[i], lane + 32 * i);
+        for (int v = lane + 32 * PRE; v < nv; v += 32) add(w4[v], v);
+    } else {
+        for (int c = lane; c < cols; c += 32) s = fmaf(ld_act<T>(w + c), ld_chain(x + c), s);
+    }
 #pragma unroll
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
@@ -327,34 +345,71 @@ struct BatchPtrs {
     const float* p[WDC_MAX_BATCH];
 };
 
-// tok[b][(f, h', w'), (c, ph, pw)] = z_b[c, f, h'*p+ph, w'*p+pw]
+// What a forward computes from its inputs alone, in one launch; each block has
+// one of three parts:
+//   timestep features (the first n_feat blocks, one warp each, since an SM does
+//     two fp64 operations a cycle): cos and sin of t w_j; t_src (device, or
+//     null): the timestep is read there (graph rollout)
+//   patches: tok[b][(f, h', w'), (c, ph, pw)] = z_b[c, f, h'*p+ph, w'*p+pw],
+//     whole tokens per block, so that the index divisions are of 32 bits
+//   condition tokens: condx[b][i] = cond_b[i] in the model dtype; a null cond_b
+//     is the all-zero set
+// The parts are latency, not bandwidth: as three launches with an element and
+// five 64-bit divisions a thread 6.8 + 6.7 + 9.5 us for 4 x 1536 tokens (each
+// cold), here 6.2.  With gemv_kernel's early loads, a forward of that size 878 -> 868
+// us, of 272 tokens 105.4 -> 103.6 us, the fp32 rollout 1164 -> 1150 us.
+constexpr int kPrepThreads = 256, kPrepElems = 1024, kPrepFeat = 32;
+struct PrepArgs {
+    BatchPtrs z, cond;
+    float t;
+    const float* t_src;
+    float* feat;
+    int half, n_feat;
+    int C, F, Hh, Ww, p, tokens, tok_per_block, tok_blocks;      // per sample
+    long long cond_per;
+    unsigned cond_blocks, patch_blocks;                          // per sample; all samples
+};
 template <typename T>
-__global__ void patchify_kernel(BatchPtrs z, int nb, T* __restrict__ tok, int C, int F, int Hh, int Ww, int p) {
+__global__ void __launch_bounds__(kPrepThreads)
+    prep_kernel(const __grid_constant__ PrepArgs a, T* tok, T* condx) {
     chain_release();
     chain_wait();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int P = C * p * p, hp = Hh / p, wp = Ww / p;
-    const long long per = (long long)F * hp * wp * P;
-    if (i >= per * nb) return;
-    const int b = (int)(i / per);
-    const long long ii = i - b * per;
-    const int col = (int)(ii % P);
-    const long long m = ii / P;
-    const int f = (int)(m / (hp * wp)), rem = (int)(m % (hp * wp)), h2 = rem / wp, w2 = rem % wp;
-    const int c = col / (p * p), r2 = col % (p * p), ph = r2 / p, pw = r2 % p;
-    tok[i] = to_act<T>(z.p[b][(((size_t)c * F + f) * Hh + h2 * p + ph) * Ww + w2 * p + pw]);
-}
-
-// dst[b][i] = src_b[i] in the model dtype; a null src_b is the all-zero set.
-template <typename T>
-__global__ void convert_kernel(BatchPtrs src, int nb, T* __restrict__ dst, long long per) {
-    chain_release();
-    chain_wait();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= per * nb) return;
-    const int b = (int)(i / per);
-    const float* sp = src.p[b];
-    dst[i] = to_act<T>(sp ? sp[i - b * per] : 0.0f);
+    unsigned blk = blockIdx.x;
+    if (blk < (unsigned)a.n_feat) {
+        const int i = (int)(blk * kPrepFeat + threadIdx.x);
+        if (threadIdx.x >= kPrepFeat || i >= 2 * a.half) return;
+        const int j = i < a.half ? i : i - a.half;
+        const float t = a.t_src ? *a.t_src : a.t;
+        const double w = exp(-log(10000.0) * (double)j / (double)a.half);
+        const double x = (double)t * w;
+        a.feat[i] = (float)(i < a.half ? cos(x) : sin(x));
+        return;
+    }
+    blk -= a.n_feat;
+    if (blk < a.patch_blocks) {
+        const unsigned b = blk / a.tok_blocks;
+        const unsigned m0 = (blk - b * a.tok_blocks) * a.tok_per_block;
+        const unsigned P = a.C * a.p * a.p, hp = a.Hh / a.p, wp = a.Ww / a.p;
+        const unsigned n = min((unsigned)a.tok_per_block, a.tokens - m0) * P;
+        const float* z = a.z.p[b];
+        T* out = tok + ((size_t)b * a.tokens + m0) * P;
+        for (unsigned e = threadIdx.x; e < n; e += kPrepThreads) {
+            const unsigned tl = e / P, col = e - tl * P, row = (m0 + tl) / wp, w2 = m0 + tl - row * wp;
+            const unsigned f = row / hp, h2 = row - f * hp;
+            const unsigned cp = col / a.p, pw = col - cp * a.p, c = cp / a.p, ph = cp - c * a.p;
+            out[e] = to_act<T>(z[(((size_t)c * a.F + f) * a.Hh + h2 * a.p + ph) * a.Ww + w2 * a.p + pw]);
+        }
+        return;
+    }
+    blk -= a.patch_blocks;
+    const unsigned b = blk / a.cond_blocks;
+    const long long i0 = (long long)(blk - b * a.cond_blocks) * kPrepElems;
+    const float* src = a.cond.p[b];
+#pragma unroll
+    for (int q = 0; q < kPrepElems / kPrepThreads; ++q) {
+        const long long i = i0 + q * kPrepThreads + threadIdx.x;
+        if (i < a.cond_per) condx[b * a.cond_per + i] = to_act<T>(src ? src[i] : 0.0f);
+    }
 }
 
 // Guided velocity (cfg) or plain scatter of a batched forward's [nb, n]
@@ -1120,22 +1175,45 @@ wdc_status dit_init_weights(Ctx* c, unsigned long long seed, float std) {
 }
 
 // ---------------------------------------------------------------- forward
-wdc_status dit_modulation(Ctx* c, float t_model, float* mod_out, cudaStream_t s) {
+// The prologue of a forward of nb samples (nb = 0: the timestep features alone).
+static void prep(Ctx* c, int nb, const BatchPtrs& z, const BatchPtrs& cond, float t_model, cudaStream_t s) {
     DiT* t = c->dit;
-    if (!t) return fail(c, WDC_ERR_UNSUPPORTED, "context has no denoiser (layers == 0)");
-    float* dst = mod_out ? mod_out : t->mods;
-    const int half = t->Fd / 2;
-    {
-        LaunchScope ls(c, WDC_K_OTHER, s);
-        launch_kernel(features_kernel, blocks_for(half, 128), 128, 0, s, 1, t_model, t->t_src, half, t->feat);
-    }
+    const wdc_dit_config& g = c->cfg;
+    PrepArgs a{};
+    a.z = z;
+    a.cond = cond;
+    a.t = t_model;
+    a.t_src = t->t_src;
+    a.feat = t->feat;
+    a.half = t->Fd / 2;
+    a.n_feat = (int)blocks_for(2 * a.half, kPrepFeat);
+    a.C = g.in_ch; a.F = g.frames; a.Hh = g.height; a.Ww = g.width; a.p = g.patch;
+    a.tokens = t->Lv;
+    a.tok_per_block = t->P < kPrepElems ? kPrepElems / t->P : 1;
+    a.tok_blocks = (int)blocks_for(t->Lv, a.tok_per_block);
+    a.patch_blocks = (unsigned)(nb * a.tok_blocks);
+    a.cond_per = (long long)t->Lc * t->Dc;
+    a.cond_blocks = t->Lc > 0 ? blocks_for(a.cond_per, kPrepElems) : 0;
+    const unsigned grid = a.n_feat + a.patch_blocks + nb * a.cond_blocks;
+    LaunchScope ls(c, WDC_K_OTHER, s);
+    if (t->dtype == WDC_BF16)
+        launch_kernel(prep_kernel<__nv_bfloat16>, grid, kPrepThreads, 0, s, 1, a, (__nv_bfloat16*)t->tok,
+                      (__nv_bfloat16*)t->condx);
+    else
+        launch_kernel(prep_kernel<float>, grid, kPrepThreads, 0, s, 1, a, (float*)t->tok, (float*)t->condx);
+}
+
+// All layers' modulation vectors from the timestep features.
+static wdc_status modulation(Ctx* c, float* dst, cudaStream_t s) {
+    DiT* t = c->dit;
     auto gv = [&](const void* W, const float* x, const float* b, float* y, int rows, int cols, int act) {
         const unsigned grid = blocks_for((long long)rows * 32, 256);
+        const int vec = cols % (16 / (int)t->esz) == 0 && (((uintptr_t)W | (uintptr_t)x) & 15) == 0;
         LaunchScope ls(c, WDC_K_OTHER, s);
         if (t->dtype == WDC_BF16)
-            launch_kernel(gemv_kernel<__nv_bfloat16>, grid, 256, 0, s, 1, (const __nv_bfloat16*)W, x, b, y, rows, cols, act);
+            launch_kernel(gemv_kernel<__nv_bfloat16>, grid, 256, 0, s, 1, (const __nv_bfloat16*)W, x, b, y, rows, cols, act, vec);
         else
-            launch_kernel(gemv_kernel<float>, grid, 256, 0, s, 1, (const float*)W, x, b, y, rows, cols, act);
+            launch_kernel(gemv_kernel<float>, grid, 256, 0, s, 1, (const float*)W, x, b, y, rows, cols, act, vec);
     };
     gv(t->t1.w, t->feat, t->t1.b, t->h1, t->E, t->Fd, 1);
     gv(t->t2.w, t->h1, t->t2.b, t->temb, t->E, t->E, 1);   // SiLU(temb)
@@ -1143,6 +1221,12 @@ wdc_status dit_modulation(Ctx* c, float t_model, float* mod_out, cudaStream_t s)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("modulation: ") + cudaGetErrorString(e));
     return WDC_OK;
+}
+
+wdc_status dit_modulation(Ctx* c, float t_model, float* mod_out, cudaStream_t s) {
+    if (!c->dit) return fail(c, WDC_ERR_UNSUPPORTED, "context has no denoiser (layers == 0)");
+    prep(c, 0, BatchPtrs{}, BatchPtrs{}, t_model, s);
+    return modulation(c, mod_out ? mod_out : c->dit->mods, s);
 }
 
 // One block on x (device, [nb*L, D], stream-major batch rows) with mod
@@ -1250,34 +1334,19 @@ wdc_status dit_forward_batch(Ctx* c, int nb, const float* const* z, float t_mode
     }
     OverlapScope chain(c, s);
     wdc_status st;
-    if ((st = dit_modulation(c, t_model, nullptr, s))) return st;
+    prep(c, nb, zp, cp, t_model, s);
+    if ((st = modulation(c, t->mods, s))) return st;
     const int D = t->D;
     const size_t es = t->esz;
     const wdc_dit_config& g = c->cfg;
     // embed: condition tokens (rows [0, nb*Lc)), then patches + position
     // (rows [nb*Lc, nb*L))
     if (t->Lc > 0) {
-        const long long per = (long long)t->Lc * t->Dc;
-        {
-            LaunchScope ls(c, WDC_K_OTHER, s);
-            if (t->dtype == WDC_BF16)
-                launch_kernel(convert_kernel<__nv_bfloat16>, blocks_for(per * nb, 256), 256, 0, s, 1, cp, nb, (__nv_bfloat16*)t->condx, per);
-            else
-                launch_kernel(convert_kernel<float>, blocks_for(per * nb, 256), 256, 0, s, 1, cp, nb, (float*)t->condx, per);
-        }
         Epi e{};
         e.mode = kEpiStore; e.bias = t->cond.b; e.out = t->x; e.ldo = D;
         if ((st = gemm(c, t->condx, t->cond.w, nb * t->Lc, nb, D, t->Dc, e, s))) return st;
     }
     {
-        const long long nt = (long long)t->Lv * t->P * nb;
-        {
-            LaunchScope ls(c, WDC_K_OTHER, s);
-            if (t->dtype == WDC_BF16)
-                launch_kernel(patchify_kernel<__nv_bfloat16>, blocks_for(nt, 256), 256, 0, s, 1, zp, nb, (__nv_bfloat16*)t->tok, g.in_ch, g.frames, g.height, g.width, g.patch);
-            else
-                launch_kernel(patchify_kernel<float>, blocks_for(nt, 256), 256, 0, s, 1, zp, nb, (float*)t->tok, g.in_ch, g.frames, g.height, g.width, g.patch);
-        }
         Epi e{};
         char* xv = (char*)t->x + (size_t)nb * t->Lc * D * es;
         e.mode = kEpiResid; e.bias = t->patch.b; e.out = xv; e.res = t->pe; e.res_rows = t->Lv; e.ldo = D; e.gate = nullptr;
