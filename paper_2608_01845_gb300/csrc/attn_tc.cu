@@ -49,8 +49,8 @@
 // at 24 x 13568 x 128).  Tiles half a step apart hold a stage of K and V
 // longer: five stages instead of three, 227 -> 203 us at 48 x 4276 x 64.
 // Grid: one CTA per (head, 256-query) unit, one CTA per SM.  The units of a
-// sample's last, partial round are split over the key range instead: each
-// part runs the same pipeline over its steps and writes its unnormalised O,
+// sample's last, partial round are split over the key range where that saves
+// enough steps (attn_split): each part runs the same pipeline over its steps and writes its unnormalised O,
 // exponent base and row sum to a workspace of the context, and
 // attn_combine_kernel merges the parts, so the round's CTAs fill the SMs.
 // Keys past L are masked (TMA zero-fills out-of-range K / V^T).  Every
@@ -564,15 +564,24 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const AttnArgs g, int
 
 // Units of a sample's last, partial round are split over the key range so
 // that its CTAs fill the SMs: r = units mod SMs leftover units, each in
-// min(8, SMs / r, steps) parts (none when the grid is whole rounds).
-int attn_split(int units, int num_sms, int n_kv, int& n_full) {
+// min(8, SMs / r, steps) parts (none when the grid is whole rounds).  The parts'
+// unnormalised rows and attn_combine_kernel cost about as much as
+// kMinSaved steps (5 - 7 us of 0.88 us steps at d = 64, 6 - 8 us of 0.67 us
+// at d = 128), so a split that saves fewer is left out.  Whole -> split, us:
+//   d = 64:  L = 272, 24 heads 8.8 -> 12.2 (saves 2); 700, 2 heads 10.4 -> 11.0
+//            (5); 900, 4 heads 12.4 -> 11.2 (7); 1600, 24 heads 32.7 -> 28.5 (11)
+//   d = 128: L = 272, 2 heads 9.8 -> 12.7 (4); 900, 12 heads 18.0 -> 18.5 (10);
+//            900, 6 heads 17.6 -> 15.7 (12); 1600, 24 heads 45.4 -> 39.8 (21)
+template <int D>
+constexpr int kMinSaved = D == 64 ? 7 : 11;
+int attn_split(int units, int num_sms, int n_kv, int min_saved, int& n_full) {
     n_full = units;
     const int r = units % num_sms;
     if (r == 0) return 1;
     int split = num_sms / r;
     if (split > 8) split = 8;
     if (split > n_kv) split = n_kv;
-    if (split < 2) return 1;
+    if (split < 2 || n_kv - (n_kv + split - 1) / split < min_saved) return 1;
     n_full = units - r;
     return split;
 }
@@ -615,7 +624,7 @@ wdc_status launch(Ctx* c, const void* q, const void* k, const void* vt, int ldv,
     g.o = reinterpret_cast<__nv_bfloat16*>(o);
     g.err = c->err;
     g.units_s = Hs * g.q_blocks;
-    g.split = attn_split(g.units_s, c->num_sms, g.n_kv, g.n_full);
+    g.split = attn_split(g.units_s, c->num_sms, g.n_kv, kMinSaved<D>, g.n_full);
     // the workspace holds num_sms part CTAs per sample of the model's batch
     if (!c->attn_part || g.nb > c->attn_part_samples) g.split = 1;
     if (g.split == 1) g.n_full = g.units_s;
