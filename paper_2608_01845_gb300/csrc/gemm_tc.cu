@@ -3,7 +3,7 @@
 // fp32 accumulation in tensor memory.
 //
 // Three kernels, 6 warps a CTA (TMA producer, MMA issuer, 4 epilogue warps):
-//   gemm_tc2_kernel   persistent, CTA pairs, 256 x 256 tiles: shapes with
+//   gemm_tc2_kernel   persistent, CTA pairs, 256 x 256, 192 or 128 tiles: shapes with
 //                     tiles for (nearly) every pair;
 //   gemm_tc_kernel    persistent, one CTA a tile of 128 x 128 or 128 x 64:
 //                     shapes that would leave most pairs without a tile;
@@ -41,7 +41,7 @@ namespace wdc {
 
 namespace {
 
-constexpr int BM = 128, BN = 256, BK = 64;
+constexpr int BM = 128, BK = 64;
 constexpr int kGemmThreads = 192;
 constexpr uint32_t A_BYTES = BM * BK * 2;
 // Epilogue staging: two slabs of 32 rows x 64 bf16 columns (128-byte rows,
@@ -629,14 +629,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 // stages and accumulators.  The pair allocation is collective (both CTAs receive the same TMEM base; the
 // leader's base is used for every access and a mismatch is reported), and two
 // 256-column accumulators let a tile's epilogue overlap the next tile's MMAs.
-constexpr int STAGES2 = 6;
+// The tile's width BNP may also be 192 or 128: a round of narrower tiles is
+// shorter, which pays where whole rounds of 256 leave many pairs idle.
 constexpr uint32_t A2_BYTES = 128 * BK * 2;
-constexpr uint32_t B2_BYTES = 128 * BK * 2;                  // half of the 256-row W tile
-constexpr uint32_t STAGE2_BYTES = A2_BYTES + B2_BYTES;
 constexpr uint32_t TMEM2_COLS = 512;
-constexpr uint32_t IDESC2 = idesc_bf16(256, 256);
-constexpr size_t SMEM2_BYTES = STAGES2 * STAGE2_BYTES + STAGING_BYTES + 1024 + 512;
-static_assert(SMEM2_BYTES <= 227 * 1024, "shared memory per CTA");
+template <int BNP>
+struct PairCfg {
+    static constexpr int STAGES = BNP == 128 ? 8 : 6;
+    static constexpr uint32_t B_BYTES = BNP / 2 * BK * 2;    // half of the W tile's rows
+    static constexpr uint32_t STAGE_BYTES = A2_BYTES + B_BYTES;
+    static constexpr uint32_t IDESC = idesc_bf16(256, BNP);
+    static constexpr size_t SMEM = STAGES * STAGE_BYTES + STAGING_BYTES + 1024 + 512;
+    static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
+    static_assert(B_BYTES % 1024 == 0 && BNP % 64 == 0, "swizzled tiles of whole 64-column chunks");
+};
 
 // Pair-kernel raster: the N tiles are split into groups of group_n; inside a
 // group the tiles run N-fastest over every 256-row M block.  A group's slab
@@ -667,18 +673,21 @@ __device__ __forceinline__ int grouped_tile(const GemmArgs& g, int m_pairs0, int
     return 1;
 }
 
-template <int FORM>
+template <int BNP, int FORM>
 __global__ void __launch_bounds__(kGemmThreads, 1)
     gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1,
                     const __grid_constant__ EpiMaps maps, const __grid_constant__ EpiMaps maps1,
                     const __grid_constant__ GemmArgs g) {
+    using C = PairCfg<BNP>;
+    constexpr int STAGES = C::STAGES;
+    constexpr uint32_t STAGE_BYTES = C::STAGE_BYTES;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* staging = smem + STAGES2 * STAGE2_BYTES;
+    uint8_t* staging = smem + STAGES * STAGE_BYTES;
     uint64_t* full = reinterpret_cast<uint64_t*>(staging + STAGING_BYTES);   // even CTA: both halves landed
-    uint64_t* empty = full + STAGES2;
-    uint64_t* tfull = empty + STAGES2;         // [2]
+    uint64_t* empty = full + STAGES;
+    uint64_t* tfull = empty + STAGES;         // [2]
     uint64_t* tempty = tfull + 2;              // [2] even CTA: both CTAs' epilogues are done
     uint64_t* mma_done = tempty + 2;
     uint64_t* rbars = mma_done + 1;            // [4 warps][2] residual slabs
@@ -692,7 +701,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     const int tiles0 = m_pairs * g.n_tiles;
     const int num_tiles = tiles0 + (g.nprob > 1 ? ((g.m_tiles1 + 1) >> 1) * g.n_tiles : 0);
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES2; ++s) {
+        for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -740,25 +749,25 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 const CUtensorMap* mA = prob ? &tmA1 : &tmA;
                 const CUtensorMap* mB = prob ? &tmB1 : &tmB;
                 const int m0 = mb * 256 + (int)rank * 128;
-                const int n0 = nb * BN + (int)rank * 128;
+                const int n0 = nb * BNP + (int)rank * (BNP / 2);
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.err)) { ok = false; break; }
                     if (elect_one()) {
-                        if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * STAGE2_BYTES);
+                        if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * STAGE_BYTES);
                         const uint32_t fb = mapa_shared(smem_u32(&full[stage]), 0);
-                        uint8_t* sa = smem + stage * STAGE2_BYTES;
+                        uint8_t* sa = smem + stage * STAGE_BYTES;
                         tma_load_2d_pair(sa, mA, fb, kb * BK, m0);
                         tma_load_2d_pair(sa + A2_BYTES, mB, fb, kb * BK, n0);
                     }
                     __syncwarp();
                     armed |= 1u << stage;
                     parity = (parity & ~(1u << stage)) | (phase << stage);
-                    if (++stage == STAGES2) { stage = 0; phase ^= 1u; }
+                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
             }
             // drain: every copy of the pair has landed (even CTA's full) and the
             // MMAs have released every stage (both CTAs' empty)
-            for (int s = 0; s < STAGES2; ++s) {
+            for (int s = 0; s < STAGES; ++s) {
                 if (!((armed >> s) & 1)) continue;
                 if (rank == 0) {
                     const unsigned long long t0 = globaltimer();
@@ -782,20 +791,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             for (int tile = cluster_id; tile < num_tiles && ok; tile += n_clusters) {
                 if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, g.err)) break;
                 tc_fence_after();
-                const uint32_t d = tmem + (uint32_t)(acc * BN);
+                const uint32_t d = tmem + (uint32_t)(acc * 256);
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
                     if (!mbar_wait(&full[stage], phase, abort_flag, g.err)) { ok = false; break; }
                     tc_fence_after();
                     if (elect_one()) {
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k)
-                            tc_mma2(d, sdesc_at(da, stage * STAGE2_BYTES + k * 32), sdesc_at(db, stage * STAGE2_BYTES + k * 32),
-                                    IDESC2, (kb | k) != 0);
+                            tc_mma2(d, sdesc_at(da, stage * STAGE_BYTES + k * 32), sdesc_at(db, stage * STAGE_BYTES + k * 32),
+                                    C::IDESC, (kb | k) != 0);
                         tc_commit2_mc(&empty[stage], (uint16_t)0x3);
                         if (kb + 1 == g.k_blocks) tc_commit2_mc(&tfull[acc], (uint16_t)0x3);
                     }
                     __syncwarp();
-                    if (++stage == STAGES2) { stage = 0; phase ^= 1u; }
+                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
                 acc ^= 1;
                 if (acc == 0) acc_phase ^= 1u;
@@ -814,14 +823,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         for (int tile = cluster_id; tile < num_tiles; tile += n_clusters) {
             int mb, n_blk;
             const int prob = grouped_tile(g, m_pairs, tiles0, tile, mb, n_blk);
-            const int m0 = mb * 256 + (int)rank * 128 + lg * 32, n0 = n_blk * BN, end = min(n0 + BN, g.N);
+            const int m0 = mb * 256 + (int)rank * 128 + lg * 32, n0 = n_blk * BNP, end = min(n0 + BNP, g.N);
             const int Mp = prob ? g.M1 : g.M, staged = prob ? g.staged1 : g.staged;
             const EpiMaps* mp = prob ? &maps1 : &maps;
             const Epi e = problem_epilogue(g, prob);
             epilogue_prefetch<FORM>(e.bias, e.gate, staged, &mp->res, Mp, n0, end, m0, ws, lane);
             if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, g.err)) break;
             tc_fence_after();
-            const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(acc * BN);
+            const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(acc * 256);
             auto release = [&] {
                 tc_fence_before();
                 __syncwarp();
@@ -1183,12 +1192,15 @@ using TileKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensor
 using SplitKernel = void (*)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const GemmArgs);
 template <int... F>
 struct Tables {
-    static constexpr TileKernel pair[] = {gemm_tc2_kernel<F>...};
+    static constexpr TileKernel pair256[] = {gemm_tc2_kernel<256, F>...};
+    static constexpr TileKernel pair192[] = {gemm_tc2_kernel<192, F>...};
+    static constexpr TileKernel pair128[] = {gemm_tc2_kernel<128, F>...};
     static constexpr TileKernel one128[] = {gemm_tc_kernel<128, F>...};
     static constexpr TileKernel one64[] = {gemm_tc_kernel<64, F>...};
     static constexpr SplitKernel split2[] = {gemm_split_kernel<F, 2>...};
     static constexpr SplitKernel split4[] = {gemm_split_kernel<F, 4>...};
     static constexpr SplitKernel split8[] = {gemm_split_kernel<F, 8>...};
+    static TileKernel pair(int bn, int f) { return bn == 256 ? pair256[f] : (bn == 192 ? pair192[f] : pair128[f]); }
     static SplitKernel split(int S, int f) { return S == 2 ? split2[f] : (S == 4 ? split4[f] : split8[f]); }
 };
 using Kernels = Tables<kFormStore, kFormGelu, kFormResid, kFormQKV, kFormUnpatch>;
@@ -1202,6 +1214,10 @@ int form_of(const Epi& e) {
     }
 }
 
+size_t pair_smem(int bn) {
+    return bn == 256 ? PairCfg<256>::SMEM : (bn == 192 ? PairCfg<192>::SMEM : PairCfg<128>::SMEM);
+}
+
 void set_attrs() {
     static bool attr_set = false;
     if (!attr_set) {
@@ -1209,7 +1225,7 @@ void set_attrs() {
             cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         };
         for (int f = 0; f < kForms; ++f) {
-            smem((const void*)Kernels::pair[f], SMEM2_BYTES);
+            for (int bn : {256, 192, 128}) smem((const void*)Kernels::pair(bn, f), pair_smem(bn));
             smem((const void*)Kernels::one128[f], GemmCfg<128>::SMEM);
             smem((const void*)Kernels::one64[f], GemmCfg<64>::SMEM);
             for (int S = 2; S <= SPLIT_MAX; S *= 2) smem((const void*)Kernels::split(S, f), SPLIT_SMEM);
@@ -1221,6 +1237,7 @@ void set_attrs() {
 // One launch: the kernel, its N tile and (split kernel) the CTAs a tile.
 struct Choice {
     enum Kind { kPair, kOne128, kOne64, kSplit } kind;
+    int bn = 256;
     int split = 1;
 };
 
@@ -1233,22 +1250,28 @@ double launch_cycles(long long tiles, int units, double main, double epi) {
 
 // The kernel for a shape is the one with the least estimated cycles; the
 // constants are fits to a sweep (us, store unless said; kb = 64-column blocks):
-//                             pair  one128  one64  split 2 / 4 / 8
-//   272 x 256 x 256 resid      8.8     5.3    4.4    6.1 / 6.5
-//   272 x 256 x 1024 resid    12.1     8.3    7.1    7.4 / 7.2 / 7.4
-//   226 x 3072 x 3072                 15.1   14.2   10.3 / 16.2 / 28.9
-//   64 x 3072 x 8192                  33.7   31.3   17.6 / 12.3 / 18.9
-//   700 x 1024 x 1024 resid   12.2     8.4    7.3    7.6 / 13.8
-//   1600 x 1024 x 4096 resid  25.0    20.1   32.3   23.7 / 28.9
-//   1600 x 3072 x 1024        14.7    15.9   21.9   29.2
-//   6400 x 1024 x 4096 resid  44.6    51.5   90.3   73.8
-// A block of K takes a pair 560 cycles (256 x 256), one CTA 470 (128 x 128) or
-// 450 (128 x 64): a launch of few tiles takes as long in either, so the
-// narrow tile wins where it still fits one wave.  The pair's cluster launch and
-// wider tile cost 1900 more to start; the split kernel's two cluster barriers,
-// exchange and epilogue 4300-6200, and it runs as many clusters at a time as
-// the GPCs hold (76, 36 and 15 of 2, 4 and 8 on this part).
-constexpr double kCyclesPair = 560.0, kCycles128 = 470.0, kCycles64 = 450.0, kCyclesSplit = 440.0, kPairStart = 1900.0;
+//                          pair 256   192   128  one128  one64  split 2 / 4
+//   272 x 768 x 256             7.1   6.5   5.9     4.7    4.1    5.3 / 6.1
+//   272 x 256 x 1024 resid     12.1                 8.3    7.1    7.4 / 7.2
+//   226 x 3072 x 3072                              15.1   14.2   10.3 / 16.2
+//   64 x 3072 x 8192                               33.7   31.3   17.6 / 12.3
+//   700 x 1024 x 1024 resid    12.2  10.2   8.7     8.4    7.3    7.6 / 13.5
+//   1600 x 1024 x 4096 resid   25.1  20.4  17.2    20.3   32.3   23.2 / 28.3
+//   1600 x 3072 x 1024         14.6  12.9  13.8    16.1   21.8   28.6
+//   6400 x 1024 x 4096 resid   44.0  37.0  40.9    51.5   90.4   70.3
+//   3000 x 3072 x 3072         33.0  35.8  38.8    51.0   89.7   71.9
+//   13568 x 3072 x 12288 res    591   613   715     852   1445    889
+// A block of K takes a pair 560, 460 or 400 cycles (256 x 256, 192 or 128; the
+// narrower, the less of it are MMAs), one CTA 470 (128 x 128) or 450 (128 x
+// 64): the widest tile is the most efficient, a narrower one wins where its
+// rounds fit the tiles better (6400 x 1024: 100 tiles of 256 on 76 pairs are
+// two rounds, of which the second is a third full; 150 of 192 fill both), and
+// a launch of few tiles takes as long in a narrow one.  The pair's cluster
+// launch and wider tile cost 1900 more to start; the split kernel's two cluster
+// barriers, exchange and epilogue 4300-6200, and it runs as many clusters at a
+// time as the GPCs hold (76, 36 and 15 of 2, 4 and 8 on this part).
+constexpr double kCyclesPair = 560.0, kCyclesPair192 = 460.0, kCyclesPair128 = 400.0, kPairStart = 1900.0;
+constexpr double kCycles128 = 470.0, kCycles64 = 450.0, kCyclesSplit = 440.0;
 
 // Clusters of `size` CTAs of a GEMM kernel resident at a time.
 int resident_clusters(const Ctx* c, const void* kernel, int size, size_t smem) {
@@ -1276,7 +1299,7 @@ int split_clusters(const Ctx* c, int S) {
 }
 int pair_clusters(const Ctx* c) {
     static int cap = 0;
-    if (cap == 0) cap = resident_clusters(c, (const void*)Kernels::pair[0], 2, SMEM2_BYTES);
+    if (cap == 0) cap = resident_clusters(c, (const void*)Kernels::pair(256, 0), 2, pair_smem(256));
     return cap < c->num_sms / 2 ? cap : c->num_sms / 2;
 }
 
@@ -1290,26 +1313,28 @@ Choice choose_gemm(Ctx* c, int form, int M, int M1, int sample, int sample1, int
     auto tiles = [&](int rows, int rows1, int bm, int bn) {
         return (long long)((rows + bm - 1) / bm + (rows1 + bm - 1) / bm) * ((N + bn - 1) / bn);
     };
-    auto whole = [&](int rows, int rows1, Choice::Kind* kind) {
-        double best = launch_cycles(tiles(rows, rows1, BM, 64), sms, kb * kCycles64, chunk);
-        *kind = Choice::kOne64;
-        const double one128 = launch_cycles(tiles(rows, rows1, BM, 128), sms, kb * kCycles128, 2 * chunk);
-        if (one128 < best) {
-            best = one128;
-            *kind = Choice::kOne128;
-        }
+    auto whole = [&](int rows, int rows1, Choice* ch) {
+        double best = 0;
+        auto offer = [&](Choice::Kind kind, int bn, double est) {
+            if (best > 0 && est >= best) return;
+            best = est;
+            ch->kind = kind;
+            ch->bn = bn;
+        };
+        offer(Choice::kOne64, 64, launch_cycles(tiles(rows, rows1, BM, 64), sms, kb * kCycles64, chunk));
+        offer(Choice::kOne128, 128, launch_cycles(tiles(rows, rows1, BM, 128), sms, kb * kCycles128, 2 * chunk));
         if (rows >= 256 && sms >= 2) {
-            const double pair =
-                kPairStart + launch_cycles(tiles(rows, rows1, 256, BN), sms / 2, kb * kCyclesPair, 4 * chunk);
-            if (pair < best) {
-                best = pair;
-                *kind = Choice::kPair;
+            const double cycles[3] = {kCyclesPair, kCyclesPair192, kCyclesPair128};
+            for (int i = 0; i < 3; ++i) {
+                const int bn = 256 - 64 * i;
+                offer(Choice::kPair, bn,
+                      kPairStart + launch_cycles(tiles(rows, rows1, 256, bn), sms / 2, kb * cycles[i], bn / 64 * chunk));
             }
         }
         return best;
     };
     Choice ch{Choice::kPair};
-    double least = 0.9 * whole(sample, sample1, &ch.kind);    // (a split that gains less is not worth its risk)
+    double least = 0.9 * whole(sample, sample1, &ch);         // (a split that gains less is not worth its risk)
     const long long t = tiles(sample, sample1, BM, SPLIT_BN);
     for (int S = 2; S <= SPLIT_MAX && 2 * S <= kb; S *= 2) {
         const int cap = split_clusters(c, S);
@@ -1318,10 +1343,11 @@ Choice choose_gemm(Ctx* c, int form, int M, int M1, int sample, int sample1, int
         if (est < least) {
             least = est;
             ch.kind = Choice::kSplit;
+            ch.bn = SPLIT_BN;
             ch.split = S;
         }
     }
-    if (ch.kind != Choice::kSplit) whole(M, M1, &ch.kind);
+    if (ch.kind != Choice::kSplit) whole(M, M1, &ch);
     return ch;
 }
 
@@ -1362,9 +1388,9 @@ wdc_status launch_gemm(Ctx* c, const Problem& p0, const Problem* p1, int N, int 
     set_attrs();
     const int form = form_of(*p0.e);
     const Choice ch = choose_gemm(c, form, p0.M, p1 ? p1->M : 0, p0.sample, p1 ? p1->sample : 0, N, K);
-    const int bn = ch.kind == Choice::kPair ? BN : (ch.kind == Choice::kOne64 ? 64 : 128);
+    const int bn = ch.bn;
     // W's box: the tile's width, or each CTA's half of it in a pair
-    const uint32_t w_rows = ch.kind == Choice::kPair ? BN / 2 : bn;
+    const uint32_t w_rows = ch.kind == Choice::kPair ? bn / 2 : bn;
     GemmArgs g{};
     g.M = p0.M;
     g.N = N;
@@ -1379,7 +1405,7 @@ wdc_status launch_gemm(Ctx* c, const Problem& p0, const Problem* p1, int N, int 
     // 17776 x 3072 x 12288 MLP-down GEMM): plain N-fastest order there.
     g.group_n = g.n_tiles;
     if (K <= 4096) {
-        const double slab_per_tile = 256.0 * K * 2.0;
+        const double slab_per_tile = (double)bn * K * 2.0;
         int gn = (int)(40.0e6 / slab_per_tile);
         gn = gn < 1 ? 1 : (gn > g.n_tiles ? g.n_tiles : gn);
         const int groups = (g.n_tiles + gn - 1) / gn;
@@ -1412,8 +1438,8 @@ wdc_status launch_gemm(Ctx* c, const Problem& p0, const Problem* p1, int N, int 
             // a persistent grid of as many CTA pairs as can be resident,
             // capped by the tile count
             const int resident = pair_clusters(c), tiles = ((g.m_tiles + 1) / 2 + (g.m_tiles1 + 1) / 2) * g.n_tiles;
-            launch_kernel(Kernels::pair[form], dim3(2 * (tiles < resident ? tiles : resident)), kGemmThreads,
-                          SMEM2_BYTES, s, 2, ta, tb, ta1, tb1, maps, maps1, g);
+            launch_kernel(Kernels::pair(bn, form), dim3(2 * (tiles < resident ? tiles : resident)), kGemmThreads,
+                          pair_smem(bn), s, 2, ta, tb, ta1, tb1, maps, maps1, g);
             break;
         }
         case Choice::kSplit:
