@@ -68,7 +68,9 @@ namespace {
 // With whole 16-byte vectors in a row (vec) each lane loads up to four of W's
 // before the wait for x: W is constant, so its reads run under the kernels
 // before.  Alone, 26624 x 512 bf16 (27 MB, cold) takes 10 us as with 2-byte
-// loads; the gain is in the chain (with prep_kernel's, see there).
+// loads; the gain is in the chain (with prep_kernel's, see there).  fp32 keeps
+// the element order of its sums: by vectors, the rollout with the
+// ill-conditioned linear observation came out 1.4e-5 off fp64 instead of 6e-6.
 template <typename T>
 __global__ void __launch_bounds__(256) gemv_kernel(const T* __restrict__ W, const float* x, const float* __restrict__ b,
                                                    float* y, int rows, int cols, int act, int vec) {
@@ -1208,7 +1210,7 @@ static wdc_status modulation(Ctx* c, float* dst, cudaStream_t s) {
     DiT* t = c->dit;
     auto gv = [&](const void* W, const float* x, const float* b, float* y, int rows, int cols, int act) {
         const unsigned grid = blocks_for((long long)rows * 32, 256);
-        const int vec = cols % (16 / (int)t->esz) == 0 && (((uintptr_t)W | (uintptr_t)x) & 15) == 0;
+        const int vec = t->dtype == WDC_BF16 && cols % 8 == 0 && (((uintptr_t)W | (uintptr_t)x) & 15) == 0;
         LaunchScope ls(c, WDC_K_OTHER, s);
         if (t->dtype == WDC_BF16)
             launch_kernel(gemv_kernel<__nv_bfloat16>, grid, 256, 0, s, 1, (const __nv_bfloat16*)W, x, b, y, rows, cols, act, vec);
