@@ -80,6 +80,10 @@ struct AttnCfg {
     static constexpr uint32_t K_TILE = BK * D * 2;
     static constexpr uint32_t V_TILE = D * BK * 2;
     static constexpr uint32_t STAGE = K_TILE + V_TILE;      // 32 KB for both head sizes
+    // steps from which tile 1 starts behind tile 0: a single step of 128 keys is
+    // longer for it (4 heads, L = 30: 5.73 us, 5.30 together), two are not (L =
+    // 130: 6.61 behind, 6.72 together), nor one of 64 (5.4 and 5.4 - 5.6)
+    static constexpr int STAGGER_FROM = D == 64 ? 2 : 1;
     static constexpr int STAGES = 5;
     static constexpr uint32_t SMEM = 2 * Q_TILE + STAGES * STAGE + 1024 + 256;
     static constexpr uint32_t TMEM_COLS = 512;
@@ -305,7 +309,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
                               (acc || ks != 0) ? 1u : 0u);
                 }
             };
-            if (ok && t == 1) ok = mbar_wait(stagger, 0, abort_flag, g.err);
+            if (ok && t == 1 && nj >= C::STAGGER_FROM) ok = mbar_wait(stagger, 0, abort_flag, g.err);
             if (ok) ok = mbar_wait(&kv_full[0], 0, abort_flag, g.err);
             for (int j = 0; j < nj && ok; ++j) {
                 // here K(j) has landed, and S(t, j - 1) is in the softmax's registers
