@@ -66,8 +66,8 @@ namespace {
 // y[r] = act(W[r,:] . x + b[r]); one warp per row.  act: 0 none, 1 SiLU.
 // Bound by the latency of its loads (E x E) or by reading W (the modulation).
 // With whole 16-byte vectors in a row (vec) each lane loads up to four of W's
-// before the wait for x: W is constant, so its reads run under the kernels
-// before.  Alone, 26624 x 512 bf16 (27 MB, cold) takes 10 us as with 2-byte
+// before the wait for x: weights change only in calls that synchronise with the
+// device before they return, so W's reads run under the kernels before.  Alone, 26624 x 512 bf16 (27 MB, cold) takes 10 us as with 2-byte
 // loads; the gain is in the chain (with prep_kernel's, see there).  fp32 keeps
 // the element order of its sums: by vectors, the rollout with the
 // ill-conditioned linear observation came out 1.4e-5 off fp64 instead of 6e-6.
