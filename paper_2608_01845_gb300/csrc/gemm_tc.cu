@@ -110,11 +110,17 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t u) {
 
 // Epilogue forms; each is its own instantiation of the kernels, so that the
 // epilogue's code stays small and without branches on the form.
-enum Form { kFormStore = 0, kFormGelu = 1, kFormResid = 2, kFormQKV = 3, kFormUnpatch = 4, kFormResidRepeat = 5, kForms = 6 };
+enum Form {
+    kFormStore = 0, kFormGelu = 1, kFormResid = 2, kFormQKV = 3, kFormUnpatch = 4, kFormResidGelu = 5,
+    kFormResidRepeat = 6, kForms = 7
+};
+// kFormResidGelu: a residual over GELU's result, an operator call's only (the
+// blocks apply GELU before another GEMM).
 // kFormResidRepeat: a residual whose rows repeat every e.res_rows (a batch's
 // position embedding).  Its index arithmetic in kFormResid cost the small
 // launches 0.1 us each.
-constexpr bool is_resid(int form) { return form == kFormResid || form == kFormResidRepeat; }
+constexpr bool is_resid(int form) { return form == kFormResid || form == kFormResidGelu || form == kFormResidRepeat; }
+constexpr bool has_gelu(int form) { return form == kFormGelu || form == kFormResidGelu; }
 
 // Direct epilogue of 32 consecutive columns col0..col0+31 of one row: the
 // unpatchify form, and the rows whose slab cannot be moved by one TMA copy.
@@ -134,6 +140,10 @@ __device__ __forceinline__ void epilogue_chunk(const Epi& e, int m, int col0, co
     } else {
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+    }
+    if constexpr (has_gelu(FORM)) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = gelu_tanh_f(v[j]);
     }
     if constexpr (is_resid(FORM)) {
         __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(e.out) + (size_t)m * e.ldo + col0;
@@ -399,7 +409,7 @@ __device__ __forceinline__ bool epilogue_tile(const Epi& e, int staged, const Ep
                         v[hb][i][2] += ws.bias[i].x; v[hb][i][3] += ws.bias[i].y;
                     }
             }
-            if constexpr (FORM == kFormGelu) {
+            if constexpr (has_gelu(FORM)) {
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
 #pragma unroll
@@ -918,7 +928,7 @@ __device__ __forceinline__ void columns8(const Epi& e, int col, float (&bias)[8]
         x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
     };
     load(e.bias, 0.f, bias);
-    if (FORM == kFormResid) load(e.gate, 1.f, gate);
+    if (is_resid(FORM)) load(e.gate, 1.f, gate);
 }
 
 // Epilogue of 8 consecutive columns (one 16-byte store) of row m.
@@ -934,7 +944,7 @@ __device__ __forceinline__ void epilogue8(const Epi& e, int m, int col, float (&
         for (int j = 0; j < 8; ++j) epi_apply<__nv_bfloat16>(plain, m, col + j, v[j]);
         return;
     }
-    if constexpr (FORM == kFormGelu) {
+    if constexpr (has_gelu(FORM)) {
 #pragma unroll
         for (int j = 0; j < 8; ++j) v[j] = gelu_tanh_f(v[j]);
     }
@@ -956,7 +966,7 @@ __device__ __forceinline__ void epilogue8(const Epi& e, int m, int col, float (&
     } else {
         dst = reinterpret_cast<__nv_bfloat16*>(e.out) + (size_t)m * e.ldo + col;
     }
-    if constexpr (FORM == kFormResid) {
+    if constexpr (is_resid(FORM)) {
         const uint32_t w[4] = {rr.x, rr.y, rr.z, rr.w};
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
@@ -1075,8 +1085,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         grp = kByRow ? i : tid % NG;
     };
     // residual rows, bias and gate are fetched before the barriers
-    uint4 resid[FORM == kFormResid ? NG : 1];
-    if (FORM == kFormResid && warp >= 2) {
+    uint4 resid[is_resid(FORM) ? NG : 1];
+    if (is_resid(FORM) && warp >= 2) {
 #pragma unroll
         for (int i = 0; i < NG; ++i) {
             int row, grp;
@@ -1137,7 +1147,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 }
             }
             if (kByRow) columns8<FORM>(e, min(col, g.N - 8), bias, gate);
-            if (m < Mp && col < g.N) epilogue8<FORM>(e, m, col, v, bias, gate, resid[FORM == kFormResid ? i : 0]);
+            if (m < Mp && col < g.N) epilogue8<FORM>(e, m, col, v, bias, gate, resid[is_resid(FORM) ? i : 0]);
         }
     }
 }
@@ -1223,8 +1233,8 @@ struct SplitKernels {
     static constexpr SplitKernel split4[] = {gemm_split_kernel<F, 4>...};
     static constexpr SplitKernel split8[] = {gemm_split_kernel<F, 8>...};
 };
-struct Kernels : TileKernels<kFormStore, kFormGelu, kFormResid, kFormQKV, kFormUnpatch, kFormResidRepeat>,
-                 SplitKernels<kFormStore, kFormGelu, kFormResid, kFormQKV, kFormUnpatch> {
+struct Kernels : TileKernels<kFormStore, kFormGelu, kFormResid, kFormQKV, kFormUnpatch, kFormResidGelu, kFormResidRepeat>,
+                 SplitKernels<kFormStore, kFormGelu, kFormResid, kFormQKV, kFormUnpatch, kFormResidGelu> {
     static TileKernel pair(int bn, int f) { return bn == 256 ? pair256[f] : (bn == 192 ? pair192[f] : pair128[f]); }
     static SplitKernel split(int S, int f) {
         if (f == kFormResidRepeat) f = kFormResid;         // reads its residual row by row, repeating or not
@@ -1234,7 +1244,9 @@ struct Kernels : TileKernels<kFormStore, kFormGelu, kFormResid, kFormQKV, kFormU
 
 int form_of(const Epi& e, int M) {
     switch (e.mode) {
-        case kEpiResid: return e.res_rows > 0 && M > e.res_rows ? kFormResidRepeat : kFormResid;
+        case kEpiResid:       // (repeating rows come from the patch embedding alone, without GELU)
+            if (e.gelu) return kFormResidGelu;
+            return e.res_rows > 0 && M > e.res_rows ? kFormResidRepeat : kFormResid;
         case kEpiQKV: return kFormQKV;
         case kEpiUnpatch: return kFormUnpatch;
         default: return e.gelu ? kFormGelu : kFormStore;

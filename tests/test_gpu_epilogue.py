@@ -123,3 +123,31 @@ def test_forward_split_k(Lc, dual, d):
         assert torch.equal(one[b], many[b])
     want = dit.forward(W, DiTConfig(**cfgd), z[0], 600.0, ct[0])
     assert rel_l2(one[0].cpu().numpy(), want) <= 2e-2
+
+
+@pytest.mark.parametrize("M,N,K", [(257, 96, 72), (129, 6176, 520),                              # one CTA a tile: 64, 128 columns
+                                   (226, 3072, 3072), (200, 1056, 1544), (257, 160, 4104),       # 2, 4, 8 CTAs a tile
+                                   (1600, 1024, 2048), (513, 4128, 520), (257, 7328, 1032)])     # pairs: 128, 192, 256 columns
+@pytest.mark.parametrize("dtype", [wdc.BF16, wdc.F32])
+@pytest.mark.parametrize("in_place", [False, True])
+def test_gemm_gelu_then_gated_residual(M, N, K, dtype, in_place):
+    """C = res + gate * GELU(A W^T + bias), both options of one call, in every
+    kernel of both dtypes.  bf16 as above; fp32: sums of K terms and the
+    hardware exponential of GELU (2^-22 relative of a factor below one) against
+    2^-24 a rounding."""
+    ctx = wdc.Context(wdc.make_config(dtype=dtype, **MODEL), 2)
+    td = torch.bfloat16 if dtype == wdc.BF16 else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    r = lambda *s: torch.randn(*s, device="cuda", generator=g)
+    A, W, b, R, gate = r(M, K).to(td), (r(N, K) * K ** -0.5).to(td), r(N), r(M, N).to(td), r(N)
+    x = A.double() @ W.double().T + b.double()
+    want = R.double() + gate.double() * 0.5 * x * (1 + torch.tanh((2 / np.pi) ** 0.5 * (x + 0.044715 * x ** 3)))
+    buf = torch.full((M + 40, N), 7.0, dtype=td, device="cuda")
+    if in_place:
+        buf[:M] = R
+    ctx.op_gemm(A, W, buf[:M], bias=b, gelu=True, res=buf[:M] if in_place else R, gate=gate)
+    torch.cuda.synchronize()
+    assert ctx.device_errors() == 0
+    err = float((buf[:M].double() - want).norm() / want.norm())
+    assert err <= (2.0 ** -8 if dtype == wdc.BF16 else 2.0 ** -20) + K * 2.0 ** -22
+    assert bool((buf[M:] == 7.0).all())
