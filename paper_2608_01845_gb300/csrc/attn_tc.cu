@@ -595,19 +595,18 @@ wdc_status launch(Ctx* c, const void* q, const void* k, const void* vt, int ldv,
                   int Lc, cudaStream_t s) {
     using Cf = AttnCfg<D>;
     constexpr int BKV = Cf::BK;
-    static bool attr = false;
-    static bool regs_ok = false;
-    if (!attr) {
-        cudaFuncSetAttribute(attn_tc_kernel<D, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cf::SMEM);
+    static PerDevice<bool> fits;
+    const bool regs_ok = fits.get(c->device, [](bool& ok) {
+        const bool smem = allow_smem(attn_tc_kernel<D, BATCH>, Cf::SMEM);
         // the warpgroups' register requests must fit the launch allocation,
         // or setmaxnreg.inc would wait forever: refuse to launch otherwise
         cudaFuncAttributes fa;
-        regs_ok = cudaFuncGetAttributes(&fa, attn_tc_kernel<D, BATCH>) == cudaSuccess &&
-                  fa.maxThreadsPerBlock >= Cf::THREADS &&
-                  (uint32_t)fa.numRegs * Cf::THREADS >= 128 * Cf::REGS_CONTROL + 256 * Cf::REGS_SOFTMAX;
+        ok = cudaFuncGetAttributes(&fa, attn_tc_kernel<D, BATCH>) == cudaSuccess &&
+             fa.maxThreadsPerBlock >= Cf::THREADS &&
+             (uint32_t)fa.numRegs * Cf::THREADS >= 128 * Cf::REGS_CONTROL + 256 * Cf::REGS_SOFTMAX;
         cudaGetLastError();
-        attr = true;
-    }
+        return smem && ok;
+    });
     if (!regs_ok) return fail(c, WDC_ERR_UNSUPPORTED, "attention kernel's register allocation is below its warpgroup split");
     CUtensorMap tq, tk, tv;
     std::string why;

@@ -815,12 +815,8 @@ void launch_ln_mod(const Ctx* c, const void* x, void* h, int r0, int r1, int D, 
                             ((uintptr_t)shift & 15) == 0 && ((uintptr_t)scale & 15) == 0;
         if (vec_ok && D == 3072) {
             constexpr size_t ring_bytes = (size_t)kLnWarps * kLnRing * 12 * 32 * sizeof(uint4);
-            static bool attr = false;
-            if (!attr) {
-                cudaFuncSetAttribute(ln_mod_stream_kernel<12>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)ring_bytes);
-                attr = true;
-            }
+            static PerDevice<bool> attr;
+            attr.get(c->device, [](bool& ok) { return ok = allow_smem(ln_mod_stream_kernel<12>, ring_bytes); });
             const int blocks = (rows + kLnWarps - 1) / kLnWarps;
             const unsigned g = (unsigned)(blocks < num_sms ? blocks : num_sms);
             launch_kernel(ln_mod_stream_kernel<12>, g, kLnWarps * 32, ring_bytes, s, 1, xp, hp, r0, r1, D, shift, scale, h_row_off);
@@ -864,14 +860,11 @@ static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int nb, int 
         launch_kernel(gemm_simt_kernel<float>, grid, 256, 0, s, 1, a, w, M, N, K, e);
         return WDC_OK;
     }
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(gemm_simt_tile_kernel<64, 8, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SimtLarge::SMEM);
-        cudaFuncSetAttribute(gemm_simt_tile_kernel<16, 4, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SimtSmall::SMEM);
-        attr = true;
-    }
+    static PerDevice<bool> attr;
+    attr.get(c->device, [](bool& ok) {
+        return ok = allow_smem(gemm_simt_tile_kernel<64, 8, 2>, SimtLarge::SMEM) &&
+                    allow_smem(gemm_simt_tile_kernel<16, 4, 1>, SimtSmall::SMEM);
+    });
     // the shape with the fewer cycles an element of k: 66 for each 64 x 64 tile
     // of the busiest SM; 28 for a 16 x 32 one alone, 13.4 each for several (600
     // x 1536 x 512: 38 us by the large shape, 48 by the small one; 272 x 256 x
@@ -918,12 +911,11 @@ static wdc_status attention(Ctx* c, const void* q, const void* k, const void* vt
     dim3 grid(blocks_for(L, kAttnRows), H);
     const float scale = 1.0f / sqrtf((float)d);
     const int nb = H / Hs;
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(attn_simt_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttnSimt<64>::SMEM);
-        cudaFuncSetAttribute(attn_simt_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttnSimt<128>::SMEM);
-        attr = true;
-    }
+    static PerDevice<bool> attr;
+    attr.get(c->device, [](bool& ok) {
+        return ok = allow_smem(attn_simt_kernel<64>, AttnSimt<64>::SMEM) &&
+                    allow_smem(attn_simt_kernel<128>, AttnSimt<128>::SMEM);
+    });
     const int wide = (((uintptr_t)q | (uintptr_t)k) & 15) == 0;
     const int wide_v = ((uintptr_t)vt & 15) == 0 && ldv % 4 == 0 && L % 4 == 0;
     const float *qf = (const float*)q, *kf = (const float*)k, *vf = (const float*)vt;

@@ -1257,20 +1257,18 @@ size_t pair_smem(int bn) {
     return bn == 256 ? PairCfg<256>::SMEM : (bn == 192 ? PairCfg<192>::SMEM : PairCfg<128>::SMEM);
 }
 
-void set_attrs() {
-    static bool attr_set = false;
-    if (!attr_set) {
-        auto smem = [](const void* f, size_t bytes) {
-            cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        };
+void set_attrs(const Ctx* c) {
+    static PerDevice<bool> attr;
+    attr.get(c->device, [](bool& ok) {
+        ok = true;
         for (int f = 0; f < kForms; ++f) {
-            for (int bn : {256, 192, 128}) smem((const void*)Kernels::pair(bn, f), pair_smem(bn));
-            smem((const void*)Kernels::one128[f], GemmCfg<128>::SMEM);
-            smem((const void*)Kernels::one64[f], GemmCfg<64>::SMEM);
-            for (int S = 2; S <= SPLIT_MAX; S *= 2) smem((const void*)Kernels::split(S, f), SPLIT_SMEM);
+            for (int bn : {256, 192, 128}) ok &= allow_smem(Kernels::pair(bn, f), pair_smem(bn));
+            ok &= allow_smem(Kernels::one128[f], GemmCfg<128>::SMEM);
+            ok &= allow_smem(Kernels::one64[f], GemmCfg<64>::SMEM);
+            for (int S = 2; S <= SPLIT_MAX; S *= 2) ok &= allow_smem(Kernels::split(S, f), SPLIT_SMEM);
         }
-        attr_set = true;
-    }
+        return ok;
+    });
 }
 
 // One launch: the kernel, its N tile and (split kernel) the CTAs a tile.
@@ -1312,8 +1310,9 @@ double launch_cycles(long long tiles, int units, double main, double epi) {
 constexpr double kCyclesPair = 560.0, kCyclesPair192 = 460.0, kCyclesPair128 = 400.0, kPairStart = 1900.0;
 constexpr double kCycles128 = 470.0, kCycles64 = 450.0, kCyclesSplit = 440.0;
 
-// Clusters of `size` CTAs of a GEMM kernel resident at a time.
-int resident_clusters(const Ctx* c, const void* kernel, int size, size_t smem) {
+// Fills in the clusters of `size` CTAs of a GEMM kernel resident at a time;
+// false where that could not be asked and n is as many as the SMs would hold.
+bool resident_clusters(const Ctx* c, const void* kernel, int size, size_t smem, int& n) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c->num_sms / size * size, 1, 1);
     cfg.blockDim = dim3(kGemmThreads, 1, 1);
@@ -1324,22 +1323,23 @@ int resident_clusters(const Ctx* c, const void* kernel, int size, size_t smem) {
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
-        cudaGetLastError();
-        n = c->num_sms / size > 0 ? c->num_sms / size : 1;
-    }
-    return n;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1) return true;
+    cudaGetLastError();
+    n = c->num_sms / size > 0 ? c->num_sms / size : 1;
+    return false;
 }
 int split_clusters(const Ctx* c, int S) {
-    static int cap[SPLIT_MAX + 1] = {};
-    if (cap[S] == 0) cap[S] = resident_clusters(c, (const void*)Kernels::split(S, 0), S, SPLIT_SMEM);
-    return cap[S];
+    static PerDevice<int> cap[SPLIT_MAX + 1];
+    return cap[S].get(c->device, [&](int& n) {
+        return resident_clusters(c, (const void*)Kernels::split(S, 0), S, SPLIT_SMEM, n);
+    });
 }
 int pair_clusters(const Ctx* c) {
-    static int cap = 0;
-    if (cap == 0) cap = resident_clusters(c, (const void*)Kernels::pair(256, 0), 2, pair_smem(256));
-    return cap < c->num_sms / 2 ? cap : c->num_sms / 2;
+    static PerDevice<int> cap;
+    const int n = cap.get(c->device, [&](int& v) {
+        return resident_clusters(c, (const void*)Kernels::pair(256, 0), 2, pair_smem(256), v);
+    });
+    return n < c->num_sms / 2 ? n : c->num_sms / 2;
 }
 
 // M, M1: the launch's rows (M1: a second problem's, or 0); sample, sample1:
@@ -1424,7 +1424,7 @@ wdc_status launch_gemm(Ctx* c, const Problem& p0, const Problem* p1, int N, int 
     wdc_status st = check_operands(c, p0.A, p0.W, *p0.e);
     if (!st && p1) st = check_operands(c, p1->A, p1->W, *p1->e);
     if (st) return st;
-    set_attrs();
+    set_attrs(c);
     const int form = form_of(*p0.e, p0.M);
     const Choice ch = choose_gemm(c, form, p0.M, p1 ? p1->M : 0, p0.sample, p1 ? p1->sample : 0, N, K);
     const int bn = ch.bn;

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "../../include/wdc.h"
+#include "per_device.h"
 
 namespace wdc {
 
@@ -237,6 +238,13 @@ __device__ __forceinline__ float4 ld_chain(const float4* p) {
     float4 v;
     asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
+}
+
+// Lets a kernel take `bytes` of dynamic shared memory on the current device; once
+// a device, see PerDevice.
+template <class... P>
+bool allow_smem(void (*kernel)(P...), size_t bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess;
 }
 
 template <class... P, class... A>
