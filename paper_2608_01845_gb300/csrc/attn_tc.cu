@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
             uint32_t phase = 0;
             uint32_t armed = 0, parity = 0;        // per stage: a copy was issued; its phase
             for (int j = j0; j < j0 + nj; ++j) {
-                if (!mbar_wait(&kv_empty[stage], phase ^ 1u, abort_flag, g.err)) break;
+                if (!mbar_wait_warp(&kv_empty[stage], phase ^ 1u, abort_flag, g.err)) break;
                 if (elect_one()) {
                     mbar_arrive_expect_tx(&kv_full[stage], C::STAGE);
                     uint8_t* sk = skv + stage * C::STAGE;
@@ -286,9 +286,16 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
             // this warp issues the MMAs of query tile t only; the other tile
             // has its own issuer, so neither waits behind the other's softmax
             const int t = warp - 1;
+            // d = 128: one lane runs the whole loop (1.44 -> 1.40 ms at 24 x
+            // 13568); d = 64: the warp does, and one lane issues (at 48 x 17776
+            // 3.03 ms, 3.24 with one lane)
+            constexpr bool kOneLane = D == 128;
+            auto leads = [] { return kOneLane || elect_one(); };
+            auto rejoin = [] { if (!kOneLane) __syncwarp(); };
+          if (!kOneLane || elect_one()) {
             const uint64_t dq = sdesc_sw128(smem_u32(sq) + t * C::Q_TILE);
             const uint64_t dk = sdesc_sw128(smem_u32(skv)), dv = sdesc_sw128(smem_u32(skv) + C::K_TILE);
-            bool ok = mbar_wait(q_full, 0, abort_flag, g.err);
+            bool ok = mbar_wait(q_full, 0, abort_flag, g.err);        // this lane's waits (elect_one)
             int stage = 0, prev = 0;
             uint32_t phase = 0;
             // S(t) = Q(t) K^T into TMEM (BK fp32 columns)
@@ -309,48 +316,48 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
                               (acc || ks != 0) ? 1u : 0u);
                 }
             };
-            if (ok && t == 1 && nj >= C::STAGGER_FROM) ok = mbar_wait(stagger, 0, abort_flag, g.err);
-            if (ok) ok = mbar_wait(&kv_full[0], 0, abort_flag, g.err);
-            for (int j = 0; j < nj && ok; ++j) {
+            if (t == 1 && nj >= C::STAGGER_FROM) ok = ok && mbar_wait(stagger, 0, abort_flag, g.err);
+            ok = ok && mbar_wait(&kv_full[0], 0, abort_flag, g.err);
+            for (int j = 0; j < nj; ++j) {
                 // here K(j) has landed, and S(t, j - 1) is in the softmax's registers
                 tc_fence_after();
-                if (elect_one()) {
+                if (leads() && ok) {
                     issue_s(stage);
                     tc_commit(&s_full[t]);
                 }
-                __syncwarp();
+                rejoin();
                 const int cur = stage;
                 if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
                 // the next step's K: awaited before P(t, j - 1) at d = 128
                 // (1.34 -> 1.31 ms at 24 x 13568), after it at d = 64, where
                 // waiting first keeps the two tiles' steps in phase (2.89 ->
                 // 2.95 ms at 48 x 17776)
-                auto next_k = [&]() { return j + 1 >= nj || mbar_wait(&kv_full[stage], phase, abort_flag, g.err); };
-                if (D == 128 && !next_k()) { ok = false; break; }
+                auto next_k = [&]() { if (j + 1 < nj) ok = ok && mbar_wait(&kv_full[stage], phase, abort_flag, g.err); };
+                if (D == 128) next_k();
                 if (j > 0) {
-                    if (!mbar_wait(&p_full[t], (j - 1) & 1, abort_flag, g.err)) { ok = false; break; }
+                    ok = ok && mbar_wait(&p_full[t], (j - 1) & 1, abort_flag, g.err);
                     tc_fence_after();
-                    if (elect_one()) {
+                    if (leads() && ok) {
                         issue_pv(prev, j > 1);
                         tc_commit(&p_free[t]);
                         tc_commit(&kv_empty[prev]);
                     }
-                    __syncwarp();
+                    rejoin();
                 }
                 prev = cur;
-                if (D == 64 && !next_k()) { ok = false; break; }
-                if (j + 1 < nj && !mbar_wait(&s_free[t], j & 1, abort_flag, g.err)) { ok = false; break; }
+                if (D == 64) next_k();
+                if (j + 1 < nj) ok = ok && mbar_wait(&s_free[t], j & 1, abort_flag, g.err);
             }
-            if (ok && mbar_wait(&p_full[t], (nj - 1) & 1, abort_flag, g.err)) {
-                tc_fence_after();
-                if (elect_one()) {
-                    issue_pv(prev, nj > 1);
-                    tc_commit(&kv_empty[prev]);
-                    tc_commit(&o_final[t]);
-                }
-                __syncwarp();
+            ok = ok && mbar_wait(&p_full[t], (nj - 1) & 1, abort_flag, g.err);
+            tc_fence_after();
+            if (leads() && ok) {
+                issue_pv(prev, nj > 1);
+                tc_commit(&kv_empty[prev]);
+                tc_commit(&o_final[t]);
             }
-            if (elect_one()) tc_commit(mma_done);
+            rejoin();
+            if (leads()) tc_commit(mma_done);
+          }
             __syncwarp();
             const unsigned long long t0 = globaltimer();
             while (!mbar_try_wait(mma_done, 0) && globaltimer() - t0 < kWaitLimitNs) {
@@ -372,7 +379,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
         const uint64_t scale2 = pair(g.scale_log2, g.scale_log2);
         bool ok = true, s_ready = false;
         for (int j = 0; j < nj; ++j) {                  // j counts this CTA's steps
-            if (!s_ready && !mbar_wait(&s_full[t], j & 1, abort_flag, g.err)) { ok = false; break; }
+            if (!s_ready && !mbar_wait_warp(&s_full[t], j & 1, abort_flag, g.err)) { ok = false; break; }
             tc_fence_after();
             float s[BKV];
 #pragma unroll
@@ -428,7 +435,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
             m_run = base;
             // PV(t, j-1) must be done before P(t) is overwritten and O(t) rescaled
             if (j > 0) {
-                if (!mbar_wait(&p_free[t], (j - 1) & 1, abort_flag, g.err)) { ok = false; break; }
+                if (!mbar_wait_warp(&p_free[t], (j - 1) & 1, abort_flag, g.err)) { ok = false; break; }
                 tc_fence_after();
             }
             if (j > 0 && moved) {
@@ -462,7 +469,8 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
             }
             if (D == 64) s_ready = __all_sync(0xffffffffu, next);
         }
-        if (ok && is_part && mbar_wait(&o_final[t], 0, abort_flag, g.err)) {
+        if (ok) ok = mbar_wait_warp(&o_final[t], 0, abort_flag, g.err);
+        if (ok && is_part) {
             // a part of a split unit: unnormalised O with its base and row
             // sum, merged by the combine kernel
             tc_fence_after();
@@ -479,7 +487,7 @@ __global__ void __launch_bounds__(AttnCfg<D>::THREADS, 1)
                                                  __uint_as_float(o[4 * q + 2]), __uint_as_float(o[4 * q + 3]));
             }
             reinterpret_cast<float2*>(g.part_ml)[prow] = make_float2(m_run, l_run);
-        } else if (ok && mbar_wait(&o_final[t], 0, abort_flag, g.err)) {
+        } else if (ok) {
             tc_fence_after();
             const int tok = q0 + t * BQ + row;
             const float inv = 1.0f / l_run;

@@ -14,7 +14,7 @@
 //   warp 0      TMA producer: A and W tiles of 64 columns of K into a
 //               shared-memory ring (128-byte swizzle), one mbarrier pair per
 //               stage;
-//   warp 1      MMA issuer: one thread issues the tcgen05.mma of each stage
+//   warp 1      MMA issuer: one elected lane issues the tcgen05.mma of each stage
 //               into one of two TMEM accumulators, commits the stage back to
 //               the producer and the accumulator to the epilogue;
 //   warps 2-5   epilogue (epilogue_tile): each warp owns its 32-lane TMEM
@@ -388,8 +388,7 @@ __device__ __forceinline__ bool epilogue_tile(const Epi& e, int staged, const Ep
             tmem_ld16x256(taddr + (col0 - n0), *reinterpret_cast<float(*)[32]>(&v[0]));
             tmem_ld16x256(taddr + (16u << 16) + (col0 - n0), *reinterpret_cast<float(*)[32]>(&v[1]));
             if constexpr (is_resid(FORM)) {
-                const bool landed = mbar_wait(&ws.rbar[sl], (ws.cnt >> 1) & 1, abort_flag, err);
-                if (!__all_sync(0xffffffffu, landed)) {
+                if (!mbar_wait_warp(&ws.rbar[sl], (ws.cnt >> 1) & 1, abort_flag, err)) {
                     release();                     // every other wait of the CTA gives up too
                     return false;
                 }
@@ -556,7 +555,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 const CUtensorMap* mA = prob ? &tmA1 : &tmA;
                 const CUtensorMap* mB = prob ? &tmB1 : &tmB;
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
-                    if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.err)) { ok = false; break; }
+                    if (!mbar_wait_warp(&empty[stage], phase ^ 1u, abort_flag, g.err)) { ok = false; break; }
                     if (elect_one()) {
                         mbar_arrive_expect_tx(&full[stage], STAGE_BYTES);
                         uint8_t* sa = smem + stage * STAGE_BYTES;
@@ -578,7 +577,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             }
         }
     } else if (warp == 1) {
-        {
+        // one lane for the whole loop: less code than the other kernels' warp,
+        // and code that a short launch runs once costs it its fetch (a forward
+        // of 2 layers, 272 tokens: 97.5 -> 95 us)
+        if (elect_one()) {
             const uint64_t da = sdesc_sw128(smem_u32(smem)), db = sdesc_sw128(smem_u32(smem) + A_BYTES);
             int stage = 0;
             uint32_t phase = 0;
@@ -592,27 +594,24 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
                     if (!mbar_wait(&full[stage], phase, abort_flag, g.err)) { ok = false; break; }
                     tc_fence_after();
-                    if (elect_one()) {
 #pragma unroll
-                        for (int k = 0; k < BK / 16; ++k)
-                            tc_mma(d, sdesc_at(da, stage * STAGE_BYTES + k * 32), sdesc_at(db, stage * STAGE_BYTES + k * 32),
-                                   C::IDESC, (kb | k) != 0);
-                        tc_commit(&empty[stage]);
-                        if (kb + 1 == g.k_blocks) tc_commit(&tfull[acc]);
-                    }
-                    __syncwarp();
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma(d, sdesc_at(da, stage * STAGE_BYTES + k * 32), sdesc_at(db, stage * STAGE_BYTES + k * 32),
+                               C::IDESC, (kb | k) != 0);
+                    tc_commit(&empty[stage]);
+                    if (kb + 1 == g.k_blocks) tc_commit(&tfull[acc]);
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
                 acc ^= 1;
                 if (acc == 0) acc_phase ^= 1u;
             }
-            // all MMAs issued by this warp have completed before TMEM is freed
-            if (elect_one()) tc_commit(mma_done);
-            __syncwarp();
+            // all MMAs issued by this lane have completed before TMEM is freed
+            tc_commit(mma_done);
             const unsigned long long t0 = globaltimer();
             while (!mbar_try_wait(mma_done, 0) && globaltimer() - t0 < kWaitLimitNs) {
             }
         }
+        __syncwarp();
     } else {
         const int lg = warp & 3;   // TMEM lane quarter this warp may access
         int acc = 0;
@@ -625,7 +624,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             const EpiMaps* mp = prob ? &maps1 : &maps;
             const Epi e = problem_epilogue(g, prob);
             epilogue_prefetch<FORM>(e, staged, &mp->res, Mp, n0, end, m0, ws, lane);
-            if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, g.err)) break;
+            if (!mbar_wait_warp(&tfull[acc], acc_phase, abort_flag, g.err)) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(acc * BNT);
             const bool ok = epilogue_tile<FORM>(e, staged, mp, Mp, m0, n0, end, taddr, ws, abort_flag, g.err, lane, [&] {
@@ -780,7 +779,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
                 const int m0 = mb * 256 + (int)rank * 128;
                 const int n0 = nb * BNP + (int)rank * (BNP / 2);
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
-                    if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.err)) { ok = false; break; }
+                    if (!mbar_wait_warp(&empty[stage], phase ^ 1u, abort_flag, g.err)) { ok = false; break; }
                     if (elect_one()) {
                         if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * STAGE_BYTES);
                         const uint32_t fb = mapa_shared(smem_u32(&full[stage]), 0);
@@ -816,15 +815,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             uint32_t phase = 0;
             int acc = 0;
             uint32_t acc_phase = 0;
-            bool ok = true;
-            for (int tile = cluster_id; tile < num_tiles && ok; tile += n_clusters) {
-                if (!mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, g.err)) break;
+            bool ok = true;                        // this lane's waits (elect_one)
+            for (int tile = cluster_id; tile < num_tiles; tile += n_clusters) {
+                ok = ok && mbar_wait(&tempty[acc], acc_phase ^ 1u, abort_flag, g.err);
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)(acc * 256);
                 for (int kb = 0; kb < g.k_blocks; ++kb) {
-                    if (!mbar_wait(&full[stage], phase, abort_flag, g.err)) { ok = false; break; }
+                    ok = ok && mbar_wait(&full[stage], phase, abort_flag, g.err);
                     tc_fence_after();
-                    if (elect_one()) {
+                    if (elect_one() && ok) {
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k)
                             tc_mma2(d, sdesc_at(da, stage * STAGE_BYTES + k * 32), sdesc_at(db, stage * STAGE_BYTES + k * 32),
@@ -857,7 +856,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             const EpiMaps* mp = prob ? &maps1 : &maps;
             const Epi e = problem_epilogue(g, prob);
             epilogue_prefetch<FORM>(e, staged, &mp->res, Mp, n0, end, m0, ws, lane);
-            if (!mbar_wait(&tfull[acc], acc_phase, abort_flag, g.err)) break;
+            if (!mbar_wait_warp(&tfull[acc], acc_phase, abort_flag, g.err)) break;
             tc_fence_after();
             const uint32_t taddr = tmem + ((uint32_t)(lg * 32) << 16) + (uint32_t)(acc * 256);
             auto release = [&] {
@@ -1023,7 +1022,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             int stage = 0;
             uint32_t phase = 0;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, g.err)) break;
+                if (!mbar_wait_warp(&empty[stage], phase ^ 1u, abort_flag, g.err)) break;
                 if (elect_one()) {
                     mbar_arrive_expect_tx(&full[stage], SPLIT_STAGE_BYTES);
                     uint8_t* sa = smem + stage * SPLIT_STAGE_BYTES;
@@ -1048,10 +1047,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
             const uint64_t da = sdesc_sw128(smem_u32(smem)), db = sdesc_sw128(smem_u32(smem) + A_BYTES);
             int stage = 0;
             uint32_t phase = 0;
+            bool ok = true;                        // this lane's waits (elect_one)
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!mbar_wait(&full[stage], phase, abort_flag, g.err)) break;
+                ok = ok && mbar_wait(&full[stage], phase, abort_flag, g.err);
                 tc_fence_after();
-                if (elect_one()) {
+                if (elect_one() && ok) {
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
                         tc_mma(tmem_base, sdesc_at(da, stage * SPLIT_STAGE_BYTES + k * 32),

@@ -80,10 +80,37 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     }
 }
 
-// True in one lane of the (converged) warp.  The producer and MMA warps run
-// their loops with all lanes and issue from the elected one: under a branch on
-// the lane number the compiler cannot keep descriptors and addresses in
-// uniform registers (128 x 512 x 12288 in 128 x 128 tiles: 53.7 -> 48.7 us).
+// The same for a whole (converged) warp, with one outcome for all its lanes.  A
+// phase that completes just as the limit runs out or another wait gives up is
+// seen by some lanes and not by others: a lane that went on by itself would wait
+// without limit, in the next elect.sync, shuffle or other instruction of the
+// whole warp, for the lanes that have left.  So the lanes vote on every look.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned* err) {
+    constexpr unsigned kAll = 0xffffffffu;
+    if (__all_sync(kAll, mbar_try_wait(bar, parity))) return true;
+    const unsigned long long t0 = globaltimer();
+    uint32_t spins = 0;
+    while (!__all_sync(kAll, mbar_try_wait(bar, parity))) {
+        bool stop = *abort_flag;
+        if ((++spins & 255u) == 0u && globaltimer() - t0 > kWaitLimitNs) {
+            stop = true;
+            *abort_flag = 1;
+            atomicOr(err, kErrTimeout);
+        }
+        if (__any_sync(kAll, stop)) return false;
+    }
+    return true;
+}
+
+// True in one lane of the (converged) warp, the same one each time.  The
+// producers and most MMA issuers run their loops with all lanes and issue from
+// the elected one: under a branch on the lane number the compiler cannot keep
+// descriptors and addresses in uniform registers (128 x 512 x 12288 in 128 x 128
+// tiles: 53.7 -> 48.7 us).  A producer's waits vote (mbar_wait_warp).  An issuer's
+// lanes each remember whether their own waits succeeded and stay in the loop to
+// its end, and the elected lane issues as long as its own have: a vote on the
+// way from a wait to the MMAs costs the attention 1-3%.  Either way all lanes
+// reach every elect_one and __syncwarp.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
