@@ -255,7 +255,9 @@ wdc_status wdc_selftest_wait_timeout(wdc_ctx* ctx, unsigned long long limit_ns, 
 /* ------------------------------------------------------------------ weights */
 /* Copies one parameter tensor (host fp32, `count` elements, shape as listed in
  * wdc_tensor_id) into the model, converting to the model dtype (bf16:
- * round-to-nearest-even).  layer/stream are ignored for global tensors. */
+ * round-to-nearest-even).  layer/stream are ignored for global tensors.
+ * Synchronous: the tensor is on the device on return, for calls on any stream;
+ * calls that still run on a non-blocking stream are not waited for. */
 wdc_status wdc_set_tensor(wdc_ctx* ctx, int tensor_id, int layer, int stream,
                           const float* host, size_t count);
 /* Reads one parameter tensor back into `host` (fp32, `count` elements, the

@@ -66,9 +66,10 @@ namespace {
 // y[r] = act(W[r,:] . x + b[r]); one warp per row.  act: 0 none, 1 SiLU.
 // Bound by the latency of its loads (E x E) or by reading W (the modulation).
 // With whole 16-byte vectors in a row (vec) each lane loads up to four of W's
-// before the wait for x: weights change only in calls that synchronise with the
-// device before they return, so W's reads run under the kernels before.  Alone, 26624 x 512 bf16 (27 MB, cold) takes 10 us as with 2-byte
-// loads; the gain is in the chain (with prep_kernel's, see there).  fp32 keeps
+// before the wait for x: weights change only in wdc_init_weights and
+// wdc_set_tensor, which return once they are on the device, so W's reads run
+// under the kernels before.  Alone, 26624 x 512 bf16 (27 MB, cold) takes 10 us
+// as with 2-byte loads; the gain is in the chain (with prep_kernel's, see there).  fp32 keeps
 // the element order of its sums: by vectors, the rollout with the
 // ill-conditioned linear observation came out 1.4e-5 off fp64 instead of 6e-6.
 template <typename T>
@@ -1048,14 +1049,18 @@ static uint16_t f32_to_bf16_bits(float f) {
     return (uint16_t)(u >> 16);
 }
 
+// The parameter is on the device when this returns: a copy from pageable memory
+// may return once it is staged, and a forward on a non-blocking stream would not
+// wait for the rest of it.
 static wdc_status upload(Ctx* c, void* dst, const float* host, size_t count, bool model_dtype) {
     if (!model_dtype || c->dit->dtype == WDC_F32) {
         WDC_CUDA_TRY(c, cudaMemcpy(dst, host, count * sizeof(float), cudaMemcpyHostToDevice));
-        return WDC_OK;
+    } else {
+        std::vector<uint16_t> tmp(count);
+        for (size_t i = 0; i < count; ++i) tmp[i] = f32_to_bf16_bits(host[i]);
+        WDC_CUDA_TRY(c, cudaMemcpy(dst, tmp.data(), count * 2, cudaMemcpyHostToDevice));
     }
-    std::vector<uint16_t> tmp(count);
-    for (size_t i = 0; i < count; ++i) tmp[i] = f32_to_bf16_bits(host[i]);
-    WDC_CUDA_TRY(c, cudaMemcpy(dst, tmp.data(), count * 2, cudaMemcpyHostToDevice));
+    WDC_CUDA_TRY(c, cudaStreamSynchronize(cudaStreamLegacy));     // the stream of cudaMemcpy
     return WDC_OK;
 }
 
