@@ -80,10 +80,10 @@ struct AttnCfg {
     static constexpr uint32_t K_TILE = BK * D * 2;
     static constexpr uint32_t V_TILE = D * BK * 2;
     static constexpr uint32_t STAGE = K_TILE + V_TILE;      // 32 KB for both head sizes
-    // steps from which tile 1 starts behind tile 0: a single step of 128 keys is
-    // longer for it (4 heads, L = 30: 5.73 us, 5.30 together), two are not (L =
-    // 130: 6.61 behind, 6.72 together), nor one of 64 (5.4 and 5.4 - 5.6)
-    static constexpr int STAGGER_FROM = D == 64 ? 2 : 1;
+    // steps from which tile 1 starts behind tile 0: a single step is longer for it
+    // (4 heads, us behind / together: d = 64, L = 30 5.73 / 5.30; d = 128, L = 30
+    // 5.50 / 5.18, L = 64 5.19 / 5.06), two are not (d = 64, L = 130 6.61 / 6.72)
+    static constexpr int STAGGER_FROM = 2;
     static constexpr int STAGES = 5;
     static constexpr uint32_t SMEM = 2 * Q_TILE + STAGES * STAGE + 1024 + 256;
     static constexpr uint32_t TMEM_COLS = 512;
