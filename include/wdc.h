@@ -235,6 +235,21 @@ const char* wdc_last_error(const wdc_ctx* ctx);
 size_t wdc_latent_numel(const wdc_ctx* ctx);
 /* Number of kernels this context has launched so far (all streams). */
 unsigned long long wdc_launch_count(const wdc_ctx* ctx);
+/* Which kernels ran a bf16 context's GEMMs so far (a diagnostic: the kernel is
+ * chosen from the shape).  counts[kernel * WDC_GEMM_FORMS + form] += 1 for a
+ * launch of one problem, += 1 << 32 for a grouped one (a dual-stream block's
+ * video and condition rows).  WDC_ERR_INVALID_ARG on a null pointer. */
+enum wdc_gemm_kernel {
+    WDC_GEMM_PAIR256 = 0, WDC_GEMM_PAIR192 = 1, WDC_GEMM_PAIR128 = 2,   /* CTA pairs, 256-row tiles this wide */
+    WDC_GEMM_ONE128 = 3, WDC_GEMM_ONE64 = 4,                            /* one CTA, 128-row tiles this wide   */
+    WDC_GEMM_SPLIT2 = 5, WDC_GEMM_SPLIT4 = 6, WDC_GEMM_SPLIT8 = 7,      /* K over this many CTAs              */
+    WDC_GEMM_KERNELS = 8
+};
+enum wdc_gemm_form {
+    WDC_GEMM_STORE = 0, WDC_GEMM_GELU = 1, WDC_GEMM_RESID = 2, WDC_GEMM_QKV = 3, WDC_GEMM_UNPATCH = 4,
+    WDC_GEMM_RESID_GELU = 5, WDC_GEMM_RESID_REPEAT = 6, WDC_GEMM_FORMS = 7
+};
+wdc_status wdc_gemm_launches(const wdc_ctx* ctx, unsigned long long* counts);
 /* Synchronises the device and returns (then clears) the bits the kernels have
  * set in the context's error word: 1 = a bounded device-side wait timed out,
  * 4 = the two CTAs of a tensor-core pair saw different tensor-memory bases,

@@ -463,6 +463,13 @@ unsigned long long wdc_launch_count(const wdc_ctx* h) {
     return c ? c->launches : 0;
 }
 
+wdc_status wdc_gemm_launches(const wdc_ctx* h, unsigned long long* counts) {
+    const Ctx* c = reinterpret_cast<const Ctx*>(h);
+    if (!c || !counts) return WDC_ERR_INVALID_ARG;
+    std::memcpy(counts, c->gemm_launches, sizeof(c->gemm_launches));
+    return WDC_OK;
+}
+
 wdc_status wdc_set_tensor(wdc_ctx* h, int tensor_id, int layer, int stream, const float* host, size_t count) {
     Ctx* c = reinterpret_cast<Ctx*>(h);
     if (!c) return WDC_ERR_INVALID_ARG;

@@ -111,8 +111,9 @@ __device__ __forceinline__ float2 unpack_bf16(uint32_t u) {
 // Epilogue forms; each is its own instantiation of the kernels, so that the
 // epilogue's code stays small and without branches on the form.
 enum Form {
-    kFormStore = 0, kFormGelu = 1, kFormResid = 2, kFormQKV = 3, kFormUnpatch = 4, kFormResidGelu = 5,
-    kFormResidRepeat = 6, kForms = 7
+    kFormStore = WDC_GEMM_STORE, kFormGelu = WDC_GEMM_GELU, kFormResid = WDC_GEMM_RESID, kFormQKV = WDC_GEMM_QKV,
+    kFormUnpatch = WDC_GEMM_UNPATCH, kFormResidGelu = WDC_GEMM_RESID_GELU, kFormResidRepeat = WDC_GEMM_RESID_REPEAT,
+    kForms = WDC_GEMM_FORMS
 };
 // kFormResidGelu: a residual over GELU's result, an operator call's only (the
 // blocks apply GELU before another GEMM).
@@ -1276,6 +1277,13 @@ struct Choice {
     enum Kind { kPair, kOne128, kOne64, kSplit } kind;
     int bn = 256;
     int split = 1;
+    wdc_gemm_kernel id() const {
+        switch (kind) {
+            case kPair: return bn == 256 ? WDC_GEMM_PAIR256 : (bn == 192 ? WDC_GEMM_PAIR192 : WDC_GEMM_PAIR128);
+            case kSplit: return split == 2 ? WDC_GEMM_SPLIT2 : (split == 4 ? WDC_GEMM_SPLIT4 : WDC_GEMM_SPLIT8);
+            default: return bn == 64 ? WDC_GEMM_ONE64 : WDC_GEMM_ONE128;
+        }
+    }
 };
 
 // Estimated cycles of a launch with `tiles` tiles on `units` SMs or pairs:
@@ -1492,6 +1500,7 @@ wdc_status launch_gemm(Ctx* c, const Problem& p0, const Problem* p1, int N, int 
     }
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("tcgen05 GEMM launch: ") + cudaGetErrorString(err));
+    c->gemm_launches[ch.id() * kForms + form] += p1 ? 1ull << 32 : 1ull;
     return WDC_OK;
 }
 

@@ -143,6 +143,7 @@ struct Ctx {
     std::vector<StepScalars> stepf;    // [T] per-step fp32 schedule values
     std::string last_error;
     unsigned long long launches = 0;
+    unsigned long long gemm_launches[WDC_GEMM_KERNELS * WDC_GEMM_FORMS] = {};   // see wdc_gemm_launches
 
     // memory
     DevState* st = nullptr;

@@ -31,6 +31,9 @@ GLOBAL_TENSORS = {"patch.w": T_PATCH_W, "patch.b": T_PATCH_B, "cond.w": T_COND_W
                   "final.mod.w": T_FMOD_W, "final.mod.b": T_FMOD_B, "final.w": T_FINAL_W, "final.b": T_FINAL_B}
 LAYER_TENSORS = {"mod.w": T_MOD_W, "mod.b": T_MOD_B, "qkv.w": T_QKV_W, "qkv.b": T_QKV_B, "o.w": T_O_W,
                  "o.b": T_O_B, "fc1.w": T_FC1_W, "fc1.b": T_FC1_B, "fc2.w": T_FC2_W, "fc2.b": T_FC2_B}
+# wdc_gemm_kernel and wdc_gemm_form, by value
+GEMM_KERNELS = ["pair256", "pair192", "pair128", "one128", "one64", "split2", "split4", "split8"]
+GEMM_FORMS = ["store", "gelu", "resid", "qkv", "unpatch", "resid_gelu", "resid_repeat"]
 
 
 class WdcError(RuntimeError):
@@ -125,6 +128,7 @@ def _load():
         "wdc_last_error": (ctypes.c_char_p, [P]),
         "wdc_latent_numel": (S, [P]),
         "wdc_launch_count": (ctypes.c_ulonglong, [P]),
+        "wdc_gemm_launches": (I, [P, ctypes.POINTER(ctypes.c_ulonglong)]),
         "wdc_set_tensor": (I, [P, I, I, I, P, S]),
         "wdc_get_tensor": (I, [P, I, I, I, P, S]),
         "wdc_init_weights": (I, [P, ctypes.c_ulonglong, F]),
@@ -241,6 +245,18 @@ class Context:
     @property
     def launches(self):
         return LIB.wdc_launch_count(self._h)
+
+    def gemm_launches(self):
+        """wdc_gemm_launches: {(kernel, form, grouped): launches} of the bf16 GEMMs so far."""
+        counts = (ctypes.c_ulonglong * (len(GEMM_KERNELS) * len(GEMM_FORMS)))()
+        self._check(LIB.wdc_gemm_launches(self._h, counts), "gemm_launches")
+        out = {}
+        for i, v in enumerate(counts):
+            key = GEMM_KERNELS[i // len(GEMM_FORMS)], GEMM_FORMS[i % len(GEMM_FORMS)]
+            for grouped, n in ((False, v & 0xffffffff), (True, v >> 32)):
+                if n:
+                    out[key + (grouped,)] = n
+        return out
 
     def set_cache_params(self, params):
         self._check(LIB.wdc_set_cache_params(self._h, ctypes.byref(params)), "set_cache_params")

@@ -14,6 +14,18 @@ def rel_l2(a, b):
     return float(np.linalg.norm(a - b) / (den if den > 0 else 1.0))
 
 
+def assert_gemms(ctx, *expected):
+    """Each of `expected`, "kernel/form" or "kernel/form grouped", is among the
+    bf16 GEMMs the context has launched: a test for a kernel's edges has reached
+    that kernel.  The launch rule's choices are those for 152 SMs."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        return
+    ran = {f"{kernel}/{form}{' grouped' if grouped else ''}" for kernel, form, grouped in ctx.gemm_launches()}
+    missing = [e for e in expected if e not in ran]
+    assert not missing, (missing, sorted(ran))
+
+
 def params_for_both(**kw):
     """The same constants as an oracle CacheParams and a wdc_cache_params."""
     from oracle.params import CacheParams

@@ -3,9 +3,9 @@ the paper rolls out one trajectory at a time and is silent on classifier-free
 guidance).
 
 * A batched forward gives each sample bitwise the velocity of a forward on it
-  alone (fp32 SIMT and bf16 tcgen05 paths; single and dual stream; a case
-  whose condition-token GEMM moves from the single-CTA to the CTA-pair kernel
-  when batched).
+  alone (fp32 SIMT and bf16 tcgen05 paths; single and dual stream; a case with
+  more condition rows; a case whose QKV and MLP GEMMs move from the single-CTA
+  to the CTA-pair kernel when batched).
 * The guided forward against the oracle's guided velocity (fp32 parity
   model, rel L2 <= 1e-5 against fp64).
 * wdc_rollout_batch against the oracle's per-sample cached rollouts: three
@@ -23,7 +23,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import params_for_both, rel_l2
+from helpers import assert_gemms, params_for_both, rel_l2
 from oracle import batch as ob
 from oracle import dit
 from oracle import schedule as sch
@@ -35,6 +35,7 @@ PARITY_MODEL = dict(layers=2, hidden=256, heads=4, head_dim=64, mlp=1024, temb_d
                     frames=4, height=16, width=16, patch=2, cond_tokens=16, cond_dim=256, dual_stream=0)
 DUAL_128 = dict(PARITY_MODEL, layers=1, heads=2, head_dim=128, dual_stream=1)
 WIDE_COND = dict(PARITY_MODEL, layers=1, cond_tokens=96)          # 96 rows alone, 288 in a batch of 3
+TO_PAIRS = dict(PARITY_MODEL, layers=1, hidden=768, heads=12, mlp=3072, height=24, width=24, cond_tokens=24)   # 600, 1800
 SHAPE = (16, 4, 16, 16)
 N = 16 * 4 * 16 * 16
 T = 10
@@ -51,21 +52,27 @@ def _ctx(cfgd, dtype, max_batch, W, params=None):
 
 
 @pytest.mark.parametrize("dtype", [wdc.F32, wdc.BF16])
-@pytest.mark.parametrize("model", ["single", "dual128", "wide_cond"])
+@pytest.mark.parametrize("model", ["single", "dual128", "wide_cond", "to_pairs"])
 def test_batched_forward_equals_single_forwards(dtype, model):
-    cfgd = {"single": PARITY_MODEL, "dual128": DUAL_128, "wide_cond": WIDE_COND}[model]
+    cfgd = {"single": PARITY_MODEL, "dual128": DUAL_128, "wide_cond": WIDE_COND, "to_pairs": TO_PAIRS}[model]
+    shape = (16, 4, cfgd["height"], cfgd["width"])
+    N = int(np.prod(shape))
     W = synth.dit_weights(cfgd, 7, std=0.02, bias_std=0.02)
     ctx = _ctx(cfgd, dtype, 4, W)
     B = 3
-    zs = [_dev(synth.latent(30 + b, SHAPE)) for b in range(B)]
+    zs = [_dev(synth.latent(30 + b, shape)) for b in range(B)]
     cts = [_dev(synth.cond_tokens(40 + b, cfgd["cond_tokens"], 256)) for b in range(B)]
     vs = [torch.empty(N, device="cuda") for _ in range(B)]
     ctx.dit_forward_batch(zs, 731.0, cts, vs)
+    if dtype == wdc.BF16 and model == "to_pairs":
+        assert_gemms(ctx, "pair256/qkv", "pair192/gelu")
     for b in range(B):
         ref = torch.empty(N, device="cuda")
         ctx.dit_forward(zs[b], 731.0, cts[b], ref)
         torch.cuda.synchronize()
         assert torch.equal(vs[b], ref), (model, b)
+    if dtype == wdc.BF16 and model == "to_pairs":
+        assert_gemms(ctx, "one128/qkv", "one128/gelu")
     assert ctx.device_errors() == 0
 
 

@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import rel_l2
+from helpers import assert_gemms, rel_l2
 from oracle import dit
 from oracle.params import DiTConfig
 from paper_2608_01845_gb300 import synth, wdc
@@ -71,11 +71,10 @@ def _h(a):
                                    (257, 32, 8)])
 @pytest.mark.parametrize("mode", ["store", "gelu", "resid"])
 def test_bf16_gemm_matches_oracle(M, N, K, mode):
-    """The tcgen05 GEMMs (one CTA per tile below 256 rows, CTA pairs from
-    256) with each fused epilogue, down to the smallest shapes they take: one
-    row, one 32-column chunk, one 8-element K step (one 64-wide K block,
-    zero-filled past K), and a pair grid whose second 256-row tile holds a
-    single row."""
+    """The tcgen05 GEMM of one-CTA 128 x 64 tiles (with GELU, 1000 x 768 x 1024
+    is split over K) with each fused epilogue, down to the smallest shapes it
+    takes: one row, one 32-column chunk, one 8-element K step (one 64-wide K
+    block, zero-filled past K), and a third 128-row tile of a single row."""
     ctx = _ctx(dict(PARITY_MODEL, layers=1), wdc.BF16)
     A = _bf(synth.normal(1, (M, K)))
     W = _bf(synth.normal(2, (N, K), 0.05))
@@ -278,8 +277,9 @@ def test_bf16_attention_full_size_sampled_rows(H, L, d):
 
 @pytest.mark.parametrize("M,N,K", [(17776, 9216, 3072), (1000, 768, 1024)])
 def test_bf16_gemm_sampled_full_size_and_no_device_errors(M, N, K):
-    """Full 5B-scale QKV shape (the CTA-pair kernel) checked on 64 sampled rows;
-    no kernel reported a timeout or a tensor-memory pair mismatch."""
+    """Full 5B-scale QKV shape (the CTA-pair kernel) and a shape of one-CTA tiles
+    checked on 64 sampled rows; no kernel reported a timeout or a tensor-memory
+    pair mismatch."""
     ctx = _ctx(dict(PARITY_MODEL, layers=1), wdc.BF16)
     g = np.random.default_rng(55)
     A = _bf(g.standard_normal((M, K), dtype=np.float32))
@@ -287,6 +287,7 @@ def test_bf16_gemm_sampled_full_size_and_no_device_errors(M, N, K):
     C = torch.empty(M, N, dtype=torch.bfloat16, device="cuda")
     ctx.op_gemm(_to_dev(A, torch.bfloat16), _to_dev(W, torch.bfloat16), C)
     torch.cuda.synchronize()
+    assert_gemms(ctx, "pair256/store" if M == 17776 else "one64/store")
     rows = np.sort(g.choice(M, 64, replace=False))
     rows[-1] = M - 1
     want = A[rows].astype(np.float64) @ W.astype(np.float64).T
@@ -323,10 +324,10 @@ def test_profiler_times_every_launch_and_dual_stream_gemms_are_grouped():
 def test_bf16_block_hidden_3072_few_ragged_rows(dual):
     """The D = 3072 kernels on a short ragged sequence: 5 condition + 272
     video tokens (277 rows: not a multiple of the LayerNorm's 8 rows per
-    block nor of the attention's 128-row tiles; 272 video rows leave a
-    16-row tail in the second 256-row GEMM tile pair; with dual-stream
-    weights each GEMM is one grouped launch whose second problem has 5
-    rows), the whole block against the fp64 oracle on every row."""
+    block nor of the attention's 128-row tiles; in the CTA pairs' 256-row
+    tiles the second holds 21 rows, or with dual-stream weights 16, and each
+    GEMM is then one grouped launch whose second problem has 5 rows), the whole
+    block against the fp64 oracle on every row."""
     cfgd = dict(layers=1, hidden=3072, heads=48, head_dim=64, mlp=12288, temb_dim=512, freq_dim=256, in_ch=16,
                 frames=1, height=32, width=34, patch=2, cond_tokens=5, cond_dim=3072, dual_stream=dual)
     cfg = DiTConfig(**cfgd)
@@ -345,6 +346,8 @@ def test_bf16_block_hidden_3072_few_ragged_rows(dual):
     xt = _to_dev(x, torch.bfloat16)
     ctx.dit_block_forward(0, xt, _to_dev(np.concatenate(mods, axis=0)))
     torch.cuda.synchronize()
+    assert_gemms(ctx, *(["pair256/gelu grouped", "pair128/resid grouped", "one128/qkv grouped"] if dual else
+                        ["pair256/qkv", "one128/gelu", "split2/resid"]))
     want = dit.block(x.astype(np.float64), W, cfg, 0, [m.astype(np.float64) for m in mods])
     got = xt.float().cpu().numpy()
     assert rel_l2(got - x, want - x) <= BF16_TOL

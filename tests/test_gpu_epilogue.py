@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import rel_l2
+from helpers import assert_gemms, rel_l2
 from oracle import dit
 from oracle.params import DiTConfig
 from paper_2608_01845_gb300 import synth, wdc
@@ -42,6 +42,7 @@ def test_gemm_rows_and_columns(M, N, mode):
         kw.update(res=_dev(R, torch.bfloat16), gate=_dev(g))
     ctx.op_gemm(_dev(A, torch.bfloat16), _dev(W, torch.bfloat16), C, bias=_dev(b), **kw)
     torch.cuda.synchronize()
+    assert_gemms(ctx, f"one64/{mode}")
     assert ctx.device_errors() == 0
     assert rel_l2(C.float().cpu().numpy(), want) <= 2.0 ** -8 + K * 2.0 ** -22
     assert bool((buf[M:] == 7.0).all())
@@ -73,10 +74,13 @@ def test_forward_slabs_across_samples_and_streams(Lc, dual, d):
     assert rel_l2(one[0].cpu().numpy(), want) <= 2e-2
 
 
-@pytest.mark.parametrize("M,N,K", [(226, 3072, 3072), (64, 1056, 8192), (128, 512, 12288), (1, 9216, 3072), (257, 160, 4104),
-                                   (130, 32, 2056), (700, 1024, 1024), (1600, 1024, 2048)])
+@pytest.mark.parametrize("M,N,K,kernel", [
+    (226, 3072, 3072, "split2"), (64, 1056, 8192, "split8"), (128, 512, 12288, "split8"), (1, 9216, 3072, "split2"),
+    (257, 160, 4104, "split8"), (130, 32, 2056, "split8"), (64, 3072, 8192, "split4"), (200, 1056, 1544, "split4"),
+    (700, 1024, 1024, {"store": "one64", "gelu": "split2", "resid": "one64"}), (129, 6176, 520, "one128"),
+    (1600, 1024, 2048, "pair128")])
 @pytest.mark.parametrize("mode", ["store", "gelu", "resid"])
-def test_gemm_few_tiles(M, N, K, mode):
+def test_gemm_few_tiles(M, N, K, kernel, mode):
     """Shapes of the narrow-tile and split-K kernels (2, 4 and 8 CTAs a tile,
     shares past N, K blocks that do not divide evenly), bound as above."""
     ctx = wdc.Context(wdc.make_config(dtype=wdc.BF16, **MODEL), 2)
@@ -94,16 +98,24 @@ def test_gemm_few_tiles(M, N, K, mode):
         kw.update(res=R, gate=gate)
     ctx.op_gemm(A, W, buf[:M], bias=b, **kw)
     torch.cuda.synchronize()
+    assert_gemms(ctx, f"{kernel if isinstance(kernel, str) else kernel[mode]}/{mode}")
     assert ctx.device_errors() == 0
     assert float((buf[:M].double() - want).norm() / want.norm()) <= 2.0 ** -8 + K * 2.0 ** -22
     assert bool((buf[M:] == 7.0).all())
 
 
-@pytest.mark.parametrize("Lc,dual,d", [(5, 0, 64), (5, 1, 128), (140, 1, 64)])
-def test_forward_split_k(Lc, dual, d):
-    """A wide model on few tokens (every GEMM of its block splits K) against the
-    oracle, and a batch of three bitwise equal to its samples' own forwards."""
-    cfgd = dict(MODEL, hidden=2048, heads=2048 // d, head_dim=d, mlp=4096, frames=1, height=8, width=10, cond_tokens=Lc,
+@pytest.mark.parametrize("Lc,dual,d,D,mlp,gemms", [
+    (5, 0, 64, 2048, 4096, ["split4/store", "split2/qkv", "split4/gelu", "split4/resid"]),
+    (5, 1, 128, 2048, 4096, ["split2/gelu grouped", "split4/resid grouped", "split8/unpatch"]),
+    (100, 1, 128, 1536, 1024, ["split8/store", "split2/qkv grouped", "split4/gelu grouped", "split4/resid grouped", "split4/unpatch"]),
+    (140, 1, 64, 2048, 1024, ["split4/gelu grouped", "split2/resid grouped"])])
+def test_forward_split_k(Lc, dual, d, D, mlp, gemms):
+    """A wide model on few tokens, whose block's GEMMs split K (those named;
+    two problems in one launch with both streams, of which the condition rows'
+    have two row tiles at 140 tokens), against the oracle, and a batch of three
+    bitwise equal to its samples' own forwards.  (QKV of more row tiles has too
+    many tiles to be split.)"""
+    cfgd = dict(MODEL, hidden=D, heads=D // d, head_dim=d, mlp=mlp, frames=1, height=8, width=10, cond_tokens=Lc,
                 cond_dim=2048, dual_stream=dual)
     W = synth.dit_weights(cfgd, 9, std=0.02, bias_std=0.05, bf16=True)
     ctx = wdc.Context(wdc.make_config(dtype=wdc.BF16, max_batch=3, **cfgd), 2)
@@ -118,6 +130,7 @@ def test_forward_split_k(Lc, dual, d):
     many = [torch.empty_like(t) for t in zd]
     ctx.dit_forward_batch(zd, 600.0, cd, many)
     torch.cuda.synchronize()
+    assert_gemms(ctx, *gemms)
     assert ctx.device_errors() == 0
     for b in range(3):
         assert torch.equal(one[b], many[b])
@@ -125,12 +138,12 @@ def test_forward_split_k(Lc, dual, d):
     assert rel_l2(one[0].cpu().numpy(), want) <= 2e-2
 
 
-@pytest.mark.parametrize("M,N,K", [(257, 96, 72), (129, 6176, 520),                              # one CTA a tile: 64, 128 columns
-                                   (226, 3072, 3072), (200, 1056, 1544), (257, 160, 4104),       # 2, 4, 8 CTAs a tile
-                                   (1600, 1024, 2048), (513, 4128, 520), (257, 7328, 1032)])     # pairs: 128, 192, 256 columns
+@pytest.mark.parametrize("M,N,K,kernel", [
+    (257, 96, 72, "one64"), (129, 6176, 520, "one128"), (226, 3072, 3072, "split2"), (200, 1056, 1544, "split4"),
+    (257, 160, 4104, "split8"), (1600, 1024, 2048, "pair128"), (513, 4128, 520, "pair192"), (257, 7328, 1032, "pair256")])
 @pytest.mark.parametrize("dtype", [wdc.BF16, wdc.F32])
 @pytest.mark.parametrize("in_place", [False, True])
-def test_gemm_gelu_then_gated_residual(M, N, K, dtype, in_place):
+def test_gemm_gelu_then_gated_residual(M, N, K, kernel, dtype, in_place):
     """C = res + gate * GELU(A W^T + bias), both options of one call, in every
     kernel of both dtypes.  bf16 as above; fp32: sums of K terms and the
     hardware exponential of GELU (2^-22 relative of a factor below one) against
@@ -147,7 +160,40 @@ def test_gemm_gelu_then_gated_residual(M, N, K, dtype, in_place):
         buf[:M] = R
     ctx.op_gemm(A, W, buf[:M], bias=b, gelu=True, res=buf[:M] if in_place else R, gate=gate)
     torch.cuda.synchronize()
+    if dtype == wdc.BF16:
+        assert_gemms(ctx, f"{kernel}/resid_gelu")
     assert ctx.device_errors() == 0
     err = float((buf[:M].double() - want).norm() / want.norm())
     assert err <= (2.0 ** -8 if dtype == wdc.BF16 else 2.0 ** -20) + K * 2.0 ** -22
     assert bool((buf[M:] == 7.0).all())
+
+
+@pytest.mark.parametrize("in_ch,p,frames,hp,wp,D,B,kernel", [
+    (16, 2, 3, 7, 11, 256, 3, "one64"), (128, 2, 5, 14, 15, 512, 3, "one128"), (64, 4, 5, 14, 15, 1024, 3, "pair128"),
+    (128, 2, 7, 10, 23, 768, 2, "pair192"), (48, 4, 7, 12, 20, 1536, 3, "pair256")])
+def test_repeating_residual(in_ch, p, frames, hp, wp, D, B, kernel):
+    """The position embedding of a batch (its rows repeat with each sample, and
+    slabs of 32 rows hold two samples) in every kernel that takes it (with at
+    most 1024 features a patch its K is never split): bitwise the samples' own
+    forwards, whose residual does not repeat, and one of them against the oracle."""
+    cfgd = dict(MODEL, hidden=D, heads=D // 64, mlp=D, in_ch=in_ch, frames=frames, height=hp * p, width=wp * p, patch=p,
+                cond_tokens=5)
+    shape = (in_ch, frames, hp * p, wp * p)
+    W = synth.dit_weights(cfgd, 11, std=0.02, bias_std=0.05, bf16=True)
+    ctx = wdc.Context(wdc.make_config(dtype=wdc.BF16, max_batch=B, **cfgd), 2)
+    ctx.set_weights(W)
+    z = [synth.latent(20 + b, shape) for b in range(B)]
+    ct = [synth.cond_tokens(30 + b, 5, 64) for b in range(B)]
+    zd, cd = [_dev(a.reshape(-1)) for a in z], [_dev(a) for a in ct]
+    many = [torch.empty_like(t) for t in zd]
+    ctx.dit_forward_batch(zd, 600.0, cd, many)
+    torch.cuda.synchronize()
+    assert_gemms(ctx, f"{kernel}/resid_repeat")
+    for b in range(B):
+        one = torch.empty_like(zd[b])
+        ctx.dit_forward(zd[b], 600.0, cd[b], one)
+        torch.cuda.synchronize()
+        assert torch.equal(one, many[b])
+    assert ctx.device_errors() == 0
+    want = dit.forward(W, DiTConfig(**cfgd), z[0], 600.0, ct[0])
+    assert rel_l2(many[0].cpu().numpy(), want) <= 2e-2

@@ -1,10 +1,10 @@
-"""The CTA-pair GEMM with 192- and 128-column tiles, at shapes for which the
-launch rule takes them on 152 SMs, with remainders of rows, columns and K."""
+"""The CTA-pair GEMM with 256-, 192- and 128-column tiles, at shapes for which
+the launch rule takes them on 152 SMs, with remainders of rows, columns and K."""
 import numpy as np
 import pytest
 import torch
 
-from helpers import rel_l2
+from helpers import assert_gemms, rel_l2
 from oracle import dit
 from oracle.params import DiTConfig
 from paper_2608_01845_gb300 import synth, wdc
@@ -19,10 +19,11 @@ def _dev(a, dtype=torch.float32):
     return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda().to(dtype)
 
 
-@pytest.mark.parametrize("M,N,K", [(1999, 1504, 1544), (2000, 1536, 1536),     # 192 columns
-                                   (1570, 1056, 4104), (1600, 1024, 4096)])    # 128 columns
+@pytest.mark.parametrize("M,N,K,width", [
+    (257, 7328, 1032, 256), (2817, 3040, 1032, 256), (1999, 1504, 1544, 192), (2000, 1536, 1536, 192),
+    (513, 4128, 520, 192), (1570, 1056, 4104, 128), (1600, 1024, 4096, 128)])     # (257 and 513: a last tile of one row)
 @pytest.mark.parametrize("mode", ["store", "gelu", "resid"])
-def test_gemm(M, N, K, mode):
+def test_gemm(M, N, K, width, mode):
     """Against fp64 on sampled rows: one rounding of the result to bf16 (at most
     2^-8 relative an element) and fp32 sums of K terms; nothing is written past
     the last row."""
@@ -41,6 +42,7 @@ def test_gemm(M, N, K, mode):
         kw.update(res=_dev(R, torch.bfloat16), gate=_dev(g))
     ctx.op_gemm(_dev(A, torch.bfloat16), _dev(W, torch.bfloat16), C, bias=_dev(b), **kw)
     torch.cuda.synchronize()
+    assert_gemms(ctx, f"pair{width}/{mode}")
     assert ctx.device_errors() == 0
     assert rel_l2(C.float().cpu().numpy()[rows], want) <= 2.0 ** -8 + K * 2.0 ** -22
     assert bool((buf[M:] == 7.0).all())
@@ -61,6 +63,7 @@ def test_qkv_of_a_block(dual):
     xt = _dev(x, torch.bfloat16)
     ctx.dit_block_forward(0, xt, _dev(mod))
     torch.cuda.synchronize()
+    assert_gemms(ctx, "pair192/qkv grouped" if dual else "pair192/qkv")
     assert ctx.device_errors() == 0
     rows = np.unique(np.r_[0, 5, 12, 13, np.linspace(14, L - 1, 60).astype(int)])
     mods = [mod[6 * s:6 * s + 6].astype(np.float64) for s in range(1 + dual)]
