@@ -44,15 +44,16 @@
 // numerator pairs in 700 cycles, both at once take 1130, and then neither has
 // any while both wait for S, store P and hand over; so tile 1's first product
 // waits for tile 0's first P (`stagger`) and the two warps stay about half a
-// step apart (3.08 -> 2.88 ms at 48 heads x 17776).  Producer and issuers run
-// with all lanes and issue from an elected one (3.17 -> 3.08 ms; 1.49 -> 1.36
-// at 24 x 13568 x 128).  Tiles half a step apart hold a stage of K and V
-// longer: five stages instead of three, 227 -> 203 us at 48 x 4276 x 64.
+// step apart (3.08 -> 2.88 ms at 48 heads x 17776).  The producer and, at d =
+// 64, the issuers run with all lanes and issue from an elected one (3.17 -> 3.08
+// ms).  Tiles half a step apart hold a stage of K and V longer: five stages instead
+// of three, 227 -> 203 us at 48 x 4276 x 64.
 // Grid: one CTA per (head, 256-query) unit, one CTA per SM.  The units of a
 // sample's last, partial round are split over the key range where that saves
-// enough steps (attn_split): each part runs the same pipeline over its steps and writes its unnormalised O,
-// exponent base and row sum to a workspace of the context, and
-// attn_combine_kernel merges the parts, so the round's CTAs fill the SMs.
+// enough steps (attn_split): each part runs the same pipeline over its steps and
+// writes its unnormalised O, exponent base and row sum to a workspace of the
+// context, and attn_combine_kernel merges the parts, so the round's CTAs fill
+// the SMs.
 // Keys past L are masked (TMA zero-fills out-of-range K / V^T).  Every
 // mbarrier wait is bounded.
 #include "dit_kernels.cuh"

@@ -65,22 +65,24 @@ namespace {
 // ---------------------------------------------------------------- small kernels
 // y[r] = act(W[r,:] . x + b[r]); one warp per row.  act: 0 none, 1 SiLU.
 // Bound by the latency of its loads (E x E) or by reading W (the modulation).
-// With whole 16-byte vectors in a row (vec) each lane loads up to four of W's
+// With whole 16-byte vectors in a bf16 row (vec) each lane loads up to four of W's
 // before the wait for x: weights change only in wdc_init_weights and
 // wdc_set_tensor, which return once they are on the device, so W's reads run
 // under the kernels before.  Alone, 26624 x 512 bf16 (27 MB, cold) takes 10 us
-// as with 2-byte loads; the gain is in the chain (with prep_kernel's, see there).  fp32 keeps
-// the element order of its sums: by vectors, the rollout with the
-// ill-conditioned linear observation came out 1.4e-5 off fp64 instead of 6e-6.
+// as with 2-byte loads; the gain is in the chain (with prep_kernel's, see
+// there).  fp32 keeps the element order of its sums: by vectors, the rollout
+// with the ill-conditioned linear observation came out 1.4e-5 off fp64 instead
+// of 6e-6.
 template <typename T>
 __global__ void __launch_bounds__(256) gemv_kernel(const T* __restrict__ W, const float* x, const float* __restrict__ b,
                                                    float* y, int rows, int cols, int act, int vec) {
-    constexpr int VEC = 16 / (int)sizeof(T), PRE = 4;
+    constexpr bool kVec = sizeof(T) == 2;
+    constexpr int VEC = 8, PRE = 4;
     chain_release();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const T* w = W + (size_t)min(warp, rows - 1) * cols;
     const uint4* w4 = reinterpret_cast<const uint4*>(w);
-    const int nv = vec ? cols / VEC : 0;
+    const int nv = kVec && vec ? cols / VEC : 0;
     uint4 u[PRE];
 #pragma unroll
     for (int i = 0; i < PRE; ++i)
@@ -100,7 +102,7 @@ __global__ void __launch_bounds__(256) gemv_kernel(const T* __restrict__ W, cons
             s = fmaf(ld_act<T>(t + 4 * k + 3), f.w, s);
         }
     };
-    if (vec) {
+    if (kVec && vec) {
 #pragma unroll
         for (int i = 0; i < PRE; ++i)
             if (lane + 32 * i < nv) add(u[i], lane + 32 * i);
@@ -881,8 +883,6 @@ static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int nb, int 
     return WDC_OK;
 }
 
-// H heads in all = nb samples x Hs heads; sample b's output rows follow the
-// batch's stream-major token layout (Lc condition tokens per sample).
 // Two GEMMs with the same N and K (the dual-stream block's video rows and
 // condition rows, each with its own weights and epilogue): one grouped
 // tcgen05 launch in bf16, two SIMT launches in the fp32 parity mode.
@@ -899,8 +899,10 @@ static wdc_status gemm2(Ctx* c, const void* A0, const void* W0, int M0, const Ep
     return tc_gemm_grouped(c, A0, W0, M0, M0 / nb, e0, A1, W1, M1, M1 / nb, e1, N, K, s);
 }
 
-// V^T rows have stride ldv (>= L).  bf16 runs on the tcgen05 kernel only;
-// the SIMT kernel serves the fp32 parity mode.
+// H heads in all = nb samples x Hs heads; sample b's output rows follow the
+// batch's stream-major token layout (Lc condition tokens per sample).  V^T rows
+// have stride ldv (>= L).  bf16 runs on the tcgen05 kernel only; the SIMT kernel
+// serves the fp32 parity mode.
 static wdc_status attention(Ctx* c, const void* q, const void* k, const void* vt, int ldv, void* o, int H, int L,
                             int d, int Hs, int Lc, cudaStream_t s) {
     if (c->cfg.dtype == WDC_BF16) {

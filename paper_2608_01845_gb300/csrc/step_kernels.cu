@@ -26,8 +26,8 @@
 // 128-element run = one bucket with 128-bit loads.
 //
 // Reductions are deterministic: per-warp bucket rows in shared memory, fixed-
-// order block combination in fp64, per-block partials, and a last-block-done
-// final reduction in fixed order.  No kernel here waits on another CTA.
+// order block combination, per-block partials, and a last-block-done final
+// reduction in fixed order, in fp32.  No kernel here waits on another CTA.
 #include "wdc_internal.h"
 
 #include <cmath>
@@ -61,7 +61,7 @@ __device__ __forceinline__ float signed_term(uint32_t idx, uint32_t seed, float 
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
-// Runs per warp whose bank reads are prefetched while warp 0 forms the head.
+// Runs per warp whose bank reads are prefetched while the first warps form the head.
 constexpr int kPrefetchRuns = 4;
 
 // Butterfly sum over the 32 lanes (a fixed-order tree: every lane ends with
@@ -955,7 +955,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
             s_out.pi[i] = i < K ? hs.pi[i] : 0.f;
         }
         if (t == 0) {
-            // controller tail in fp32; the stored risk R stays fp64
+            // controller tail and stored risk R in fp32
             const ParamsDev& p = a.prm;
             const float eps = p.eps;
             const StateIn& S = ps.S;
@@ -1028,7 +1028,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a_in) {
         return;
     }
 
-    // ---- anchor pass tail (MODE == kModeAnchor): fp32 arithmetic, fp64 state
+    // ---- anchor pass tail (MODE == kModeAnchor), in fp32
     __shared__ float s_rms[2];
     if (t == 0) {
         const ParamsDev& p = a.prm;

@@ -203,8 +203,8 @@ struct LaunchScope {
 // starts once every block of that kernel has called chain_release() (or
 // exited), sets itself up, and calls chain_wait() before it touches global
 // memory (the weights aside, see gemv_kernel), which returns when that kernel is
-// complete and its writes are visible.  Every kernel of the chain waits, so a kernel's wait also covers all
-// earlier ones.  chain_release() comes after a kernel has its tensor memory: a
+// complete and its writes are visible.  Every kernel of the chain waits, so a
+// kernel's wait also covers all earlier ones.  chain_release() comes after a kernel has its tensor memory: a
 // dependent block on the same SM must not take it first.  Launched plainly,
 // both are no-ops.  The fp32 kernels, of which several blocks share an SM, wait
 // but do not release early: the next kernel's blocks, placed beside them, end
