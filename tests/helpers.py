@@ -14,6 +14,13 @@ def rel_l2(a, b):
     return float(np.linalg.norm(a - b) / (den if den > 0 else 1.0))
 
 
+def to_dev(a, dtype=None):
+    """A numpy array as a float32 (or `dtype`) CUDA tensor."""
+    import torch
+    t = torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
+    return t if dtype is None else t.to(dtype)
+
+
 def assert_gemms(ctx, *expected):
     """Each of `expected`, "kernel/form" or "kernel/form grouped", is among the
     bf16 GEMMs the context has launched: a test for a kernel's edges has reached

@@ -23,7 +23,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import assert_gemms, params_for_both, rel_l2
+from helpers import assert_gemms, params_for_both, rel_l2, to_dev
 from oracle import batch as ob
 from oracle import dit
 from oracle import schedule as sch
@@ -41,10 +41,6 @@ N = 16 * 4 * 16 * 16
 T = 10
 
 
-def _dev(a):
-    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
-
-
 def _ctx(cfgd, dtype, max_batch, W, params=None):
     ctx = wdc.Context(wdc.make_config(dtype=dtype, max_batch=max_batch, **cfgd), T, params=params)
     ctx.set_weights(W)
@@ -60,8 +56,8 @@ def test_batched_forward_equals_single_forwards(dtype, model):
     W = synth.dit_weights(cfgd, 7, std=0.02, bias_std=0.02)
     ctx = _ctx(cfgd, dtype, 4, W)
     B = 3
-    zs = [_dev(synth.latent(30 + b, shape)) for b in range(B)]
-    cts = [_dev(synth.cond_tokens(40 + b, cfgd["cond_tokens"], 256)) for b in range(B)]
+    zs = [to_dev(synth.latent(30 + b, shape)) for b in range(B)]
+    cts = [to_dev(synth.cond_tokens(40 + b, cfgd["cond_tokens"], 256)) for b in range(B)]
     vs = [torch.empty(N, device="cuda") for _ in range(B)]
     ctx.dit_forward_batch(zs, 731.0, cts, vs)
     if dtype == wdc.BF16 and model == "to_pairs":
@@ -84,7 +80,7 @@ def test_guided_forward_matches_oracle():
     zs = [synth.latent(50 + b, SHAPE) for b in range(2)]
     cts = [synth.cond_tokens(60 + b, 16, 256) for b in range(2)]
     vs = [torch.empty(N, device="cuda") for _ in range(2)]
-    ctx.dit_forward_batch([_dev(z) for z in zs], 640.0, [_dev(c) for c in cts], vs, cfg=True, guidance=g)
+    ctx.dit_forward_batch([to_dev(z) for z in zs], 640.0, [to_dev(c) for c in cts], vs, cfg=True, guidance=g)
     torch.cuda.synchronize()
     for b in range(2):
         want = ob.guided_velocity(dit.forward(W, cfg, zs[b], 640.0, cts[b]),
@@ -140,10 +136,10 @@ def test_rollout_batch_matches_oracle(parity, guided):
     ctxs = [_ctx(PARITY_MODEL, wdc.F32, 6, W, params=cps[0])]
     ctxs += [wdc.Context(wdc.make_config(in_ch=16, frames=4, height=16, width=16), T, params=cps[b])
              for b in (1, 2)]
-    ct_d = [_dev(c) for c in cts]
+    ct_d = [to_dev(c) for c in cts]
     conds = [wdc.make_cond(ct_d[b], descs[b]["cam"], descs[b]["depth"]) for b in range(3)]
     outs = [torch.empty(N, device="cuda") for _ in range(3)]
-    decs, traces = wdc.rollout_batch(ctxs, [_dev(z) for z in zs], conds, outs, cfg=guided, guidance=g or 1.0)
+    decs, traces = wdc.rollout_batch(ctxs, [to_dev(z) for z in zs], conds, outs, cfg=guided, guidance=g or 1.0)
     for b in range(3):
         zf, dec, tr = want[b]
         assert decs[b] == dec, b
@@ -163,8 +159,8 @@ def test_rollout_batch_equals_single_rollouts_bf16():
     cfgd = dict(PARITY_MODEL, layers=1)
     W = synth.dit_weights(cfgd, 11, std=0.02, bf16=True)
     B = 3
-    zs = [_dev(synth.latent(70 + b, SHAPE)) for b in range(B)]
-    cts = [_dev(synth.cond_tokens(80 + b, 16, 256, bf16=True)) for b in range(B)]
+    zs = [to_dev(synth.latent(70 + b, SHAPE)) for b in range(B)]
+    cts = [to_dev(synth.cond_tokens(80 + b, 16, 256, bf16=True)) for b in range(B)]
     descs = [synth.cond_descriptors(90 + b) for b in range(B)]
     taus = [0.3, 0.6, 1.0]
     conds = [wdc.make_cond(cts[b], descs[b]["cam"], descs[b]["depth"]) for b in range(B)]
@@ -186,8 +182,8 @@ def test_rollout_batch_equals_single_rollouts_bf16():
 def test_batch_argument_errors(parity):
     W, cfg, zs, cts, descs = parity
     ctx = _ctx(PARITY_MODEL, wdc.F32, 2, W)
-    z = [_dev(zs[0]) for _ in range(3)]
-    c = [_dev(cts[0]) for _ in range(3)]
+    z = [to_dev(zs[0]) for _ in range(3)]
+    c = [to_dev(cts[0]) for _ in range(3)]
     v = [torch.empty(N, device="cuda") for _ in range(3)]
     with pytest.raises(wdc.WdcError) as e:
         ctx.dit_forward_batch(z, 500.0, c, v)                     # 3 > max_batch
@@ -213,8 +209,8 @@ def test_batched_forward_at_max_batch_bf16():
     W = synth.dit_weights(PARITY_MODEL, 9, std=0.02, bias_std=0.02, bf16=True)
     ctx = _ctx(PARITY_MODEL, wdc.BF16, wdc.MAX_BATCH, W)
     B = wdc.MAX_BATCH
-    zs = [_dev(synth.latent(100 + b, SHAPE)) for b in range(B)]
-    cts = [_dev(synth.cond_tokens(200 + b, 16, 256, bf16=True)) for b in range(B)]
+    zs = [to_dev(synth.latent(100 + b, SHAPE)) for b in range(B)]
+    cts = [to_dev(synth.cond_tokens(200 + b, 16, 256, bf16=True)) for b in range(B)]
     vs = [torch.empty(N, device="cuda") for _ in range(B)]
     ctx.dit_forward_batch(zs, 420.0, cts, vs)
     for b in (0, 7, B - 1):
@@ -240,14 +236,14 @@ def test_rollout_batch_per_step_conditions_and_host_latents(parity):
     W, cfg, zs, cts, _ = parity
     B = 2
     descs = [synth.cond_descriptors(300 + b, T, static=False) for b in range(B)]
-    ct_d = [_dev(c) for c in cts[:B]]
+    ct_d = [to_dev(c) for c in cts[:B]]
     conds = [[wdc.make_cond(ct_d[b], d["cam"], d["depth"]) for d in descs[b]] for b in range(B)]
     taus = [0.5, 0.3]
     ctxs = [_ctx(PARITY_MODEL, wdc.F32, B, W, params=wdc.make_params(tau_risk=taus[0]))]
     ctxs.append(wdc.Context(wdc.make_config(in_ch=16, frames=4, height=16, width=16), T,
                             params=wdc.make_params(tau_risk=taus[1])))
     outs = [torch.empty(N, device="cuda") for _ in range(B)]
-    decs, tr = wdc.rollout_batch(ctxs, [_dev(z) for z in zs[:B]], conds, outs)
+    decs, tr = wdc.rollout_batch(ctxs, [to_dev(z) for z in zs[:B]], conds, outs)
     # host (pinned) latents in and out give the same result
     zh = [torch.from_numpy(np.ascontiguousarray(z, dtype=np.float32).ravel()).pin_memory() for z in zs[:B]]
     oh = [torch.empty(N).pin_memory() for _ in range(B)]
@@ -260,7 +256,7 @@ def test_rollout_batch_per_step_conditions_and_host_latents(parity):
     for b in range(B):
         single.set_cache_params(wdc.make_params(tau_risk=taus[b]))
         out = torch.empty(N, device="cuda")
-        dec, trs = single.rollout(_dev(zs[b]), conds[b], out)
+        dec, trs = single.rollout(to_dev(zs[b]), conds[b], out)
         assert dec == decs[b]
         assert torch.equal(out, outs[b])
         assert [t["d_hat"] for t in trs] == [t["d_hat"] for t in tr[b]]

@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 import torch
 
+from helpers import to_dev
 from paper_2608_01845_gb300 import synth, wdc
 
 pytestmark = pytest.mark.gpu
@@ -29,9 +30,8 @@ def test_chained_forwards_equal_plain_launches(dtype, model):
     ctx.set_weights(synth.dit_weights(cfgd, 5, std=0.02, bias_std=0.02))
     shape = (cfgd["in_ch"], cfgd["frames"], cfgd["height"], cfgd["width"])
     n = int(np.prod(shape))
-    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda()
-    zs = [dev(synth.latent(70 + r, shape)) for r in range(REPEATS)]
-    cts = [dev(synth.cond_tokens(80 + r, cfgd["cond_tokens"], 256)) for r in range(REPEATS)]
+    zs = [to_dev(synth.latent(70 + r, shape)) for r in range(REPEATS)]
+    cts = [to_dev(synth.cond_tokens(80 + r, cfgd["cond_tokens"], 256)) for r in range(REPEATS)]
 
     def forwards():
         out = torch.full((REPEATS, n), float("nan"), device="cuda")

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import assert_gemms, rel_l2
+from helpers import assert_gemms, rel_l2, to_dev
 from oracle import dit
 from oracle.params import DiTConfig
 from paper_2608_01845_gb300 import synth, wdc
@@ -14,10 +14,6 @@ pytestmark = pytest.mark.gpu
 
 MODEL = dict(layers=1, hidden=256, heads=4, head_dim=64, mlp=512, temb_dim=256, freq_dim=256, in_ch=16, frames=3,
              height=14, width=22, patch=2, cond_tokens=16, cond_dim=64, dual_stream=0)
-
-
-def _dev(a, dtype=torch.float32):
-    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda().to(dtype)
 
 
 @pytest.mark.parametrize("M", [1, 31, 33, 127, 128, 255, 256, 257, 289])
@@ -39,8 +35,8 @@ def test_gemm_rows_and_columns(M, N, mode):
     elif mode == "resid":
         R, g = synth.bf16_round(synth.normal(4, (M, N))), synth.normal(5, (N,))
         want = R.astype(np.float64) + g * want
-        kw.update(res=_dev(R, torch.bfloat16), gate=_dev(g))
-    ctx.op_gemm(_dev(A, torch.bfloat16), _dev(W, torch.bfloat16), C, bias=_dev(b), **kw)
+        kw.update(res=to_dev(R, torch.bfloat16), gate=to_dev(g))
+    ctx.op_gemm(to_dev(A, torch.bfloat16), to_dev(W, torch.bfloat16), C, bias=to_dev(b), **kw)
     torch.cuda.synchronize()
     assert_gemms(ctx, f"one64/{mode}")
     assert ctx.device_errors() == 0
@@ -59,7 +55,7 @@ def test_forward_slabs_across_samples_and_streams(Lc, dual, d):
     ctx.set_weights(W)
     z = [synth.latent(20 + b, (16, 3, 14, 22)) for b in range(3)]
     ct = [synth.cond_tokens(30 + b, Lc, 64) for b in range(3)]
-    zd, cd = [_dev(a.reshape(-1)) for a in z], [_dev(a) for a in ct]
+    zd, cd = [to_dev(a.reshape(-1)) for a in z], [to_dev(a) for a in ct]
     one = []
     for b in range(3):
         one.append(torch.empty_like(zd[b]))
@@ -107,7 +103,8 @@ def test_gemm_few_tiles(M, N, K, kernel, mode):
 @pytest.mark.parametrize("Lc,dual,d,D,mlp,gemms", [
     (5, 0, 64, 2048, 4096, ["split4/store", "split2/qkv", "split4/gelu", "split4/resid"]),
     (5, 1, 128, 2048, 4096, ["split2/gelu grouped", "split4/resid grouped", "split8/unpatch"]),
-    (100, 1, 128, 1536, 1024, ["split8/store", "split2/qkv grouped", "split4/gelu grouped", "split4/resid grouped", "split4/unpatch"]),
+    (100, 1, 128, 1536, 1024, ["split8/store", "split2/qkv grouped", "split4/gelu grouped", "split4/resid grouped",
+                               "split4/unpatch"]),
     (140, 1, 64, 2048, 1024, ["split4/gelu grouped", "split2/resid grouped"])])
 def test_forward_split_k(Lc, dual, d, D, mlp, gemms):
     """A wide model on few tokens, whose block's GEMMs split K (those named;
@@ -122,7 +119,7 @@ def test_forward_split_k(Lc, dual, d, D, mlp, gemms):
     ctx.set_weights(W)
     z = [synth.latent(20 + b, (16, 1, 8, 10)) for b in range(3)]
     ct = [synth.cond_tokens(30 + b, Lc, 2048) for b in range(3)]
-    zd, cd = [_dev(a.reshape(-1)) for a in z], [_dev(a) for a in ct]
+    zd, cd = [to_dev(a.reshape(-1)) for a in z], [to_dev(a) for a in ct]
     one = []
     for b in range(3):
         one.append(torch.empty_like(zd[b]))
@@ -184,7 +181,7 @@ def test_repeating_residual(in_ch, p, frames, hp, wp, D, B, kernel):
     ctx.set_weights(W)
     z = [synth.latent(20 + b, shape) for b in range(B)]
     ct = [synth.cond_tokens(30 + b, 5, 64) for b in range(B)]
-    zd, cd = [_dev(a.reshape(-1)) for a in z], [_dev(a) for a in ct]
+    zd, cd = [to_dev(a.reshape(-1)) for a in z], [to_dev(a) for a in ct]
     many = [torch.empty_like(t) for t in zd]
     ctx.dit_forward_batch(zd, 600.0, cd, many)
     torch.cuda.synchronize()

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import assert_gemms, rel_l2
+from helpers import assert_gemms, rel_l2, to_dev
 from oracle import dit
 from oracle.params import DiTConfig
 from paper_2608_01845_gb300 import synth, wdc
@@ -13,10 +13,6 @@ pytestmark = pytest.mark.gpu
 
 MODEL = dict(layers=1, hidden=512, heads=8, head_dim=64, mlp=2048, temb_dim=256, freq_dim=256, in_ch=16, frames=4,
              height=40, width=40, patch=2, cond_tokens=13, cond_dim=64, dual_stream=0)
-
-
-def _dev(a, dtype=torch.float32):
-    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32)).cuda().to(dtype)
 
 
 @pytest.mark.parametrize("M,N,K,width", [
@@ -39,8 +35,8 @@ def test_gemm(M, N, K, width, mode):
     elif mode == "resid":
         R, g = synth.bf16_round(synth.normal(4, (M, N))), synth.normal(5, (N,))
         want = R[rows].astype(np.float64) + g * want
-        kw.update(res=_dev(R, torch.bfloat16), gate=_dev(g))
-    ctx.op_gemm(_dev(A, torch.bfloat16), _dev(W, torch.bfloat16), C, bias=_dev(b), **kw)
+        kw.update(res=to_dev(R, torch.bfloat16), gate=to_dev(g))
+    ctx.op_gemm(to_dev(A, torch.bfloat16), to_dev(W, torch.bfloat16), C, bias=to_dev(b), **kw)
     torch.cuda.synchronize()
     assert_gemms(ctx, f"pair{width}/{mode}")
     assert ctx.device_errors() == 0
@@ -60,8 +56,8 @@ def test_qkv_of_a_block(dual):
     ctx.set_weights(W)
     x = synth.bf16_round(synth.normal(41, (L, D)))
     mod = synth.normal(42, (6 * (1 + dual), D), 0.3)
-    xt = _dev(x, torch.bfloat16)
-    ctx.dit_block_forward(0, xt, _dev(mod))
+    xt = to_dev(x, torch.bfloat16)
+    ctx.dit_block_forward(0, xt, to_dev(mod))
     torch.cuda.synchronize()
     assert_gemms(ctx, "pair192/qkv grouped" if dual else "pair192/qkv")
     assert ctx.device_errors() == 0

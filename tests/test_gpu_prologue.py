@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import rel_l2
+from helpers import rel_l2, to_dev
 from oracle import batch as ob
 from oracle import dit
 from oracle.params import DiTConfig
@@ -38,9 +38,8 @@ def test_guided_forward(dtype, in_ch, patch, frames, height, width, Lc, Dc, Fd, 
         z, ct = synth.bf16_round(z), synth.bf16_round(ct)
     ctx = wdc.Context(wdc.make_config(dtype=dtype, max_batch=2, **cfgd), 2)
     ctx.set_weights(W)
-    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a).reshape(-1)).cuda()
     v = torch.empty(z.size, device="cuda")
-    ctx.dit_forward_batch([dev(z)], 412.5, [dev(ct)], [v], cfg=True, guidance=1.5)
+    ctx.dit_forward_batch([to_dev(z.reshape(-1))], 412.5, [to_dev(ct)], [v], cfg=True, guidance=1.5)
     torch.cuda.synchronize()
     assert ctx.device_errors() == 0
     cfg = DiTConfig(**cfgd)

@@ -22,7 +22,7 @@ def test_the_upload_waits_for_its_copy():
     code = re.sub(r"//[^\n]*", "", open(os.path.join(ROOT, "paper_2608_01845_gb300", "csrc", "dit.cu")).read())
     body = re.search(r"static wdc_status upload\([^{]*\{(.*?)\n\}", code, re.S).group(1)
     assert "cudaMemcpy(" in body
-    assert re.search(r"cudaMemcpy\(.*(cudaStreamSynchronize|cudaDeviceSynchronize)\([^\n]*\n\s*return WDC_OK;\s*$", body, re.S)
+    assert re.search(r"cudaMemcpy\(.*cuda(Stream|Device)Synchronize\([^\n]*\n\s*return WDC_OK;\s*$", body, re.S)
     assert body.count("return WDC_OK") == 1
 
 
