@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(SimtTile<BM, TM, TN>::THREADS)
         }
 }
 
-// Any K and alignment: 64 x 64 tiles loaded element by element.
+// Any K and alignment, and short K: 64 x 64 tiles loaded element by element.
 template <typename T>
 __global__ void __launch_bounds__(256) gemm_simt_kernel(const T* A, const T* __restrict__ W, int M,
                                                          int N, int K, const Epi e) {
@@ -856,9 +856,22 @@ static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int nb, int 
     LaunchScope ls(c, WDC_K_GEMM, s);
     const float* a = reinterpret_cast<const float*>(A);
     const float* w = reinterpret_cast<const float*>(W);
-    const long long large = (long long)blocks_for(M, 64) * blocks_for(N, 64);
-    const long long small = (long long)blocks_for(M, 16) * blocks_for(N, 32);
-    if (K % 4 || (((uintptr_t)A | (uintptr_t)W) & 15) || blocks_for(M, 16) > 65535) {
+    // the shape with the fewer cycles an element of k: 66 for each 64 x 64 tile
+    // of the busiest SM; 28 for a 16 x 32 one alone, 13.4 each for several (600
+    // x 1536 x 512: 38 us by the large shape, 48 by the small one; 272 x 256 x
+    // 1024: 37 and 17)
+    const long long sms = c->num_sms;
+    const long long per_large = ((long long)blocks_for(M, 64) * blocks_for(N, 64) + sms - 1) / sms;
+    const long long per_small = ((long long)blocks_for(M, 16) * blocks_for(N, 32) + sms - 1) / sms;
+    const bool large = 660 * per_large <= (per_small > 2 ? 134 * per_small : 280);
+    // The element-wise kernel works in blocks of 16 k, not 32, and fits more
+    // blocks on an SM: it is the faster one for one such block (8000 x 2048 x 16:
+    // 38 us, 52 by the large shape) and, with four tiles an SM or more, for two
+    // of them and for an odd number up to 11, of which the large shape pads the
+    // last (8000 x 2048 x 48: 62 and 77; x 176: 181 and 190; x 208: 210 and 219,
+    // but 1% either way at other sizes).
+    const bool short_k = K <= 16 || (per_large >= 4 && (K <= 32 || (K <= 176 && blocks_for(K, 16) % 2)));
+    if (K % 4 || (((uintptr_t)A | (uintptr_t)W) & 15) || blocks_for(M, 16) > 65535 || (large && short_k)) {
         dim3 grid(blocks_for(N, 64), blocks_for(M, 64));
         launch_kernel(gemm_simt_kernel<float>, grid, 256, 0, s, 1, a, w, M, N, K, e);
         return WDC_OK;
@@ -868,13 +881,7 @@ static wdc_status gemm(Ctx* c, const void* A, const void* W, int M, int nb, int 
         return ok = allow_smem(gemm_simt_tile_kernel<64, 8, 2>, SimtLarge::SMEM) &&
                     allow_smem(gemm_simt_tile_kernel<16, 4, 1>, SimtSmall::SMEM);
     });
-    // the shape with the fewer cycles an element of k: 66 for each 64 x 64 tile
-    // of the busiest SM; 28 for a 16 x 32 one alone, 13.4 each for several (600
-    // x 1536 x 512: 38 us by the large shape, 48 by the small one; 272 x 256 x
-    // 1024: 37 and 17)
-    const long long sms = c->num_sms;
-    const long long per_large = (large + sms - 1) / sms, per_small = (small + sms - 1) / sms;
-    if (660 * per_large <= (per_small > 2 ? 134 * per_small : 280))
+    if (large)
         launch_kernel(gemm_simt_tile_kernel<64, 8, 2>, dim3(blocks_for(N, 64), blocks_for(M, 64)), SimtLarge::THREADS,
                       SimtLarge::SMEM, s, 1, a, w, M, N, K, e);
     else

@@ -46,6 +46,24 @@ def test_gemm(M, N, K, offset, mode):
     assert bool((buf[M:] == 7.0).all())
 
 
+@pytest.mark.parametrize("M,N,K", [(600, 768, 4), (600, 768, 16), (600, 768, 20), (2000, 1024, 32), (2000, 1024, 36),
+                                   (2000, 1024, 48), (2000, 1024, 52), (2000, 1024, 176), (2000, 1024, 180)])
+def test_gemm_of_short_k_has_the_bits_of_any_other_shape(M, N, K):
+    """On both sides of the rule by which short K goes to the element-wise
+    kernel: the rows of a large product are bit for bit those of a product of 16
+    of them, which takes the small tiles."""
+    ctx = wdc.Context(wdc.make_config(dtype=wdc.F32, **MODEL), 2)
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A, W, b = (torch.randn(*s, device="cuda", generator=g) for s in ((M, K), (N, K), (N,)))
+    C = torch.empty(M, N, device="cuda")
+    ctx.op_gemm(A, W, C, bias=b)
+    for m in (0, 336, M - 16):
+        part = torch.empty(16, N, device="cuda")
+        ctx.op_gemm(A[m:m + 16].clone(), W, part, bias=b)
+        torch.cuda.synchronize()
+        assert torch.equal(part, C[m:m + 16])
+
+
 @pytest.mark.parametrize("H,L,d,offset", [(1, 1, 64, 0), (2, 15, 128, 0), (3, 16, 64, 0), (2, 63, 64, 0), (2, 65, 128, 0),
                                           (4, 272, 64, 0), (2, 129, 64, 1), (1, 130, 128, 3)])
 def test_attention(H, L, d, offset):
