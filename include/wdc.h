@@ -262,7 +262,8 @@ wdc_status wdc_device_errors(wdc_ctx* ctx, unsigned* bits);
  * bounded wait the tensor-core kernels use, with a limit of `limit_ns`
  * (1 us .. 1 s).  When the limit passes the wait gives up, sets bit 1 in the
  * context's error word and raises the CTA's abort flag, which releases the
- * CTA's other waiting thread; the kernel then returns normally.  Lets a test
+ * CTA's other waiting thread and a waiting warp; another warp waits out a limit
+ * of its own; the kernel then returns normally.  Lets a test
  * check the timeout path and that the context stays usable afterwards,
  * without faulting or hanging the GPU.  Asynchronous on `stream`. */
 wdc_status wdc_selftest_wait_timeout(wdc_ctx* ctx, unsigned long long limit_ns, wdc_stream stream);

@@ -88,19 +88,26 @@ __global__ void psi_kernel(const float* __restrict__ z, const float* __restrict_
 }
 
 // Bounded-wait self-test: an mbarrier that nothing completes (see
-// wdc_selftest_wait_timeout).  Thread 0 gives up after limit_ns; thread 32
-// is released by the abort flag that thread 0 raises.
+// wdc_selftest_wait_timeout).  Thread 0 gives up after limit_ns; thread 32 and
+// the whole third warp are released by the abort flag that thread 0 raises.  The
+// fourth warp waits by itself, on its own flag, until its own limit.
 __global__ void wait_probe_kernel(unsigned* err, unsigned long long limit_ns) {
     __shared__ uint64_t bar;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag, own_flag;
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
-        abort_flag = 0;
+        abort_flag = own_flag = 0;
         fence_barrier_init();
     }
     __syncthreads();
     if (threadIdx.x == 0) mbar_wait(&bar, 0, &abort_flag, err, limit_ns);
     if (threadIdx.x == 32) mbar_wait(&bar, 0, &abort_flag, err, 2 * limit_ns + 1000000ull);
+    if (threadIdx.x >= 64) {
+        int* flag = threadIdx.x < 96 ? &abort_flag : &own_flag;
+        const bool done = mbar_wait_warp(&bar, 0, flag, err, threadIdx.x < 96 ? 2 * limit_ns + 1000000ull : limit_ns);
+        // no lane is left behind: the warp's instructions can follow
+        if (elect_one() && done) atomicOr(err, kErrBounds);
+    }
     __syncthreads();
 }
 
@@ -390,7 +397,7 @@ wdc_status wdc_selftest_wait_timeout(wdc_ctx* h, unsigned long long limit_ns, wd
     if (limit_ns < 1000ull || limit_ns > 1000000000ull) return fail(c, WDC_ERR_INVALID_ARG, "limit_ns must be 1e3..1e9");
     cudaSetDevice(c->device);
     LaunchScope ls(c, WDC_K_OTHER, (cudaStream_t)stream);
-    wait_probe_kernel<<<1, 64, 0, (cudaStream_t)stream>>>(c->err, limit_ns);
+    wait_probe_kernel<<<1, 128, 0, (cudaStream_t)stream>>>(c->err, limit_ns);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(c, WDC_ERR_CUDA, std::string("wait self-test: ") + cudaGetErrorString(e));
     return WDC_OK;

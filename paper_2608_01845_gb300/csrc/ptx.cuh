@@ -85,14 +85,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // seen by some lanes and not by others: a lane that went on by itself would wait
 // without limit, in the next elect.sync, shuffle or other instruction of the
 // whole warp, for the lanes that have left.  So the lanes vote on every look.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned* err) {
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned* err,
+                                               unsigned long long limit_ns = kWaitLimitNs) {
     constexpr unsigned kAll = 0xffffffffu;
     if (__all_sync(kAll, mbar_try_wait(bar, parity))) return true;
     const unsigned long long t0 = globaltimer();
     uint32_t spins = 0;
     while (!__all_sync(kAll, mbar_try_wait(bar, parity))) {
         bool stop = *abort_flag;
-        if ((++spins & 255u) == 0u && globaltimer() - t0 > kWaitLimitNs) {
+        if ((++spins & 255u) == 0u && globaltimer() - t0 > limit_ns) {
             stop = true;
             *abort_flag = 1;
             atomicOr(err, kErrTimeout);

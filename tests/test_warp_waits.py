@@ -52,3 +52,18 @@ def test_the_warp_wait_votes():
     looks = re.findall(r"[^\n]*mbar_try_wait[^\n]*", body)
     assert looks and all("__all_sync(kAll, mbar_try_wait(" in x for x in looks)
     assert re.findall(r"[^\n]*return false[^\n]*", body) == ["        if (__any_sync(kAll, stop)) return false;"]
+
+
+@pytest.mark.gpu
+def test_a_whole_warps_wait_gives_up():
+    """The self-test's warps, one released by the abort flag and one by its own
+    limit, return with all their lanes and report the timeout only."""
+    import torch
+
+    from paper_2608_01845_gb300 import wdc
+    ctx = wdc.Context(wdc.make_config(width=4096), 4)
+    for limit_ns in (1000, 50_000, 2_000_000):
+        ctx.selftest_wait_timeout(limit_ns)
+        torch.cuda.synchronize()
+        assert ctx.device_errors() == 1
+    assert ctx.device_errors() == 0
