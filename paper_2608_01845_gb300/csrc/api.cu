@@ -241,6 +241,13 @@ wdc_status enqueue_anchor(Ctx* c, int k, const wdc_cond* cd, const float* z_t, c
     return WDC_OK;
 }
 
+// cudaMemset returns before the zeros are written, on a stream that a caller's
+// non-blocking stream does not wait for: calls that use it end with this.
+wdc_status zeros_written(Ctx* c) {
+    WDC_CUDA_TRY(c, cudaStreamSynchronize(cudaStreamLegacy));
+    return WDC_OK;
+}
+
 // Per-slot exact-step displacements for the secant and the residual reading
 // (allocated on first use, zeroed).
 wdc_status ensure_disp(Ctx* c) {
@@ -249,7 +256,7 @@ wdc_status ensure_disp(Ctx* c) {
         WDC_CUDA_TRY(c, cudaMalloc((void**)&c->disp[i], c->n * sizeof(float)));
         WDC_CUDA_TRY(c, cudaMemset(c->disp[i], 0, c->n * sizeof(float)));
     }
-    return WDC_OK;
+    return zeros_written(c);
 }
 
 wdc_status clear_disp(Ctx* c, cudaStream_t s) {
@@ -361,6 +368,7 @@ wdc_status wdc_create(const wdc_dit_config* cfg, const wdc_schedule* sched, cons
     if (cfg->layers > 0) {
         if ((st = dit_create(c))) return bail(st);
     }
+    if ((st = zeros_written(c))) return bail(st);
     *out = reinterpret_cast<wdc_ctx*>(c);
     return WDC_OK;
 }
@@ -432,7 +440,7 @@ wdc_status wdc_device_errors(wdc_ctx* h, unsigned* bits) {
     WDC_CUDA_TRY(c, cudaDeviceSynchronize());
     WDC_CUDA_TRY(c, cudaMemcpy(bits, c->err, sizeof(unsigned), cudaMemcpyDeviceToHost));
     WDC_CUDA_TRY(c, cudaMemset(c->err, 0, sizeof(unsigned)));
-    return WDC_OK;
+    return zeros_written(c);
 }
 
 wdc_status wdc_profile_enable(wdc_ctx* h, int on) {

@@ -1,4 +1,5 @@
-"""A parameter that wdc_set_tensor has returned from is on the device, whatever
+"""What a call has written is there for the next one, whatever its stream.  A
+parameter that wdc_set_tensor has returned from is on the device, whatever
 stream uses it next: the timestep products read their weights before they wait
 for the kernels ahead of them."""
 import os
@@ -24,6 +25,16 @@ def test_the_upload_waits_for_its_copy():
     assert "cudaMemcpy(" in body
     assert re.search(r"cudaMemcpy\(.*cuda(Stream|Device)Synchronize\([^\n]*\n\s*return WDC_OK;\s*$", body, re.S)
     assert body.count("return WDC_OK") == 1
+
+
+def test_calls_that_zero_memory_wait_for_it():
+    """A context's buffers and its cleared error word (read from the source)."""
+    code = re.sub(r"//[^\n]*", "", open(os.path.join(ROOT, "paper_2608_01845_gb300", "csrc", "api.cu")).read())
+    functions = re.findall(r"\nwdc_status (\w+)\([^{;]*\{(.*?)\n\}", code, re.S)
+    zeroing = {name: body for name, body in functions if re.search(r"\bcudaMemset\(", body)}
+    assert {"ensure_disp", "wdc_create", "wdc_device_errors"} <= set(zeroing)
+    for name, body in zeroing.items():
+        assert "zeros_written(c)" in body[body.rindex("cudaMemset("):], name
 
 
 @pytest.mark.gpu
